@@ -98,9 +98,16 @@ struct Tree::Dev {
   int64_t nnorm_pieces = 0;
   // matvec lists (row side; the column side's serve the adjoint product)
   int64_t *own_ptr, *par_ptr;
-  int32_t *own_blk, *par_pair, *par_son;
+  OwnItem *own, *own_c;
+  int32_t *par_pair, *par_son;
   int64_t *own_ptr_c, *par_ptr_c;
-  int32_t *own_blk_c, *par_pair_c, *par_son_c;
+  int32_t *par_pair_c, *par_son_c;
+  // nearfield of the product ([0], by row cluster) and of its adjoint ([1], by
+  // column cluster); runs of leaf pairs of one cluster per side
+  NearItem* near_items[2];
+  NearUnit *near_units[2], *leaf_units[2];
+  int32_t nnear_units[2] = {0, 0}, nleaf_units[2] = {0, 0};
+  int64_t nown[2] = {0, 0};
   // launch orders: leaf launch (both sides) then non-leaf per level
   uint32_t* codes;
   // R tiles in the same order: code << 32 | first column, 32 columns each
@@ -208,6 +215,34 @@ cudaError_t dev_malloc_async(void** p, size_t bytes, cudaStream_t st) {
   return cudaMallocAsync(p, bytes, st);
 }
 
+// The nearfield products' units (dh2_ops.cuh) of the row or the column side,
+// from each cluster's number of inadmissible blocks and their extent in the
+// other dimension; the device writes the lists (NearFill).  A
+// unit holds about `target` entries: at most kNearUnitMax, so that its sums pay
+// for their atomic additions, and few enough that a small matrix still gives
+// every SM tens of units (n = 8192 in FP64, eight vectors: 3.1 ms with half
+// as many, 2.95 so).
+constexpr int64_t kNearUnitMin = 2048, kNearUnitMax = 65536;
+void near_units_of(const Tree& tr, const std::vector<int32_t>& cnt, const std::vector<int64_t>& extent,
+                   int64_t near_elems, std::vector<int32_t>& item_begin, std::vector<int32_t>& unit_begin) {
+  const int32_t nc = tr.nclusters();
+  const int64_t target = std::min(kNearUnitMax, std::max(kNearUnitMin, near_elems / (152 * 32)));
+  item_begin.assign(nc + 1, 0);
+  unit_begin.assign(nc + 1, 0);
+  for (int32_t c = 0; c < nc; ++c) {
+    item_begin[c + 1] = item_begin[c] + cnt[c];
+    int64_t units = 0;
+    if (cnt[c] > 0) {
+      const int32_t mine = tr.size[c];
+      const int64_t e = std::min(mine, kNearRows) * extent[c];
+      const int64_t runs = std::min<int64_t>(cnt[c], (e + target - 1) / target);
+      const int64_t per = (cnt[c] + runs - 1) / runs;
+      units = ((cnt[c] + per - 1) / per) * near_slabs(mine);
+    }
+    unit_begin[c + 1] = unit_begin[c] + (int32_t)units;
+  }
+}
+
 // Capacities: leaf rank <= min(rows, #F); non-leaf rank <= min(k_cap(t1c') +
 // k_cap(t2c'), #F, 128).  Offsets of R (k_cap x #F), Q ([E1;E2] rowcap x k_cap)
 // and of the expanded non-leaf bases (#t x k_cap) follow.
@@ -227,6 +262,11 @@ dh2_status upload_tree(Tree& tr) {
   // keep host arrays alive until the copy
   std::vector<std::vector<int32_t>> i32;
   std::vector<std::vector<int64_t>> i64;
+  std::vector<NearUnit> leaf_units[2];
+  // nearfield product lists: counted per cluster here, written on the device
+  std::vector<int32_t> near_cnt[2];
+  std::vector<int64_t> near_ext[2];
+  int32_t *near_ibegin[2], *near_ubegin[2], *near_cursor[2], *own_blk[2];
   i32.reserve(64);
   i64.reserve(32);
   auto add32 = [&](std::vector<int32_t>&& v, int32_t** dst) {
@@ -342,6 +382,12 @@ dh2_status upload_tree(Tree& tr) {
   std::vector<int32_t> bt(nb), bs(nb), ba(nb), bpr(nb), bpc(nb), bo(nb), adm, inadm;
   std::vector<int64_t> noff(nb, 0), soffs(nb, 0), mxoff(nb, -1);
   int64_t S_e = 0, N_e = 0, MX_e = 0;
+  adm.reserve(tr.nadm);
+  inadm.reserve(nb - tr.nadm);
+  for (int sd = 0; sd < 2; ++sd) {
+    near_cnt[sd].assign(nc, 0);
+    near_ext[sd].assign(nc, 0);
+  }
   for (int64_t b = 0; b < nb; ++b) {
     const Block& B = tr.blocks[b];
     bt[b] = B.t;
@@ -359,7 +405,11 @@ dh2_status upload_tree(Tree& tr) {
     } else {
       inadm.push_back((int32_t)b);
       noff[b] = N_e;
-      N_e += (int64_t)tr.size[B.t] * tr.size[B.s];
+      N_e += ((int64_t)tr.size[B.t] * tr.size[B.s] + 1) & ~(int64_t)1;  // blocks start at even entries
+      ++near_cnt[0][B.t];
+      ++near_cnt[1][B.s];
+      near_ext[0][B.t] += tr.size[B.s];
+      near_ext[1][B.s] += tr.size[B.t];
     }
   }
   D->S_elems = S_e;
@@ -374,7 +424,6 @@ dh2_status upload_tree(Tree& tr) {
   add32(std::move(bpr), &D->bpair[0]);
   add32(std::move(bpc), &D->bpair[1]);
   add32(std::move(bo), &D->boff_row);
-  add64(std::move(noff), &D->near_off);
   add64(std::move(soffs), &D->Soff);
   add64(std::move(mxoff), &D->bmax_off);
   {
@@ -391,6 +440,28 @@ dh2_status upload_tree(Tree& tr) {
     add64(std::move(pcs), &D->norm_pieces);
     add64(std::move(pbeg), &D->norm_pbegin);
   }
+  std::vector<int32_t> item_begin[2], unit_begin[2];
+  for (int sd = 0; sd < 2; ++sd) {
+    near_units_of(tr, near_cnt[sd], near_ext[sd], N_e, item_begin[sd], unit_begin[sd]);
+    // runs of at most 8 consecutive leaf pairs of one cluster
+    const std::vector<int64_t>& lp = tr.side[sd].leaf_pairs;
+    for (size_t i = 0; i < lp.size();) {
+      const int32_t c = tr.side[sd].pairs[lp[i]].cluster;
+      size_t j = i + 1;
+      while (j < lp.size() && j < i + 8 && tr.side[sd].pairs[lp[j]].cluster == c) ++j;
+      leaf_units[sd].push_back({(int32_t)i, (int32_t)(j - i), 0, tr.size[c], tr.start[c], 0});
+      i = j;
+    }
+    D->nnear_units[sd] = unit_begin[sd].back();
+    D->nleaf_units[sd] = (int32_t)leaf_units[sd].size();
+    bufs.push_back({nullptr, sizeof(NearItem) * inadm.size(), (void**)&D->near_items[sd]});
+    bufs.push_back({nullptr, sizeof(NearUnit) * (size_t)D->nnear_units[sd], (void**)&D->near_units[sd]});
+    bufs.push_back({nullptr, 4 * (size_t)nc, (void**)&near_cursor[sd]});
+    add32(std::move(item_begin[sd]), &near_ibegin[sd]);
+    add32(std::move(unit_begin[sd]), &near_ubegin[sd]);
+    bufs.push_back({leaf_units[sd].data(), bytes_of(leaf_units[sd]), (void**)&D->leaf_units[sd]});
+  }
+  add64(std::move(noff), &D->near_off);
   add32(std::move(adm), &D->adm_list);
   add32(std::move(inadm), &D->inadm_list);
   // matvec lists: own blocks and father pairs per pair, row side (the
@@ -412,7 +483,9 @@ dh2_status upload_tree(Tree& tr) {
     }
     add64(std::move(optr), sd == 0 ? &D->own_ptr : &D->own_ptr_c);
     add64(std::move(pptr), sd == 0 ? &D->par_ptr : &D->par_ptr_c);
-    add32(std::move(oblk), sd == 0 ? &D->own_blk : &D->own_blk_c);
+    D->nown[sd] = (int64_t)oblk.size();
+    bufs.push_back({nullptr, sizeof(OwnItem) * oblk.size(), sd == 0 ? (void**)&D->own : (void**)&D->own_c});
+    add32(std::move(oblk), &own_blk[sd]);
     add32(std::move(ppair), sd == 0 ? &D->par_pair : &D->par_pair_c);
     add32(std::move(pson), sd == 0 ? &D->par_son : &D->par_son_c);
   }
@@ -487,20 +560,48 @@ dh2_status upload_tree(Tree& tr) {
     delete D;
     return DH2_ENOMEM;
   }
-  size_t off = 0;
+  // neighbouring small lists go up in one copy each (a copy of a few bytes costs
+  // as much as one of 100 KB)
+  constexpr size_t kSmallList = 64 << 10;
+  std::vector<char> run;
+  size_t off = 0, run_off = 0;
+  bool up_ok = true;
+  auto flush = [&]() {
+    if (!run.empty() && up_ok)
+      up_ok = cudaMemcpy((char*)D->arena + run_off, run.data(), run.size(), cudaMemcpyHostToDevice) == cudaSuccess;
+    run.clear();
+  };
   for (auto& b : bufs) {
     *b.dst = (char*)D->arena + off;
-    if (b.bytes && b.src && cudaMemcpy(*b.dst, b.src, b.bytes, cudaMemcpyHostToDevice) != cudaSuccess) {
-      cudaGetLastError();
-      cudaFree(D->arena);
-      delete D;
-      return DH2_ECUDA;
+    const size_t step = align256(std::max<size_t>(b.bytes, 4));
+    if (step <= kSmallList) {
+      if (run.empty()) run_off = off;
+      const size_t at = run.size();
+      run.resize(at + step);
+      if (b.bytes && b.src) std::memcpy(run.data() + at, b.src, b.bytes);
+    } else {
+      flush();
+      if (b.src && up_ok) up_ok = cudaMemcpy(*b.dst, b.src, b.bytes, cudaMemcpyHostToDevice) == cudaSuccess;
     }
-    off += align256(std::max<size_t>(b.bytes, 4));
+    off += step;
+  }
+  flush();
+  if (!up_ok) {
+    cudaGetLastError();
+    cudaFree(D->arena);
+    delete D;
+    return DH2_ECUDA;
   }
   for (int sd = 0; sd < 2; ++sd)
     launch_colmap_expand(D->seg_dst[sd], D->seg_col0[sd], D->seg_w[sd], D->seg_blk[sd],
                          (int64_t)tr.side[sd].seg_dst.size(), D->gcol[sd], D->gblk[sd], nullptr);
+  for (int sd = 0; sd < 2; ++sd) {
+    cudaMemsetAsync(near_cursor[sd], 0, 4 * (size_t)nc, nullptr);
+    launch_mv_lists({D->inadm_list, (int32_t)D->ninadm, sd == 0 ? D->bt : D->bs, sd == 0 ? D->bs : D->bt, D->bt,
+                     D->cstart, D->csize, D->near_off, nc, near_ibegin[sd], near_ubegin[sd], near_cursor[sd], sd,
+                     D->near_items[sd], D->near_units[sd]},
+                    own_blk[sd], D->nown[sd], D->Soff, D->bpair[1 - sd], sd == 0 ? D->own : D->own_c, nullptr);
+  }
   if (cudaDeviceSynchronize() != cudaSuccess) {
     cudaGetLastError();
     cudaFree(D->arena);
@@ -2275,121 +2376,73 @@ void dh2_matrix_free(dh2_matrix* M) { matrix_release(M); }
 
 namespace {
 
+// The launches of y = G~ x (adj = 0: forward transformation on W, coupling
+// with S_b, backward on V, nearfield) or y = G~^* x (adj = 1: the sides
+// exchanged, S_b^* and G_b^*), with the coefficient vectors in buf (hx bytes
+// for x's, then y's).  Every coefficient is written before it is read.
 template <typename T>
-dh2_status run_matvec(const dh2_matrix* M, const void* xv, void* yv, int nrhs, cudaStream_t st) {
+dh2_status matvec_launches(const dh2_matrix* M, int adj, const void* xv, void* yv, int nrhs, void* buf, size_t hx,
+                           cudaStream_t st) {
   Tree& tr = M->tree->tr;
   Tree::Dev* D = tr.dev;
   const int64_t n = tr.n;
-  void* buf = nullptr;
-  const size_t hx = align256(sizeof(C2<T>) * D->h_elems[1] * nrhs);
-  const size_t hy = align256(sizeof(C2<T>) * D->h_elems[0] * nrhs);
-  if (dev_malloc_async(&buf, hx + hy + 256, st) != cudaSuccess) {
-    cudaGetLastError();
-    return DH2_ENOMEM;
-  }
+  const int si = adj ? 0 : 1, so = 1 - si;  // side of the input's basis, of the output's
   C2<T>* xh = (C2<T>*)buf;
   C2<T>* yh = (C2<T>*)((char*)buf + hx);
   const C2<T>* x = (const C2<T>*)xv;
   C2<T>* y = (C2<T>*)yv;
-  cudaMemsetAsync(y, 0, sizeof(C2<T>) * n * nrhs, st);
-  SideView<T> Vv = side_view<T>(tr, M, 0), Wv = side_view<T>(tr, M, 1);
-  // forward transformation (column basis), leaves then upwards
-  launch_mv_forward_leaf<T>(Wv, D->leaf_list[1], (int)D->nleaf[1], x, nrhs, n, xh, D->hoff[1], st);
+  DH2_CUDA_TRY(cudaMemsetAsync(y, 0, sizeof(C2<T>) * n * nrhs, st));
+  const SideView<T> Vin = side_view<T>(tr, M, si);
+  launch_mv_forward_leaf<T>(Vin, D->leaf_list[si], (int)D->nleaf[si], x, nrhs, n, xh, D->hoff[si], st);
   for (int l = tr.depth; l >= 0; --l) {
-    const int64_t b = D->lvl_nl_begin[1][l], e = D->lvl_end[1][l];
-    if (e > b) launch_mv_forward_up<T>(Wv, D->iota[1] + b, (int)(e - b), nrhs, xh, D->hoff[1], st);
+    const int64_t b = D->lvl_nl_begin[si][l], e = D->lvl_end[si][l];
+    if (e > b) launch_mv_forward_up<T>(Vin, D->iota[si] + b, (int)(e - b), nrhs, xh, D->hoff[si], st);
   }
   MvArgs<T> a;
-  a.V = Vv;
-  a.W = Wv;
+  a.V = side_view<T>(tr, M, so);
+  a.W = Vin;
+  a.items = D->near_items[adj];
+  a.units = D->near_units[adj];
+  a.nunits = D->nnear_units[adj];
   a.S = (const C2<T>*)M->S;
-  a.Soff = D->Soff;
-  a.own_ptr = D->own_ptr;
-  a.own_blk = D->own_blk;
-  a.bpair_col = D->bpair[1];
+  a.own_ptr = adj ? D->own_ptr_c : D->own_ptr;
+  a.own = adj ? D->own_c : D->own;
   a.xh = xh;
-  a.xhoff = D->hoff[1];
+  a.xhoff = D->hoff[si];
   a.yh = yh;
-  a.yhoff = D->hoff[0];
-  a.par_ptr = D->par_ptr;
-  a.par_pair = D->par_pair;
-  a.par_son = D->par_son;
-  a.bt = D->bt;
-  a.bs = D->bs;
+  a.yhoff = D->hoff[so];
+  a.par_ptr = adj ? D->par_ptr_c : D->par_ptr;
+  a.par_pair = adj ? D->par_pair_c : D->par_pair;
+  a.par_son = adj ? D->par_son_c : D->par_son;
   a.near = (const C2<T>*)M->near;
-  a.near_off = D->near_off;
   a.G = (const C2<T>*)M->G;
   a.ld = M->ld;
-  launch_mv_coupling<T>(a, (int)D->npairs[0], nrhs, st);
+  if (adj) launch_mv_coupling_adj<T>(a, (int)D->npairs[so], nrhs, st);
+  else launch_mv_coupling<T>(a, (int)D->npairs[so], nrhs, st);
   // backward transformation, top-down
   for (int l = 1; l <= tr.depth; ++l) {
-    const int64_t b = D->lvl_begin[0][l], e = D->lvl_end[0][l];
-    if (e > b) launch_mv_backward_down<T>(a, D->iota[0] + b, (int)(e - b), nrhs, st);
+    const int64_t b = D->lvl_begin[so][l], e = D->lvl_end[so][l];
+    if (e > b) launch_mv_backward_down<T>(a, D->iota[so] + b, (int)(e - b), nrhs, st);
   }
-  launch_mv_backward_leaf<T>(a, D->leaf_list[0], (int)D->nleaf[0], nrhs, y, n, st);
-  launch_mv_near<T>(a, D->inadm_list, (int)D->ninadm, nrhs, x, y, n, st);
-  cudaFreeAsync(buf, st);
+  launch_mv_backward_leaf<T>(a, D->leaf_list[so], D->leaf_units[so], D->nleaf_units[so], nrhs, y, n, st);
+  launch_mv_near<T>(a, adj != 0, nrhs, x, y, n, st);
   DH2_CUDA_TRY(cudaGetLastError());
   return DH2_OK;
 }
 
-// y = G~^* x: the product of Section 4 with the roles of the row and column
-// bases exchanged (forward on V, coupling with S_b^*, backward on W) plus
-// G_b^* on the nearfield.
 template <typename T>
-dh2_status run_matvec_adj(const dh2_matrix* M, const void* xv, void* yv, int nrhs, cudaStream_t st) {
-  Tree& tr = M->tree->tr;
-  Tree::Dev* D = tr.dev;
-  const int64_t n = tr.n;
+dh2_status run_matvec(const dh2_matrix* M, int adj, const void* x, void* y, int nrhs, cudaStream_t st) {
+  const Tree::Dev* D = M->tree->tr.dev;
   void* buf = nullptr;
-  const size_t hx = align256(sizeof(C2<T>) * D->h_elems[0] * nrhs);
-  const size_t hy = align256(sizeof(C2<T>) * D->h_elems[1] * nrhs);
+  const size_t hx = align256(sizeof(C2<T>) * D->h_elems[adj ? 0 : 1] * nrhs);
+  const size_t hy = align256(sizeof(C2<T>) * D->h_elems[adj ? 1 : 0] * nrhs);
   if (dev_malloc_async(&buf, hx + hy + 256, st) != cudaSuccess) {
     cudaGetLastError();
     return DH2_ENOMEM;
   }
-  C2<T>* xh = (C2<T>*)buf;
-  C2<T>* yh = (C2<T>*)((char*)buf + hx);
-  const C2<T>* x = (const C2<T>*)xv;
-  C2<T>* y = (C2<T>*)yv;
-  cudaMemsetAsync(y, 0, sizeof(C2<T>) * n * nrhs, st);
-  SideView<T> Vv = side_view<T>(tr, M, 0), Wv = side_view<T>(tr, M, 1);
-  launch_mv_forward_leaf<T>(Vv, D->leaf_list[0], (int)D->nleaf[0], x, nrhs, n, xh, D->hoff[0], st);
-  for (int l = tr.depth; l >= 0; --l) {
-    const int64_t b = D->lvl_nl_begin[0][l], e = D->lvl_end[0][l];
-    if (e > b) launch_mv_forward_up<T>(Vv, D->iota[0] + b, (int)(e - b), nrhs, xh, D->hoff[0], st);
-  }
-  MvArgs<T> a;
-  a.V = Wv;  // exchanged sides
-  a.W = Vv;
-  a.S = (const C2<T>*)M->S;
-  a.Soff = D->Soff;
-  a.own_ptr = D->own_ptr_c;
-  a.own_blk = D->own_blk_c;
-  a.bpair_col = D->bpair[0];
-  a.xh = xh;
-  a.xhoff = D->hoff[0];
-  a.yh = yh;
-  a.yhoff = D->hoff[1];
-  a.par_ptr = D->par_ptr_c;
-  a.par_pair = D->par_pair_c;
-  a.par_son = D->par_son_c;
-  a.bt = D->bt;
-  a.bs = D->bs;
-  a.near = (const C2<T>*)M->near;
-  a.near_off = D->near_off;
-  a.G = (const C2<T>*)M->G;
-  a.ld = M->ld;
-  launch_mv_coupling_adj<T>(a, (int)D->npairs[1], nrhs, st);
-  for (int l = 1; l <= tr.depth; ++l) {
-    const int64_t b = D->lvl_begin[1][l], e = D->lvl_end[1][l];
-    if (e > b) launch_mv_backward_down<T>(a, D->iota[1] + b, (int)(e - b), nrhs, st);
-  }
-  launch_mv_backward_leaf<T>(a, D->leaf_list[1], (int)D->nleaf[1], nrhs, y, n, st);
-  launch_mv_near_adj<T>(a, D->inadm_list, (int)D->ninadm, nrhs, x, y, n, st);
+  const dh2_status s = matvec_launches<T>(M, adj, x, y, nrhs, buf, hx, st);
   cudaFreeAsync(buf, st);
-  DH2_CUDA_TRY(cudaGetLastError());
-  return DH2_OK;
+  return s;
 }
 
 // Relative spectral error |G_ref - G~|_2 / |G_ref|_2 by power iteration (the
@@ -2444,14 +2497,14 @@ dh2_status run_error_spectral(dh2_matrix* M, const void* Gref, dh2_dtype rdt, in
       gemv(false, v, u);
       if (err) {
         launch_to_type<T>(v, xt, n, st);
-        s = run_matvec<T>(M, xt, yt, 1, st);
+        s = run_matvec<T>(M, 0, xt, yt, 1, st);
         if (s != DH2_OK) return s;
         launch_sub<T>(u, yt, n, st);
       }
       gemv(true, u, w);
       if (err) {
         launch_to_type<T>(u, xt, n, st);
-        s = run_matvec_adj<T>(M, xt, yt, 1, st);
+        s = run_matvec<T>(M, 1, xt, yt, 1, st);
         if (s != DH2_OK) return s;
         launch_sub<T>(w, yt, n, st);
       }
@@ -2533,14 +2586,14 @@ extern "C" {
 
 dh2_status dh2_matvec(const dh2_matrix* M, const void* x, void* y, int32_t nrhs, void* stream) {
   if (!M || !x || !y || nrhs < 1) return DH2_EINVAL;
-  return mode_f32(M->mode) ? run_matvec<float>(M, x, y, nrhs, (cudaStream_t)stream)
-                                  : run_matvec<double>(M, x, y, nrhs, (cudaStream_t)stream);
+  return mode_f32(M->mode) ? run_matvec<float>(M, 0, x, y, nrhs, (cudaStream_t)stream)
+                           : run_matvec<double>(M, 0, x, y, nrhs, (cudaStream_t)stream);
 }
 
 dh2_status dh2_matvec_adjoint(const dh2_matrix* M, const void* x, void* y, int32_t nrhs, void* stream) {
   if (!M || !x || !y || nrhs < 1) return DH2_EINVAL;
-  return mode_f32(M->mode) ? run_matvec_adj<float>(M, x, y, nrhs, (cudaStream_t)stream)
-                           : run_matvec_adj<double>(M, x, y, nrhs, (cudaStream_t)stream);
+  return mode_f32(M->mode) ? run_matvec<float>(M, 1, x, y, nrhs, (cudaStream_t)stream)
+                           : run_matvec<double>(M, 1, x, y, nrhs, (cudaStream_t)stream);
 }
 
 dh2_status dh2_error(const dh2_matrix* Mc, const void* G_ref, dh2_dtype ref_dtype, int64_t ld, int32_t which,
@@ -2790,9 +2843,7 @@ dh2_status noalloc_scratch_address(int dev, void** out) {
 
 template <typename T>
 dh2_status run_matvec_noalloc(const dh2_matrix* M, const void* xv, void* yv, int nrhs, cudaStream_t st) {
-  Tree& tr = M->tree->tr;
-  Tree::Dev* D = tr.dev;
-  const int64_t n = tr.n;
+  const Tree::Dev* D = M->tree->tr.dev;
   const size_t hx = align256(sizeof(C2<T>) * D->h_elems[1] * nrhs);
   const size_t hy = align256(sizeof(C2<T>) * D->h_elems[0] * nrhs);
   if (hx + hy > kNoAllocScratchBytes) return DH2_EUNSUPPORTED;
@@ -2804,49 +2855,7 @@ dh2_status run_matvec_noalloc(const dh2_matrix* M, const void* xv, void* yv, int
     const dh2_status s = noalloc_scratch_address(dev, &buf);
     if (s != DH2_OK) return s;
   }
-  // every coefficient is written before it is read (forward transformation,
-  // then coupling), so nothing in the scratch array needs clearing
-  C2<T>* xh = (C2<T>*)buf;
-  C2<T>* yh = (C2<T>*)((char*)buf + hx);
-  const C2<T>* x = (const C2<T>*)xv;
-  C2<T>* y = (C2<T>*)yv;
-  DH2_CUDA_TRY(cudaMemsetAsync(y, 0, sizeof(C2<T>) * n * nrhs, st));
-  SideView<T> Vv = side_view<T>(tr, M, 0), Wv = side_view<T>(tr, M, 1);
-  launch_mv_forward_leaf<T>(Wv, D->leaf_list[1], (int)D->nleaf[1], x, nrhs, n, xh, D->hoff[1], st);
-  for (int l = tr.depth; l >= 0; --l) {
-    const int64_t b = D->lvl_nl_begin[1][l], e = D->lvl_end[1][l];
-    if (e > b) launch_mv_forward_up<T>(Wv, D->iota[1] + b, (int)(e - b), nrhs, xh, D->hoff[1], st);
-  }
-  MvArgs<T> a;
-  a.V = Vv;
-  a.W = Wv;
-  a.S = (const C2<T>*)M->S;
-  a.Soff = D->Soff;
-  a.own_ptr = D->own_ptr;
-  a.own_blk = D->own_blk;
-  a.bpair_col = D->bpair[1];
-  a.xh = xh;
-  a.xhoff = D->hoff[1];
-  a.yh = yh;
-  a.yhoff = D->hoff[0];
-  a.par_ptr = D->par_ptr;
-  a.par_pair = D->par_pair;
-  a.par_son = D->par_son;
-  a.bt = D->bt;
-  a.bs = D->bs;
-  a.near = (const C2<T>*)M->near;
-  a.near_off = D->near_off;
-  a.G = (const C2<T>*)M->G;
-  a.ld = M->ld;
-  launch_mv_coupling<T>(a, (int)D->npairs[0], nrhs, st);
-  for (int l = 1; l <= tr.depth; ++l) {
-    const int64_t b = D->lvl_begin[0][l], e = D->lvl_end[0][l];
-    if (e > b) launch_mv_backward_down<T>(a, D->iota[0] + b, (int)(e - b), nrhs, st);
-  }
-  launch_mv_backward_leaf<T>(a, D->leaf_list[0], (int)D->nleaf[0], nrhs, y, n, st);
-  launch_mv_near<T>(a, D->inadm_list, (int)D->ninadm, nrhs, x, y, n, st);
-  DH2_CUDA_TRY(cudaGetLastError());
-  return DH2_OK;
+  return matvec_launches<T>(M, 0, xv, yv, nrhs, buf, hx, st);
 }
 
 }  // namespace

@@ -1,6 +1,6 @@
 // Kernels around the per-pair factorisation: block norms and nearfield copy,
-// basis expansion by Eq. (nested), the projection S_b, the matrix-vector
-// product of Section 4 and the blockwise error.
+// basis expansion by Eq. (nested), the projection S_b and the error measures
+// (the matrix-vector products are in dh2_mv.cu).
 #include "dh2_check.cuh"
 #include "dh2_internal.h"
 #include "dh2_ops.cuh"
@@ -19,13 +19,6 @@ template <typename T>
 __device__ __forceinline__ C2<T> cmul(C2<T> a, C2<T> b) {
   return C2<T>{a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re};
 }
-template <typename T>
-__device__ __forceinline__ C2<T> cmulc(C2<T> a, C2<T> b) {  // a * conj(b)
-  return C2<T>{a.re * b.re + a.im * b.im, a.im * b.re - a.re * b.im};
-}
-template <typename T>
-__device__ __forceinline__ C2<T> cconj(C2<T> a) { return C2<T>{a.re, -a.im}; }
-
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v) {
 #pragma unroll
@@ -396,138 +389,6 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? DH2_PROJ_MINB : 1) proje
   }
 }
 
-// ---------------------------------------------------------------- matvec
-// forward transformation, leaves: xh_sc = W_sc^* x|_s (Eq. mvm1)
-template <typename T>
-__global__ void mv_forward_leaf(SideView<T> W, const int32_t* pairs, const C2<T>* x, int nrhs, int64_t n,
-                                C2<T>* xh, const int64_t* hoff) {
-  const int pid = pairs[blockIdx.x];
-  const int k = W.rank[pid];
-  const int m = W.csize[W.cluster[pid]];
-  const int64_t s0 = W.cstart[W.cluster[pid]];
-  const C2<T>* Q = W.Q + W.Qoff[pid];
-  for (int idx = threadIdx.x; idx < k * nrhs; idx += blockDim.x) {
-    const int qq = idx % k, rh = idx / k;
-    C2<T> acc = czero<T>();
-    for (int i = 0; i < m; ++i) acc = cadd(acc, cmulc(x[s0 + i + rh * n], Q[i + (int64_t)qq * m]));
-    xh[hoff[pid] * nrhs + qq + (int64_t)rh * k] = acc;
-  }
-}
-
-// forward transformation, non-leaves: xh_sc = sum_s' E_s'c^* xh_s'c'
-template <typename T>
-__global__ void mv_forward_up(SideView<T> W, const int32_t* pairs, int nrhs, C2<T>* xh, const int64_t* hoff) {
-  const int pid = pairs[blockIdx.x];
-  const int k = W.rank[pid];
-  const int ldq = W.rowcap[pid];
-  const C2<T>* E = W.Q + W.Qoff[pid];
-  for (int idx = threadIdx.x; idx < k * nrhs; idx += blockDim.x) {
-    const int qq = idx % k, rh = idx / k;
-    C2<T> acc = czero<T>();
-    int eoff = 0;
-    for (int j = 0; j < 2; ++j) {
-      const int sp = W.son[2 * pid + j];
-      const int kj = W.rank[sp];
-      const C2<T>* xs = xh + hoff[sp] * nrhs + (int64_t)rh * kj;
-      for (int l = 0; l < kj; ++l) acc = cadd(acc, cmulc(xs[l], E[eoff + l + (int64_t)qq * ldq]));
-      eoff += kj;
-    }
-    xh[hoff[pid] * nrhs + qq + (int64_t)rh * k] = acc;
-  }
-}
-
-// coupling: yh_tc = sum over own blocks b of S_b xh_{s c} (Eq. mvm2)
-template <typename T>
-__global__ void mv_coupling(MvArgs<T> a, int nrhs) {
-  const int pid = blockIdx.x;
-  const int kt = a.V.rank[pid];
-  for (int idx = threadIdx.x; idx < kt * nrhs; idx += blockDim.x) {
-    const int qq = idx % kt, rh = idx / kt;
-    C2<T> acc = czero<T>();
-    for (int64_t e = a.own_ptr[pid]; e < a.own_ptr[pid + 1]; ++e) {
-      const int b = a.own_blk[e];
-      const int Ps = a.bpair_col[b];
-      const int ks = a.W.rank[Ps];
-      const C2<T>* S = a.S + a.Soff[b];
-      const C2<T>* xs = a.xh + a.xhoff[Ps] * nrhs + (int64_t)rh * ks;
-      for (int l = 0; l < ks; ++l) acc = cadd(acc, cmul(S[qq + (int64_t)l * kt], xs[l]));
-    }
-    a.yh[a.yhoff[pid] * nrhs + qq + (int64_t)rh * kt] = acc;
-  }
-}
-
-// backward transformation: yh_t'c' += E_t'c yh_tc over the father pairs (t, c)
-// with sd(c) = c', gathered per son pair (figure "Fast forward and backward
-// transformation", right).
-template <typename T>
-__global__ void mv_backward_down(MvArgs<T> a, const int32_t* pairs, int nrhs) {
-  const int pid = pairs[blockIdx.x];
-  const int k = a.V.rank[pid];
-  for (int idx = threadIdx.x; idx < k * nrhs; idx += blockDim.x) {
-    const int qq = idx % k, rh = idx / k;
-    C2<T> acc = a.yh[a.yhoff[pid] * nrhs + qq + (int64_t)rh * k];
-    for (int64_t e = a.par_ptr[pid]; e < a.par_ptr[pid + 1]; ++e) {
-      const int fp = a.par_pair[e];
-      const int j = a.par_son[e];
-      const int kf = a.V.rank[fp];
-      const int ldq = a.V.rowcap[fp];
-      const int eoff = j == 0 ? 0 : a.V.rank[a.V.son[2 * fp]];
-      const C2<T>* E = a.V.Q + a.V.Qoff[fp];
-      const C2<T>* yf = a.yh + a.yhoff[fp] * nrhs + (int64_t)rh * kf;
-      for (int l = 0; l < kf; ++l) acc = cadd(acc, cmul(E[eoff + qq + (int64_t)l * ldq], yf[l]));
-    }
-    a.yh[a.yhoff[pid] * nrhs + qq + (int64_t)rh * k] = acc;
-  }
-}
-
-template <typename T>
-__device__ __forceinline__ void catomic_add(C2<T>* p, C2<T> v) {
-  atomicAdd(&p->re, v.re);
-  atomicAdd(&p->im, v.im);
-}
-
-// leaves: y|_t += V_tc yh_tc (Eq. mvm3)
-template <typename T>
-__global__ void mv_backward_leaf(MvArgs<T> a, const int32_t* pairs, int nrhs, C2<T>* y, int64_t n) {
-  const int pid = pairs[blockIdx.x];
-  const int k = a.V.rank[pid];
-  if (k == 0) return;
-  const int m = a.V.csize[a.V.cluster[pid]];
-  const int64_t t0 = a.V.cstart[a.V.cluster[pid]];
-  const C2<T>* Q = a.V.Q + a.V.Qoff[pid];
-  for (int idx = threadIdx.x; idx < m * nrhs; idx += blockDim.x) {
-    const int i = idx % m, rh = idx / m;
-    const C2<T>* yh = a.yh + a.yhoff[pid] * nrhs + (int64_t)rh * k;
-    C2<T> acc = czero<T>();
-    for (int l = 0; l < k; ++l) acc = cadd(acc, cmul(Q[i + (int64_t)l * m], yh[l]));
-    catomic_add(y + t0 + i + rh * n, acc);
-  }
-}
-
-// nearfield: y|_t += G_b x|_s for inadmissible leaves
-template <typename T>
-__global__ void mv_near(MvArgs<T> a, const int32_t* blocks, int nrhs, const C2<T>* x, C2<T>* y, int64_t n) {
-  const int b = blocks[blockIdx.x];
-  const int t = a.bt[b], s = a.bs[b];
-  const int mt = a.V.csize[t], ms = a.V.csize[s];
-  const int64_t t0 = a.V.cstart[t], s0 = a.V.cstart[s];
-  const C2<T>* Gb;
-  int64_t ldb;
-  if (a.near) {
-    Gb = a.near + a.near_off[b];
-    ldb = mt;
-  } else {
-    Gb = a.G + s0 * a.ld + t0;
-    ldb = a.ld;
-  }
-  for (int idx = threadIdx.x; idx < mt * nrhs; idx += blockDim.x) {
-    const int i = idx % mt, rh = idx / mt;
-    C2<T> acc = czero<T>();
-    for (int j = 0; j < ms; ++j) acc = cadd(acc, cmul(Gb[i + (int64_t)j * ldb], x[s0 + j + rh * n]));
-    catomic_add(y + t0 + i + rh * n, acc);
-  }
-}
-
 // ---------------------------------------------------------------- error
 // sum over blocks of |G_ref - G~|_F^2 and |G_ref|_F^2 in FP64.
 template <typename T, typename RT>
@@ -601,63 +462,6 @@ __global__ void __launch_bounds__(256) error_kernel(ErrArgs<T> a, const C2<RT>* 
   if (threadIdx.x == 0) {
     atomicAdd(acc_out, se);
     atomicAdd(acc_out + 1, sr);
-  }
-}
-
-// ---------------------------------------------------------------- adjoint product
-// y = G~^* x: the forward transformation runs on the row basis V, the
-// coupling applies S_b^* from row pairs to column pairs, the backward
-// transformation runs on the column basis W (the roles of V and W in
-// Section 4 exchanged), plus G_b^* on the nearfield.  The kernels of the
-// product are reused with an MvArgs whose V and W, coefficient vectors and
-// pair lists are those of the exchanged sides; coupling and nearfield need
-// their own (conjugate-transposed) loops.
-//
-// coupling: yh_sc = sum over the column pair's blocks b of S_b^* xh_tc
-template <typename T>
-__global__ void mv_coupling_adj(MvArgs<T> a, int nrhs) {
-  const int pid = blockIdx.x;
-  const int kout = a.V.rank[pid];  // rank of this column pair
-  for (int idx = threadIdx.x; idx < kout * nrhs; idx += blockDim.x) {
-    const int qq = idx % kout, rh = idx / kout;
-    C2<T> acc = czero<T>();
-    for (int64_t e = a.own_ptr[pid]; e < a.own_ptr[pid + 1]; ++e) {
-      const int b = a.own_blk[e];
-      const int Pt = a.bpair_col[b];   // the block's row pair
-      const int kin = a.W.rank[Pt];
-      const C2<T>* S = a.S + a.Soff[b];  // kin x kout, column-major
-      const C2<T>* xs = a.xh + a.xhoff[Pt] * nrhs + (int64_t)rh * kin;
-      for (int l = 0; l < kin; ++l) acc = cadd(acc, cmul(cconj(S[l + (int64_t)qq * kin]), xs[l]));
-    }
-    a.yh[a.yhoff[pid] * nrhs + qq + (int64_t)rh * kout] = acc;
-  }
-}
-
-// nearfield: y|_s += G_b^* x|_t for inadmissible leaves
-template <typename T>
-__global__ void mv_near_adj(MvArgs<T> a, const int32_t* blocks, int nrhs, const C2<T>* x, C2<T>* y, int64_t n) {
-  const int b = blocks[blockIdx.x];
-  const int t = a.bt[b], s = a.bs[b];
-  const int mt = a.V.csize[t], ms = a.V.csize[s];
-  const int64_t t0 = a.V.cstart[t], s0 = a.V.cstart[s];
-  const C2<T>* Gb;
-  int64_t ldb;
-  if (a.near) {
-    Gb = a.near + a.near_off[b];
-    ldb = mt;
-  } else {
-    Gb = a.G + s0 * a.ld + t0;
-    ldb = a.ld;
-  }
-  // one warp per column of the block: lanes over its rows
-  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int cj = wp; cj < ms * nrhs; cj += nw) {
-    const int j = cj % ms, rh = cj / ms;
-    C2<T> acc = czero<T>();
-    for (int i = lane; i < mt; i += 32) acc = cadd(acc, cmul(cconj(Gb[i + (int64_t)j * ldb]), x[t0 + i + rh * n]));
-    acc.re = warp_sum(acc.re);
-    acc.im = warp_sum(acc.im);
-    if (lane == 0) catomic_add(y + s0 + j + rh * n, acc);
   }
 }
 
@@ -921,49 +725,12 @@ template <typename T>
 void launch_project(const ProjArgs<T>& a, int nadm, cudaStream_t st) {
   if (nadm > 0) project_kernel<T><<<(nadm + 3) / 4, 128, 0, st>>>(a, nadm);
 }
-template <typename T>
-void launch_mv_forward_leaf(const SideView<T>& W, const int32_t* pairs, int np, const C2<T>* x, int nrhs,
-                            int64_t n, C2<T>* xh, const int64_t* hoff, cudaStream_t st) {
-  if (np > 0) mv_forward_leaf<T><<<np, 128, 0, st>>>(W, pairs, x, nrhs, n, xh, hoff);
-}
-template <typename T>
-void launch_mv_forward_up(const SideView<T>& W, const int32_t* pairs, int np, int nrhs, C2<T>* xh,
-                          const int64_t* hoff, cudaStream_t st) {
-  if (np > 0) mv_forward_up<T><<<np, 128, 0, st>>>(W, pairs, nrhs, xh, hoff);
-}
-template <typename T>
-void launch_mv_coupling(const MvArgs<T>& a, int npairs_row, int nrhs, cudaStream_t st) {
-  if (npairs_row > 0) mv_coupling<T><<<npairs_row, 128, 0, st>>>(a, nrhs);
-}
-template <typename T>
-void launch_mv_backward_down(const MvArgs<T>& a, const int32_t* pairs, int np, int nrhs, cudaStream_t st) {
-  if (np > 0) mv_backward_down<T><<<np, 128, 0, st>>>(a, pairs, nrhs);
-}
-template <typename T>
-void launch_mv_backward_leaf(const MvArgs<T>& a, const int32_t* pairs, int np, int nrhs, C2<T>* y, int64_t n,
-                             cudaStream_t st) {
-  if (np > 0) mv_backward_leaf<T><<<np, 128, 0, st>>>(a, pairs, nrhs, y, n);
-}
-template <typename T>
-void launch_mv_near(const MvArgs<T>& a, const int32_t* blocks, int nb, int nrhs, const C2<T>* x, C2<T>* y,
-                    int64_t n, cudaStream_t st) {
-  if (nb > 0) mv_near<T><<<nb, 128, 0, st>>>(a, blocks, nrhs, x, y, n);
-}
 template <typename T, typename RT>
 void launch_error(const ErrArgs<T>& a, const C2<RT>* Gref, int64_t ldr, int nblocks, double* acc,
                   cudaStream_t st) {
   if (nblocks > 0) error_kernel<T, RT><<<nblocks, 256, 0, st>>>(a, Gref, ldr, acc);
 }
 
-template <typename T>
-void launch_mv_coupling_adj(const MvArgs<T>& a, int npairs_col, int nrhs, cudaStream_t st) {
-  if (npairs_col > 0) mv_coupling_adj<T><<<npairs_col, 128, 0, st>>>(a, nrhs);
-}
-template <typename T>
-void launch_mv_near_adj(const MvArgs<T>& a, const int32_t* blocks, int nb, int nrhs, const C2<T>* x, C2<T>* y,
-                        int64_t n, cudaStream_t st) {
-  if (nb > 0) mv_near_adj<T><<<nb, 128, 0, st>>>(a, blocks, nrhs, x, y, n);
-}
 template <typename RT>
 void launch_gemv(const C2<RT>* G, int64_t ld, const ErrArgs<float>& gen, int64_t n, bool trans, const C2<double>* x,
                  C2<double>* y, cudaStream_t st) {
@@ -1045,23 +812,10 @@ void launch_colw(const int32_t* gblk, const double* invw, T* colw, int64_t n, cu
   template void launch_norms_near<T>(const NormsArgs<T>*, const uint32_t*, int, cudaStream_t);            \
   template void launch_expand<T>(const SideView<T>&, const int32_t*, int, cudaStream_t);                   \
   template void launch_project<T>(const ProjArgs<T>&, int, cudaStream_t);                                  \
-  template void launch_mv_forward_leaf<T>(const SideView<T>&, const int32_t*, int, const C2<T>*, int,      \
-                                          int64_t, C2<T>*, const int64_t*, cudaStream_t);                  \
-  template void launch_mv_forward_up<T>(const SideView<T>&, const int32_t*, int, int, C2<T>*,              \
-                                        const int64_t*, cudaStream_t);                                     \
-  template void launch_mv_coupling<T>(const MvArgs<T>&, int, int, cudaStream_t);                           \
-  template void launch_mv_backward_down<T>(const MvArgs<T>&, const int32_t*, int, int, cudaStream_t);      \
-  template void launch_mv_backward_leaf<T>(const MvArgs<T>&, const int32_t*, int, int, C2<T>*, int64_t,    \
-                                           cudaStream_t);                                                  \
-  template void launch_mv_near<T>(const MvArgs<T>&, const int32_t*, int, int, const C2<T>*, C2<T>*,        \
-                                  int64_t, cudaStream_t);                                                  \
   template void launch_error<T, float>(const ErrArgs<T>&, const C2<float>*, int64_t, int, double*,        \
                                        cudaStream_t);                                                      \
   template void launch_error<T, double>(const ErrArgs<T>&, const C2<double>*, int64_t, int, double*,      \
                                         cudaStream_t);                                                      \
-  template void launch_mv_coupling_adj<T>(const MvArgs<T>&, int, int, cudaStream_t);                       \
-  template void launch_mv_near_adj<T>(const MvArgs<T>&, const int32_t*, int, int, const C2<T>*, C2<T>*,    \
-                                      int64_t, cudaStream_t);                                              \
   template void launch_closed_form<T>(const ErrArgs<T>&, const double*, int, double*, cudaStream_t);            \
   template void launch_to_type<T>(const C2<double>*, C2<T>*, int64_t, cudaStream_t);                       \
   template void launch_norms_adm<T>(const NormsArgs<T>*, const uint64_t*, int64_t, const uint32_t*, const int64_t*, \

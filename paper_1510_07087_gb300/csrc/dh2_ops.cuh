@@ -66,14 +66,67 @@ struct ProjArgs {
   const int64_t* Soff;
 };
 
+// Work lists of the nearfield products (built once per tree).  A product
+// y|_t += G_b x|_s gathers the blocks of one row cluster: unit = a run of items
+// (blocks of that cluster) and a slab of at most kNearRows of its rows.  The
+// adjoint product gathers the blocks of one column cluster: unit = a run of
+// items and at most kNearRows of its columns.
+// The nearfield copy's blocks start at even entries (16-byte copies); a block
+// is taken in pieces of at most kNearElems entries and kNearPiece columns (the
+// adjoint: rows), an even number each but the last.
+constexpr int32_t kNearRows = 128;
+constexpr int32_t kNearElems = 1792;
+constexpr int32_t kNearPiece = 48;
+struct NearItem {
+  int64_t off;  // nearfield copy: element offset of the block
+  int32_t o0;   // first index of the block in the gathered dimension (column of G; adjoint: row of G)
+  int32_t w;    // its extent in that dimension
+  int32_t ld;   // nearfield copy: leading dimension of the block
+  int32_t pw;   // columns (adjoint: rows) of a piece
+};
+struct NearUnit {
+  int32_t first, count;  // items
+  int32_t c0, cw;        // first row (adjoint: column) of the unit in its cluster, and how many
+  int32_t out;           // their first index in the vectors
+  int32_t pad;
+};
+// slabs of a cluster of `mine` rows (columns), and their height
+__host__ __device__ constexpr int32_t near_slabs(int32_t mine) { return (mine + kNearRows - 1) / kNearRows; }
+__host__ __device__ constexpr int32_t near_slab(int32_t mine) {
+  return (mine + near_slabs(mine) - 1) / near_slabs(mine);
+}
+// Inputs and outputs of the lists of one side: the inadmissible blocks, their
+// clusters (own: gathered by; other), sizes and nearfield offsets; per cluster
+// its first item and first unit (counted on the host), a zeroed cursor.
+struct NearFill {
+  const int32_t* blocks;
+  int32_t nblocks;
+  const int32_t *own, *other, *bt, *cstart, *csize;
+  const int64_t* near_off;
+  int32_t nclusters;
+  const int32_t *item_begin, *unit_begin;
+  int32_t* cursor;
+  int32_t sd;
+  NearItem* items;
+  NearUnit* units;
+};
+
+// One block of a pair's own blocks: where S_b lies and the block's other pair.
+struct OwnItem {
+  int64_t soff;
+  int32_t pair;
+  int32_t pad;
+};
+
 template <typename T>
 struct MvArgs {
   SideView<T> V, W;
+  const NearItem* items;
+  const NearUnit* units;
+  int32_t nunits;
   const C2<T>* S;
-  const int64_t* Soff;
   const int64_t* own_ptr;   // row pairs: own blocks (CSR)
-  const int32_t* own_blk;
-  const int32_t* bpair_col;
+  const OwnItem* own;
   const C2<T>* xh;
   const int64_t* xhoff;     // column pairs
   C2<T>* yh;
@@ -81,10 +134,7 @@ struct MvArgs {
   const int64_t* par_ptr;   // row pairs: father pairs (CSR)
   const int32_t* par_pair;
   const int32_t* par_son;
-  const int32_t* bt;
-  const int32_t* bs;
-  const C2<T>* near;
-  const int64_t* near_off;
+  const C2<T>* near;  // nearfield copy, or NULL: the blocks are read from G
   const C2<T>* G;
   int64_t ld;
 };
@@ -130,6 +180,11 @@ void launch_norms_near(const NormsArgs<T>* args_dev, const uint32_t* codes, int 
 template <typename T>
 void launch_norms_adm(const NormsArgs<T>* args_dev, const uint64_t* pieces, int64_t npieces, const uint32_t* codes,
                       const int64_t* pbegin, int64_t nblocks, double* partial, cudaStream_t st);
+struct OwnItem;
+// the nearfield lists of one side, and its own-block records from the block
+// ids, coupling offsets and the blocks' pairs of the other side
+void launch_mv_lists(const NearFill& f, const int32_t* own_blk, int64_t nown, const int64_t* Soff,
+                     const int32_t* other_pair, OwnItem* own, cudaStream_t st);
 template <typename T> void launch_expand(const SideView<T>& S, const int32_t* pairs, int n, cudaStream_t st);
 template <typename T> void launch_project(const ProjArgs<T>& a, int nadm, cudaStream_t st);
 template <typename T>
@@ -142,21 +197,16 @@ template <typename T> void launch_mv_coupling(const MvArgs<T>& a, int npairs_row
 template <typename T>
 void launch_mv_backward_down(const MvArgs<T>& a, const int32_t* pairs, int np, int nrhs, cudaStream_t st);
 template <typename T>
-void launch_mv_backward_leaf(const MvArgs<T>& a, const int32_t* pairs, int np, int nrhs, C2<T>* y, int64_t n,
-                             cudaStream_t st);
+void launch_mv_backward_leaf(const MvArgs<T>& a, const int32_t* pairs, const NearUnit* units, int nunits, int nrhs,
+                             C2<T>* y, int64_t n, cudaStream_t st);
 template <typename T>
-void launch_mv_near(const MvArgs<T>& a, const int32_t* blocks, int nb, int nrhs, const C2<T>* x, C2<T>* y,
-                    int64_t n, cudaStream_t st);
+void launch_mv_near(const MvArgs<T>& a, bool adj, int nrhs, const C2<T>* x, C2<T>* y, int64_t n, cudaStream_t st);
 template <typename T, typename RT>
 void launch_error(const ErrArgs<T>& a, const C2<RT>* Gref, int64_t ldr, int nblocks, double* acc,
                   cudaStream_t st);
-// adjoint product: coupling with S_b^* into column pairs, nearfield with G_b^*
-// (MvArgs with the sides exchanged: V = column basis, W = row basis, own and
+// adjoint product: coupling with S_b^* into column pairs (MvArgs with the sides exchanged: V = column basis, W = row basis, own and
 // father lists of the column side, bpair_col = the blocks' row pairs)
 template <typename T> void launch_mv_coupling_adj(const MvArgs<T>& a, int npairs_col, int nrhs, cudaStream_t st);
-template <typename T>
-void launch_mv_near_adj(const MvArgs<T>& a, const int32_t* blocks, int nb, int nrhs, const C2<T>* x, C2<T>* y,
-                        int64_t n, cudaStream_t st);
 // y = G_ref x or G_ref^* x in FP64 (G NULL: entries generated from gen's points)
 template <typename RT>
 void launch_gemv(const C2<RT>* G, int64_t ld, const ErrArgs<float>& gen, int64_t n, bool trans, const C2<double>* x,
