@@ -174,6 +174,8 @@ struct dh2_matrix {
   double* pts = nullptr;  // device, permuted order
   double kappa = 0.0, diag = 0.0;
   std::vector<double> pts_h;
+  double pts_factor = 1.0;
+  float4* pts32 = nullptr;  // FP32 modes: points and normals split into two floats (Gen<float>)
   double* nrm = nullptr;  // device normals after the points (double layer), or NULL
 };
 
@@ -687,10 +689,18 @@ void fill_args(dh2_matrix* M, const dh2_compress_params& cp, PairArgs<T>& pa, No
   na.near = (C2<T>*)M->near;
   na.near_off = D->near_off;
   na.copy = M->nearfield_copy;
-  na.pts = M->pts;
-  na.nrm = M->nrm;
-  na.kappa = M->kappa;
-  na.diag = M->diag;
+  if constexpr (sizeof(T) == 8) {
+    pa.entry = {M->pts, M->nrm, M->kappa, M->diag};
+  } else {
+    const auto split = [](double v) {
+      const float h = (float)v;
+      return Df{h, (float)(v - (double)h)};
+    };
+    const double f = M->pts_factor, kap = M->kappa / f;  // f: a power of two
+    pa.entry = {M->pts32, M->nrm != nullptr, split(kap * 0.31830988618379067), split(kap), (float)M->diag,
+                (float)(M->nrm ? f * f : f)};
+  }
+  na.entry = pa.entry;
   na.gen = M->gen;
   na.bmax = nullptr;  // set by run_compress in the mixed modes
   na.bmax_off = D->bmax_off;
@@ -732,10 +742,6 @@ void fill_args(dh2_matrix* M, const dh2_compress_params& cp, PairArgs<T>& pa, No
   pa.seg_buf = nullptr;
   pa.seg_cols = 0;
   pa.status = M->status;
-  pa.pts = M->pts;
-  pa.nrm = M->nrm;
-  pa.kappa = M->kappa;
-  pa.diag = M->diag;
   pa.gen = M->gen;
 }
 
@@ -1419,26 +1425,21 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
       if (e) cudaEventDestroy(e);
     if (cs) cudaStreamDestroy(cs);
   } else {
-    if (!any_gen) {
-      // stored G: the admissible blocks in pieces of 32 rows by kNormCols
-      // columns (maxima merged atomically into zeroed buffers, sums per piece,
-      // then the weights), then the nearfield copies.  (The copies on a second
-      // stream beside the leaf work slowed the kernels beside them by more than
-      // their own time: measured, not kept.)
-      for (int i = 0; i < nprob; ++i)
-        if (nas[i].bmax)
-          cudaMemsetAsync(nas[i].bmax, 0, sizeof(float) * (size_t)Ms[i]->tree->tr.dev->bmax_elems, st);
-      launch_norms_adm<T>(d_na, d_pieces, n_pieces, d_norm_adm, d_pbegin, n_norm_adm, d_partial, st);
-      counted(DH2_KC_NORMS, n_pieces > 0);
-      counted(DH2_KC_NORMS, n_norm_adm > 0);
-      const int64_t n_near = n_norm - n_norm_adm;
-      if (n_near > 0 && cp.nearfield == 0) {
-        launch_norms_near<T>(d_na, d_norm_near, (int)n_near, st);
-        counted(DH2_KC_NORMS, true);
-      }
-    } else {
-      launch_norms_near<T>(d_na, d_norm, (int)n_norm, st);
-      counted(DH2_KC_NORMS, n_norm > 0);
+    // the admissible blocks in pieces of 32 rows by kNormCols columns (maxima
+    // merged atomically into zeroed buffers, sums per piece, then the weights),
+    // then the nearfield copies.  (The copies on a second stream beside the
+    // leaf work slowed the kernels beside them by more than their own time:
+    // measured, not kept.)
+    for (int i = 0; i < nprob; ++i)
+      if (nas[i].bmax)
+        cudaMemsetAsync(nas[i].bmax, 0, sizeof(float) * (size_t)Ms[i]->tree->tr.dev->bmax_elems, st);
+    launch_norms_adm<T>(d_na, d_pieces, n_pieces, d_norm_adm, d_pbegin, n_norm_adm, d_partial, any_gen, st);
+    counted(DH2_KC_NORMS, n_pieces > 0);
+    counted(DH2_KC_NORMS, n_norm_adm > 0);
+    const int64_t n_near = n_norm - n_norm_adm;
+    if (n_near > 0 && cp.nearfield == 0) {
+      launch_norms_near<T>(d_na, d_norm_near, (int)n_near, st);
+      counted(DH2_KC_NORMS, true);
     }
     colw_side(kSideRow);
     colw_side(kSideCol);
@@ -1926,7 +1927,7 @@ dh2_status prepare_matrix(const dh2_tree* Tc, const void* G, dh2_dtype dtype, in
   M->diag = diag;
   const size_t es = M->es;
   const int nl = tr.depth + 1;
-  size_t sz[21];
+  size_t sz[22];
   int ns = 0;
   sz[ns++] = align256(es * D->R_elems[0]);
   sz[ns++] = align256(es * D->R_elems[1]);
@@ -1949,6 +1950,7 @@ dh2_status prepare_matrix(const dh2_tree* Tc, const void* G, dh2_dtype dtype, in
   sz[ns++] = align256(es / 2 * (size_t)tr.side[0].nleafcols);
   sz[ns++] = align256(es / 2 * (size_t)tr.side[1].nleafcols);
   sz[ns++] = align256(8 * tr.blocks.size());
+  sz[ns++] = align256(gen && mode_f32(cp.mode) ? (nrm_host ? 64 : 32) * (size_t)tr.n : 0);  // split points
   size_t total = 0;
   for (int i = 0; i < ns; ++i) total += sz[i];
   if (dev_malloc_async(&M->arena, total, M->stream) != cudaSuccess) {
@@ -1966,10 +1968,11 @@ dh2_status prepare_matrix(const dh2_tree* Tc, const void* G, dh2_dtype dtype, in
     return DH2_ENOMEM;
   }
   char* p = (char*)M->arena;
-  void** dst[21] = {&M->R[0], &M->R[1], &M->Q[0], &M->Q[1], &M->X[0], &M->X[1], &M->S, &M->near,
+  void** dst[22] = {&M->R[0], &M->R[1], &M->Q[0], &M->Q[1], &M->X[0], &M->X[1], &M->S, &M->near,
                     (void**)&M->sig[0], (void**)&M->sig[1], (void**)&M->rank[0], (void**)&M->rank[1],
                     (void**)&M->invw, (void**)&M->eps2, (void**)&M->zpow, (void**)&M->status, (void**)&M->acc,
-                    (void**)&M->pts, &M->colw[0], &M->colw[1], (void**)&M->bnorm2};
+                    (void**)&M->pts, &M->colw[0], &M->colw[1], (void**)&M->bnorm2,
+                    (void**)&M->pts32};
   for (int i = 0; i < ns; ++i) {
     *dst[i] = p;
     p += sz[i];
@@ -2003,6 +2006,21 @@ dh2_status prepare_matrix(const dh2_tree* Tc, const void* G, dh2_dtype dtype, in
         if (nrm_host) M->pts_h[n3 + 3 * i + c] = nrm_host[3 * tr.perm[i] + c];
       }
     ce = cudaMemcpyAsync(M->pts, M->pts_h.data(), 8 * M->pts_h.size(), cudaMemcpyHostToDevice, M->stream);
+    if (ce == cudaSuccess && mode_f32(cp.mode)) {
+      double lo[3], hi[3], ext = 0.0;
+      for (int c = 0; c < 3; ++c) lo[c] = hi[c] = M->pts_h[c];
+      for (int64_t i = 0; i < tr.n; ++i)
+        for (int c = 0; c < 3; ++c) {
+          lo[c] = std::min(lo[c], M->pts_h[3 * i + c]);
+          hi[c] = std::max(hi[c], M->pts_h[3 * i + c]);
+        }
+      for (int c = 0; c < 3; ++c) ext = std::max(ext, hi[c] - lo[c]);
+      int e = 0;
+      if (ext > 0.0 && std::isfinite(ext)) std::frexp(ext, &e);
+      M->pts_factor = std::ldexp(1.0, -e);
+      const auto mid = [&](int c) { return lo[c] + 0.5 * (hi[c] - lo[c]); };
+      launch_split_points(M->pts, M->nrm, tr.n, make_double3(mid(0), mid(1), mid(2)), M->pts_factor, M->pts32, M->stream);
+    }
   }
   if (ce != cudaSuccess) {
     cudaGetLastError();

@@ -29,6 +29,147 @@ __host__ __device__ constexpr int factor_class(int P_T) {
   return P_T <= 32 ? 0 : P_T <= 40 ? 1 : P_T <= 48 ? 2 : P_T <= 64 ? 3 : 4;
 }
 
+// ---------------------------------------------------------------- generated entries
+// Entry G_ij generated from the points, with `diag` on the diagonal:
+//  - without normals: the Helmholtz single layer of Eq. (helmholtz),
+//    exp(i kappa r) / (4 pi r), r = |x_i - x_j|;
+//  - otherwise the double layer of Section 7 ("DLP matrix"),
+//    (1 - i kappa r) exp(i kappa r) / (4 pi r^3) <x_i - x_j, n(x_j)>.
+template <typename T>
+struct Gen;
+
+// FP64: points and unit normals (NULL: single layer), 3 doubles each.
+template <>
+struct Gen<double> {
+  const double* pts;
+  const double* nrm;
+  double kappa, diag;
+};
+__device__ __forceinline__ C2<double> gen_entry(const Gen<double>& g, int64_t i, int64_t j) {
+  if (i == j) return C2<double>{g.diag, 0.0};
+  const double dx = g.pts[3 * i] - g.pts[3 * j];
+  const double dy = g.pts[3 * i + 1] - g.pts[3 * j + 1];
+  const double dz = g.pts[3 * i + 2] - g.pts[3 * j + 2];
+  const double r = sqrt(dx * dx + dy * dy + dz * dz);
+  // single layer: scale 1/(4 pi r); double layer: <x_i - x_j, n_j>/(4 pi r^3)
+  // times (1 - i kappa r)
+  double scale;
+  double kr = 0.0;
+  if (g.nrm) {
+    const double dn = dx * g.nrm[3 * j] + dy * g.nrm[3 * j + 1] + dz * g.nrm[3 * j + 2];
+    scale = dn / (12.566370614359172 * r * r * r);
+    kr = g.kappa * r;
+  } else {
+    scale = 1.0 / (12.566370614359172 * r);
+  }
+  double sn, cs;
+  sincos(g.kappa * r, &sn, &cs);
+  // (cs + i sn)(1 - i kr) = cs + kr sn + i (sn - kr cs)
+  return C2<double>{(cs + kr * sn) * scale, (sn - kr * cs) * scale};
+}
+
+// A value hi + lo of two floats (|lo| <= ulp(hi)/2, about 48 significant
+// bits), with the error-free sum of Knuth and the error-free product from a
+// fused multiply-add (Dekker's double-length arithmetic in FP32 registers).
+struct Df {
+  float hi, lo;
+};
+__device__ __forceinline__ Df df_fast_sum(float s, float e) {  // |s| >= |e|
+  const float h = __fadd_rn(s, e);
+  return Df{h, __fsub_rn(e, __fsub_rn(h, s))};
+}
+__device__ __forceinline__ Df df_add(Df x, Df y) {
+  const float s = __fadd_rn(x.hi, y.hi);
+  const float bb = __fsub_rn(s, x.hi);
+  const float e = (__fsub_rn(x.hi, __fsub_rn(s, bb)) + __fsub_rn(y.hi, bb)) + x.lo + y.lo;
+  return df_fast_sum(s, e);
+}
+__device__ __forceinline__ Df df_neg(Df x) { return Df{-x.hi, -x.lo}; }
+__device__ __forceinline__ Df df_mul(Df x, Df y) {
+  const float p = __fmul_rn(x.hi, y.hi);
+  float e = fmaf(x.hi, y.hi, -p);
+  e = fmaf(x.hi, y.lo, e);
+  e = fmaf(x.lo, y.hi, e);
+  return df_fast_sum(p, e);
+}
+// unnormalised forms: a leading float and the sum of the errors behind it
+struct Df2 {
+  float p, e;
+};
+__device__ __forceinline__ Df2 two_sum(float x, float y) {
+  const float s = __fadd_rn(x, y), bb = __fsub_rn(s, x);
+  return Df2{s, __fadd_rn(__fsub_rn(x, __fsub_rn(s, bb)), __fsub_rn(y, bb))};
+}
+__device__ __forceinline__ Df2 df_sq(Df x) {
+  const float p = __fmul_rn(x.hi, x.hi);
+  return Df2{p, fmaf(2.f * x.hi, x.lo, fmaf(x.hi, x.hi, -p))};
+}
+__device__ __forceinline__ Df2 df_prod(Df x, Df y) {
+  const float p = __fmul_rn(x.hi, y.hi);
+  return Df2{p, fmaf(x.lo, y.hi, fmaf(x.hi, y.lo, fmaf(x.hi, y.hi, -p)))};
+}
+__device__ __forceinline__ Df df_diff(float xh, float xl, float yh, float yl) {
+  const Df2 s = two_sum(xh, -yh);
+  return df_fast_sum(s.p, s.e + __fsub_rn(xl, yl));
+}
+__device__ __forceinline__ Df df_split(double v) {
+  const float h = (float)v;
+  return Df{h, (float)(v - (double)h)};
+}
+
+// FP32: coordinates, relative to the middle of their bounding box and to a power
+// of two above its extent, (and normals) split into two floats each, per point
+// two (with normals four) float4: hi parts, lo parts.  Differences, r, the phase
+// and its reduction are formed in double-float, sin and cos of the reduced
+// phase in FP32: an entry's error is that of its FP32 roundings, as with FP64
+// differences and phase, which GB300's narrow FP64 pipe (about 2 lanes per SM
+// against 128) had made most of the matrix-free mode's time.  n = 16384 cube,
+// before -> after: norms and nearfield 14.9 -> 1.7 ms, leaf R 4.7 -> 0.9 ms, leaf
+// factors 11.5 -> 7.8 ms.  Bound by instruction issue (~120 per entry).
+template <>
+struct Gen<float> {
+  const float4* pts;
+  int dlp;       // with normals
+  Df ppi, kap;   // kappa / pi, kappa, for the scaled points
+  float diag;
+  float scale;   // of the entries: the points' factor (double layer: its square)
+};
+__device__ __forceinline__ C2<float> gen_entry(const Gen<float>& g, int64_t i, int64_t j) {
+  if (i == j) return C2<float>{g.diag, 0.f};
+  const int st = g.dlp ? 4 : 2;
+  const float4 *pi = g.pts + i * st, *pj = g.pts + j * st;
+  const float4 xh = __ldg(pi), xl = __ldg(pi + 1), yh = __ldg(pj), yl = __ldg(pj + 1);
+  const Df dx = df_diff(xh.x, xl.x, yh.x, yl.x);
+  const Df dy = df_diff(xh.y, xl.y, yh.y, yl.y);
+  const Df dz = df_diff(xh.z, xl.z, yh.z, yl.z);
+  // |x_i - x_j|^2: the products' and the sums' errors gathered in one float
+  const Df2 sx = df_sq(dx), sy = df_sq(dy), sz = df_sq(dz);
+  const Df2 s1 = two_sum(sx.p, sy.p), s2 = two_sum(s1.p, sz.p);
+  const Df d2 = df_fast_sum(s2.p, ((sx.e + sy.e) + sz.e) + (s1.e + s2.e));
+  // r = sqrt(d2): one Newton step from the FP32 square root
+  const float ir = rsqrtf(d2.hi), r0 = __fmul_rn(d2.hi, ir);
+  const float rest = fmaf(-r0, r0, d2.hi) + d2.lo;
+  const Df r = df_fast_sum(r0, 0.5f * ir * rest);
+  // phase / pi, reduced to [-1, 1]: the integer part leaves the leading float exactly
+  const Df2 ph = df_prod(r, g.ppi);
+  const float th = __fsub_rn(ph.p, 2.f * rintf(0.5f * ph.p)) + ph.e;
+  float sn, cs;
+  sincospif(th, &sn, &cs);
+  const Df2 q4 = df_prod(r, Df{12.566371f, -8.742278e-7f});  // 4 pi r
+  if (!g.dlp) {  // 1 / (4 pi r), the quotient corrected by its remainder
+    const float s0 = ir * 0.07957747f;
+    const float sc = fmaf(s0, fmaf(-s0, q4.p, 1.f) - s0 * q4.e, s0) * g.scale;
+    return C2<float>{cs * sc, sn * sc};
+  }
+  const float4 nh = __ldg(pj + 2), nl = __ldg(pj + 3);
+  const Df dn = df_add(df_add(df_mul(dx, Df{nh.x, nl.x}), df_mul(dy, Df{nh.y, nl.y})), df_mul(dz, Df{nh.z, nl.z}));
+  const Df q = df_mul(df_fast_sum(q4.p, q4.e), d2);
+  const float iq = __frcp_rn(q.hi), s0 = dn.hi * iq;
+  const float sc = fmaf((fmaf(-s0, q.hi, dn.hi) + dn.lo) - s0 * q.lo, iq, s0) * g.scale;
+  const Df kr = df_mul(r, g.kap);
+  return C2<float>{fmaf(kr.hi, sn, cs) * sc, fmaf(-kr.hi, cs, sn) * sc};
+}
+
 template <typename T>
 struct PairArgs {
   const int32_t* start[2];            // first row index of the pair's cluster
@@ -66,56 +207,9 @@ struct PairArgs {
   C2<T>* seg_buf;
   int32_t seg_cols;
   uint32_t* status;
-  // matrix-free mode: entries generated from points (permuted order, 3 doubles
-  // each) and, for the double layer, their normals (NULL for the single layer)
-  const double* pts;
-  const double* nrm;
-  double kappa;
-  double diag;
+  Gen<T> entry;  // matrix-free mode (gen != 0): entries generated from points
   int32_t gen;
 };
-
-// Entry G_ij generated from the points, with `diag` on the diagonal:
-//  - nrm == NULL: the Helmholtz single layer of Eq. (helmholtz),
-//    exp(i kappa r) / (4 pi r), r = |x_i - x_j|;
-//  - otherwise the double layer of Section 7 ("DLP matrix"),
-//    (1 - i kappa r) exp(i kappa r) / (4 pi r^3) <x_i - x_j, n(x_j)>, with
-//    nrm the unit normals (3 doubles per point, same order as pts).
-// Distances, <x_i - x_j, n_j> and the phase reduction are formed in FP64; the
-// FP32 variant evaluates sin/cos of the reduced phase (|phase| <= pi) in FP32.
-template <typename T>
-__device__ __forceinline__ C2<T> kernel_entry(const double* pts, const double* nrm, int64_t i, int64_t j,
-                                              double kappa, double diag) {
-  if (i == j) return C2<T>{(T)diag, T(0)};
-  const double dx = pts[3 * i] - pts[3 * j];
-  const double dy = pts[3 * i + 1] - pts[3 * j + 1];
-  const double dz = pts[3 * i + 2] - pts[3 * j + 2];
-  const double r = sqrt(dx * dx + dy * dy + dz * dz);
-  // single layer: scale 1/(4 pi r); double layer: <x_i - x_j, n_j>/(4 pi r^3)
-  // times (1 - i kappa r)
-  double scale;
-  double kr = 0.0;
-  if (nrm) {
-    const double dn = dx * nrm[3 * j] + dy * nrm[3 * j + 1] + dz * nrm[3 * j + 2];
-    scale = dn / (12.566370614359172 * r * r * r);
-    kr = kappa * r;
-  } else {
-    scale = 1.0 / (12.566370614359172 * r);
-  }
-  if (sizeof(T) == 8) {
-    double sn, cs;
-    sincos(kappa * r, &sn, &cs);
-    // (cs + i sn)(1 - i kr) = cs + kr sn + i (sn - kr cs)
-    return C2<T>{(T)((cs + kr * sn) * scale), (T)((sn - kr * cs) * scale)};
-  } else {
-    double th = kappa * r * 0.31830988618379067;  // phase / pi
-    th -= 2.0 * rint(0.5 * th);                    // reduced to [-1, 1]
-    float sn, cs;
-    sincospif((float)th, &sn, &cs);
-    const float krf = (float)kr, sc = (float)scale;
-    return C2<T>{(T)((cs + krf * sn) * sc), (T)((sn - krf * cs) * sc)};
-  }
-}
 
 // One CTA per launch code: args_dev holds one PairArgs per problem (device
 // memory); P is the row capacity of the shared-memory factor (even).  With

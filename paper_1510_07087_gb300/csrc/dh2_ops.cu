@@ -1,6 +1,8 @@
 // Kernels around the per-pair factorisation: block norms and nearfield copy,
 // basis expansion by Eq. (nested), the projection S_b and the error measures
 // (the matrix-vector products are in dh2_mv.cu).
+#include <type_traits>
+
 #include "dh2_check.cuh"
 #include "dh2_internal.h"
 #include "dh2_ops.cuh"
@@ -103,24 +105,19 @@ __global__ void __launch_bounds__(256) norms_near_kernel(const NormsArgs<T>* __r
   const int mt = a.csize[t], ms = a.csize[s];
   const int64_t t0 = a.cstart[t], s0 = a.cstart[s];
   if (a.gen) {
-    // matrix-free: generate the block's entries from the points
-    if (a.badm[b]) {
-      double acc = 0.0;
-      for (int64_t e = lane; e < (int64_t)mt * ms; e += 32) {
-        const int r = (int)(e % mt), j = (int)(e / mt);
-        const C2<T> g = kernel_entry<T>(a.pts, a.nrm, t0 + r, s0 + j, a.kappa, a.diag);
-        acc += (double)g.re * g.re + (double)g.im * g.im;
-      }
-      const double tot = warp_sum(acc);
-      if (lane == 0 && DH2_IN(b, c_lim.nblocks, 23, b))
-        a.invw[b] = tot > 0.0 ? 1.0 / (sqrt(tot) * a.zpow[a.clevel[t]]) : 1.0;
-    if (lane == 0 && a.bnorm2) a.bnorm2[b] = tot;
-    } else if (a.copy) {
+    // matrix-free (nearfield blocks only; the admissible ones: norms_gen_kernel)
+    if (!a.badm[b] && a.copy) {
       C2<T>* out = a.near + a.near_off[b];
+      int r = lane % mt, j = lane / mt;
+      const int dr = 32 % mt, dj = 32 / mt;
       for (int64_t e = lane; e < (int64_t)mt * ms; e += 32) {
-        const int r = (int)(e % mt), j = (int)(e / mt);
-        if (DH2_IN(a.near_off[b] + e, c_lim.near, 21, b))
-          out[e] = kernel_entry<T>(a.pts, a.nrm, t0 + r, s0 + j, a.kappa, a.diag);
+        if (DH2_IN(a.near_off[b] + e, c_lim.near, 21, b)) out[e] = gen_entry(a.entry, t0 + r, s0 + j);
+        r += dr;
+        j += dj;
+        if (r >= mt) {
+          r -= mt;
+          ++j;
+        }
       }
     }
     return;
@@ -394,7 +391,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? DH2_PROJ_MINB : 1) proje
 template <typename T, typename RT>
 __device__ __forceinline__ C2<double> ref_entry(const ErrArgs<T>& a, const C2<RT>* Gref, int64_t ldr, int64_t i,
                                                 int64_t j) {
-  if (a.ref_gen) return kernel_entry<double>(a.pts, a.nrm, i, j, a.kappa, a.diag);
+  if (a.ref_gen) return gen_entry(Gen<double>{a.pts, a.nrm, a.kappa, a.diag}, i, j);
   const C2<RT> g = Gref[i + j * ldr];
   return C2<double>{(double)g.re, (double)g.im};
 }
@@ -472,7 +469,7 @@ __global__ void __launch_bounds__(256) error_kernel(ErrArgs<T> a, const C2<RT>* 
 template <typename RT>
 __device__ __forceinline__ C2<double> gref(const C2<RT>* G, int64_t ld, const ErrArgs<float>& g, int64_t i,
                                            int64_t j) {
-  if (!G) return kernel_entry<double>(g.pts, g.nrm, i, j, g.kappa, g.diag);
+  if (!G) return gen_entry(Gen<double>{g.pts, g.nrm, g.kappa, g.diag}, i, j);
   const C2<RT> v = G[i + j * ld];
   return C2<double>{(double)v.re, (double)v.im};
 }
@@ -640,6 +637,57 @@ __global__ void __launch_bounds__(256) norms_adm_kernel(const NormsArgs<T>* __re
   if (lane == 0) partial[w] = tot;
 }
 
+// The admissible blocks' pass of the matrix-free mode, by the same pieces: the
+// entries are generated and their squares added, in FP64 (double) or
+// double-float (float: the FP64 pipe would take longer than the entries do).
+// One warp per block had left the few coarse blocks of millions of entries to
+// one warp each.
+__device__ __forceinline__ void sq_acc(double& s, C2<double> g) { s += g.re * g.re + g.im * g.im; }
+__device__ __forceinline__ void sq_acc(Df& s, C2<float> g) {  // lo: the errors so far
+  const Df2 a = df_sq(Df{g.re, 0.f}), b = df_sq(Df{g.im, 0.f});
+  const Df2 t = two_sum(s.hi, a.p), u = two_sum(t.p, b.p);
+  s = Df{u.p, s.lo + ((a.e + b.e) + (t.e + u.e))};
+}
+__device__ __forceinline__ double sq_value(double s) { return s; }
+__device__ __forceinline__ double sq_value(Df s) { return (double)s.hi + (double)s.lo; }
+template <typename T>
+__global__ void __launch_bounds__(256) norms_gen_kernel(const NormsArgs<T>* __restrict__ args,
+                                                        const uint64_t* __restrict__ pieces, int64_t n,
+                                                        double* __restrict__ partial) {
+  const int64_t w = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (w >= n) return;
+  const uint64_t pc = pieces[w];
+  const uint32_t code = (uint32_t)(pc >> 32);
+  const int slab = (int)((pc >> 16) & 0xFFFFu), grp = (int)(pc & 0xFFFFu);
+  const NormsArgs<T>& a = args[code >> 26];
+  const int b = (int)(code & ((1u << 26) - 1u));
+  const int t = a.bt[b], s = a.bs[b];
+  const int64_t t0 = a.cstart[t], s0 = a.cstart[s];
+  const int r = slab * 32 + lane;
+  const int c0 = grp * kNormCols, c1 = min(a.csize[s], c0 + kNormCols);
+  typename std::conditional<sizeof(T) == 8, double, Df>::type acc{};
+  if (r < a.csize[t])
+    for (int j = c0; j < c1; ++j) sq_acc(acc, gen_entry(a.entry, t0 + r, s0 + j));
+  const double tot = warp_sum(sq_value(acc));
+  if (lane == 0) partial[w] = tot;
+}
+
+// coordinates (and normals) of the matrix-free mode split for Gen<float>
+__global__ void split_points_kernel(const double* __restrict__ pts, const double* __restrict__ nrm, int64_t n,
+                                    double3 mid, double factor, float4* __restrict__ out) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  auto put = [&](double vx, double vy, double vz, float4* o) {
+    const Df x = df_split(vx), y = df_split(vy), z = df_split(vz);
+    o[0] = make_float4(x.hi, y.hi, z.hi, 0.f);
+    o[1] = make_float4(x.lo, y.lo, z.lo, 0.f);
+  };
+  float4* o = out + i * (nrm ? 4 : 2);
+  put((pts[3 * i] - mid.x) * factor, (pts[3 * i + 1] - mid.y) * factor, (pts[3 * i + 2] - mid.z) * factor, o);
+  if (nrm) put(nrm[3 * i], nrm[3 * i + 1], nrm[3 * i + 2], o + 2);
+}
+
 // the admissible blocks' |G_b|_F^2 (their pieces pbegin[i] .. pbegin[i+1] - 1
 // added in order) and weights 1/omega_b
 template <typename T>
@@ -748,10 +796,17 @@ void launch_to_type(const C2<double>* v, C2<T>* o, int64_t n, cudaStream_t st) {
 }
 template <typename T>
 void launch_norms_adm(const NormsArgs<T>* args_dev, const uint64_t* pieces, int64_t npieces, const uint32_t* codes,
-                      const int64_t* pbegin, int64_t nblocks, double* partial, cudaStream_t st) {
-  if (npieces > 0) norms_adm_kernel<T><<<(int)((npieces + 7) / 8), 256, 0, st>>>(args_dev, pieces, npieces, partial);
+                      const int64_t* pbegin, int64_t nblocks, double* partial, bool gen, cudaStream_t st) {
+  const int grid = (int)((npieces + 7) / 8);
+  if (npieces > 0 && gen) norms_gen_kernel<T><<<grid, 256, 0, st>>>(args_dev, pieces, npieces, partial);
+  else if (npieces > 0) norms_adm_kernel<T><<<grid, 256, 0, st>>>(args_dev, pieces, npieces, partial);
   if (nblocks > 0)
     norms_finish_kernel<T><<<(int)((nblocks + 255) / 256), 256, 0, st>>>(args_dev, codes, pbegin, partial, nblocks);
+}
+
+void launch_split_points(const double* pts, const double* nrm, int64_t n, double3 mid, double factor, float4* out,
+                         cudaStream_t st) {
+  if (n > 0) split_points_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(pts, nrm, n, mid, factor, out);
 }
 
 void launch_norm2(const C2<double>* v, int64_t n, double* acc, cudaStream_t st) {
@@ -819,7 +874,7 @@ void launch_colw(const int32_t* gblk, const double* invw, T* colw, int64_t n, cu
   template void launch_closed_form<T>(const ErrArgs<T>&, const double*, int, double*, cudaStream_t);            \
   template void launch_to_type<T>(const C2<double>*, C2<T>*, int64_t, cudaStream_t);                       \
   template void launch_norms_adm<T>(const NormsArgs<T>*, const uint64_t*, int64_t, const uint32_t*, const int64_t*, \
-                                    int64_t, double*, cudaStream_t);                                           \
+                                    int64_t, double*, bool, cudaStream_t);                                           \
   template void launch_sub<T>(C2<double>*, const C2<T>*, int64_t, cudaStream_t);
 
 DH2_INST(float)

@@ -40,10 +40,7 @@ struct NormsArgs {
   C2<T>* near;
   const int64_t* near_off;
   int copy;
-  const double* pts;  // matrix-free mode
-  const double* nrm;  // matrix-free double layer: normals (NULL: single layer)
-  double kappa;
-  double diag;
+  Gen<T> entry;  // matrix-free mode
   int gen;
   // mixed modes: per admissible block the largest |re|, |im| of each of its
   // rows, then of each of its columns (bmax + bmax_off[b]); NULL otherwise
@@ -172,14 +169,14 @@ void launch_colw(const int32_t* gblk, const double* invw, T* colw, int64_t n, cu
 // codes: (problem << 26) | block for a batch, or NULL for blocks 0..n-1 of args_dev[0]
 template <typename T>
 void launch_norms_near(const NormsArgs<T>* args_dev, const uint32_t* codes, int n, cudaStream_t st);
-// admissible blocks of a stored G in pieces (code << 32 | 32-row slab << 16 |
+// admissible blocks of a stored G (gen: generated entries) in pieces (code << 32 | 32-row slab << 16 |
 // kNormCols-column group; block i's pieces are pbegin[i] .. pbegin[i+1] - 1):
 // partial sums per piece (scratch `partial`, npieces doubles), in the mixed modes
 // the row/column maxima (zeroed before) merged atomically, then bnorm2 and the
 // weights of the nblocks codes
 template <typename T>
 void launch_norms_adm(const NormsArgs<T>* args_dev, const uint64_t* pieces, int64_t npieces, const uint32_t* codes,
-                      const int64_t* pbegin, int64_t nblocks, double* partial, cudaStream_t st);
+                      const int64_t* pbegin, int64_t nblocks, double* partial, bool gen, cudaStream_t st);
 struct OwnItem;
 // the nearfield lists of one side, and its own-block records from the block
 // ids, coupling offsets and the blocks' pairs of the other side
@@ -216,6 +213,9 @@ template <typename T>
 void launch_closed_form(const ErrArgs<T>& a, const double* bnorm2, int nblocks, double* acc, cudaStream_t st);
 // o = (T) v; u -= t  (vectors of n complex entries)
 template <typename T> void launch_to_type(const C2<double>* v, C2<T>* o, int64_t n, cudaStream_t st);
+// points (and normals, or NULL) in FP64 as the split coordinates of Gen<float>: (point - mid) * factor
+void launch_split_points(const double* pts, const double* nrm, int64_t n, double3 mid, double factor, float4* out,
+                         cudaStream_t st);
 // *acc += |v|^2; v = w / sqrt(*n2) (device scalar; v may be w); a seeded vector with entries in [-1/2, 1/2)^2
 void launch_norm2(const C2<double>* v, int64_t n, double* acc, cudaStream_t st);
 void launch_normalize(C2<double>* v, const C2<double>* w, int64_t n, const double* n2, cudaStream_t st);

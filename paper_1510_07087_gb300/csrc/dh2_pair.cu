@@ -190,9 +190,7 @@ struct Source {
   const int32_t* gcol;
   const T* colw;
   int64_t cmo;
-  const double* pts;  // matrix-free mode
-  const double* nrm;  // double layer: normals (NULL: single layer)
-  double kappa, diag;
+  Gen<T> entry;  // matrix-free mode
   int gen;
   // non-leaf
   const C2<T>* R0;
@@ -230,8 +228,7 @@ struct Source {
   // leaf: element (r, j) given column j's global index gc and weight w
   __device__ __forceinline__ C2<T> leaf_at(int r, int gc, T w) const {
     if (gen) {
-      C2<T> g = side == 0 ? kernel_entry<T>(pts, nrm, r0 + r, gc, kappa, diag)
-                          : kernel_entry<T>(pts, nrm, gc, r0 + r, kappa, diag);
+      const C2<T> g = side == 0 ? gen_entry(entry, r0 + r, gc) : gen_entry(entry, gc, r0 + r);
       return C2<T>{g.re * w, side == 0 ? g.im * w : -g.im * w};
     }
     if (side == 0) {
@@ -312,31 +309,7 @@ __device__ __forceinline__ void stage_cols(const Source<T, FROM_R>& src, int p, 
   }
 }
 
-// ---------------------------------------------------------------- double-float arithmetic
-// A value hi + lo of two floats (|lo| <= ulp(hi)/2, about 48 significant
-// bits), with the error-free sum of Knuth and the error-free product from a
-// fused multiply-add (Dekker's double-length arithmetic in FP32 registers).
-struct Df {
-  float hi, lo;
-};
-__device__ __forceinline__ Df df_fast_sum(float s, float e) {  // |s| >= |e|
-  const float h = s + e;
-  return Df{h, e - (h - s)};
-}
-__device__ __forceinline__ Df df_add(Df x, Df y) {
-  const float s = x.hi + y.hi;
-  const float bb = s - x.hi;
-  const float e = (x.hi - (s - bb)) + (y.hi - bb) + x.lo + y.lo;
-  return df_fast_sum(s, e);
-}
-__device__ __forceinline__ Df df_neg(Df x) { return Df{-x.hi, -x.lo}; }
-__device__ __forceinline__ Df df_mul(Df x, Df y) {
-  const float p = x.hi * y.hi;
-  float e = fmaf(x.hi, y.hi, -p);
-  e = fmaf(x.hi, y.lo, e);
-  e = fmaf(x.lo, y.hi, e);
-  return df_fast_sum(p, e);
-}
+// ---------------------------------------------------------------- double-float arithmetic (Df: dh2_kernels.cuh)
 // one Newton step from the FP32 square root / reciprocal
 __device__ __forceinline__ Df df_sqrt(Df x) {
   const float r = sqrtf(x.hi);
@@ -873,10 +846,7 @@ __global__ void __launch_bounds__(NT, (GRAM ? gram_min_blocks<NT>() : pair_min_b
     src.colw = a.colw[side] + src.cmo;
     src.G = a.G;
     src.ld = a.ld;
-    src.pts = a.pts;
-    src.nrm = a.nrm;
-    src.kappa = a.kappa;
-    src.diag = a.diag;
+    src.entry = a.entry;
     src.gen = a.gen;
   }
   // column segments of a wide non-leaf pair (Section 6's Ghat_tc = [L_1 Q_1,
@@ -1467,10 +1437,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 6 : 2)
     src.colw = a.colw[side] + src.cmo;
     src.G = a.G;
     src.ld = a.ld;
-    src.pts = a.pts;
-    src.nrm = a.nrm;
-    src.kappa = a.kappa;
-    src.diag = a.diag;
+    src.entry = a.entry;
     src.gen = a.gen;
   }
   if (p <= 0 || p > P) return;  // reported by pair_kernel

@@ -137,3 +137,47 @@ def test_matrix_free_rejects_view_nearfield():
     st = B._lib().dh2_compress_kernel(T.handle, B._ptr(np.ascontiguousarray(pts)), 4.0, 1.0, B.byref(p),
                                       B.c_void_p(torch.cuda.current_stream().cuda_stream), B.byref(h))
     assert st == 1 and not h.value
+
+
+@pytest.mark.parametrize("scale,offset,kappa", [(1.0, 0.0, 3.0), (1.0, 0.0, 400.0), (2.0 ** -20, 0.0, 5.0e6),
+                                                (1.0e3, 40.0, 0.5), (1.0, 37.25, 60.0)])
+@pytest.mark.parametrize("dlp", [False, True])
+def test_generated_fp32_entries(scale, offset, kappa, dlp):
+    """Entries generated in the FP32 mode, read off by products with unit vectors (one cluster: nearfield
+    only, every product exact), against FP64 from the same points.  An entry carries the rounding of the
+    reduced phase (pi 2^-25), of sin and cos (2 ulp) and of three FP32 operations: below 5e-7 of its size
+    (double layer: of (1 + kappa r) times its scale).  Point pairs down to 1e-5 of the extent, scaled and
+    shifted point sets."""
+    D = _dev()
+    n = 90
+    rng = np.random.default_rng(8)
+    pts = rng.standard_normal((n, 3))
+    pts[40:] = pts[:50] + 10.0 ** rng.uniform(-5, -1, (50, 1)) * rng.standard_normal((50, 3))
+    pts = pts * scale + offset
+    nrm = rng.standard_normal((n, 3))
+    nrm /= np.linalg.norm(nrm, axis=1, keepdims=True)
+    T = D.dh2_tree_build(pts, 100, 0.0)
+    perm = T.perm()
+    if dlp:
+        M = D.dh2_compress_kernel_dlp(T, pts, nrm, kappa, mode=D.MODE_FP32)
+    else:
+        M = D.dh2_compress_kernel(T, pts, kappa, 0.25, mode=D.MODE_FP32)
+    got = _matvec(D, M, np.eye(n), torch.complex64)
+    p, q = pts[perm], nrm[perm]
+    d = p[:, None, :] - p[None, :, :]
+    r = np.sqrt((d * d).sum(-1))
+    np.fill_diagonal(r, 1.0)
+    s = 1.0 / (4.0 * math.pi * r)
+    if dlp:
+        s = s * (d * q[None, :, :]).sum(-1) / r ** 2
+        ref = s * (1.0 - 1j * kappa * r) * np.exp(1j * kappa * r)
+        size = np.abs(s) * (1.0 + kappa * r)
+    else:
+        ref = s * np.exp(1j * kappa * r)
+        size = s
+    np.fill_diagonal(ref, 0.5 if dlp else 0.25)
+    np.fill_diagonal(size, 1.0)
+    # the FP64 reference's own phase and direction errors: kappa r 2^-52, and 2^-52 of the coordinates
+    fp64 = np.abs(kappa * r) * 4e-16 + 1e-15 * np.abs(p).max() * (kappa + 10.0 / r)
+    bound = 5e-7 * size + fp64 * (size + (1.0 + kappa * r) / (4.0 * math.pi * r * r) if dlp else size)
+    assert np.all(np.abs(got - ref) <= bound), np.max(np.abs(got - ref) / bound)
