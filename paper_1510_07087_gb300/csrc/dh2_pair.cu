@@ -121,13 +121,29 @@ struct Eps<double> {
   static constexpr double tiny = 1e-280;
 };
 
-// Reciprocal square root and quotient for the rotation and reflector scalars:
+// Reciprocal square root and reciprocal for the rotation and reflector scalars:
 // hardware approximations in FP32 (a few ulp; the rotations and reflections
-// stay unitary to that level), correctly rounded in FP64.
+// stay unitary to that level).  In FP64 the hardware's approximation (better
+// than 2^-18) and one third-order (Halley) step from h = 1 - x y0^2 or 1 - x y0:
+// within 2 ulp in 5 and 3 operations of the narrow FP64 pipe; arguments are
+// normal and finite (squared norms above Eps::tiny), or give NaN.
 __device__ __forceinline__ float frsqrt(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double frsqrt(double x) { return rsqrt(x); }
-__device__ __forceinline__ float fdiv(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ double fdiv(double a, double b) { return a / b; }
+__device__ __forceinline__ double rsqrt_from(double x, double y0) {
+  const double h = fma(-x * y0, y0, 1.0);
+  return fma(y0 * h, fma(0.375, h, 0.5), y0);
+}
+__device__ __forceinline__ double frsqrt(double x) {
+  double y0;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
+  return rsqrt_from(x, y0);
+}
+__device__ __forceinline__ float frcp(float x) { return __fdividef(1.f, x); }
+__device__ __forceinline__ double frcp(double x) {
+  double y0;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
+  const double h = fma(-x, y0, 1.0);
+  return fma(y0, fma(h, h, h), y0);
+}
 
 // Asynchronous global -> shared copies (cp.async): not held up by CTA
 // barriers; completed by cp_async_wait_all in the issuing thread.
@@ -529,26 +545,114 @@ __device__ void gram_cholesky(const PairArgs<T>& a, int side, int pid, int p, in
 #ifndef DH2_LQT
 #define DH2_LQT 8  // threads per row in the streamed LQ (4 or 8)
 #endif
-// Steps 2-4 of a pair (Jacobi on the K leading columns of L in shared memory,
-// the rank from the tail sums, Q), shared by pair_kernel and
-// gram_jacobi_kernel.
-template <typename T, int P_T, int NT>
-__device__ __forceinline__ void jacobi_rank_q(const PairArgs<T>& a, int side, int pid, int p, int LDL, int K,
-                                              double E_K, int kcap, int lvl, C2<T>* Lm, double* sig2, int* ord,
-                                              int32_t* rank_out, double* sig_out, long long t_b) {
+// ---------------------------------------------------------------- 2. Jacobi
+// Scalars of the rotation that makes two columns with squared norms al, be and
+// product ga = a^* b orthogonal: a' = c a - s e b, b' = s a + c e b, c^2 + s^2 =
+// |e|^2 = 1, and tg = t |gamma| (the norms become al - tg, be + tg).  False
+// where the pair is orthogonal to tol (relative); `off` is the pair's ratio
+// |gamma| / sqrt(alpha beta), in FP64 only whether it exceeds sqrt(tol) / 4 (1
+// or 0).
+template <typename T>
+struct Rot {
+  T c, s, tg;
+  C2<T> e;
+};
+// WIDE: |gamma| formed without squaring gamma, whose square leaves FP32's range
+// for columns 1e-10 below the largest one (the FP64 preconditioner; |e| must be
+// 1 to FP32 rounding for every pair it turns).
+template <bool WIDE = false>
+__device__ __forceinline__ bool rot_scalars(float al, float be, C2<float> ga, float tol, Rot<float>& r, float& off) {
+  float g, rg;
+  if constexpr (WIDE) {
+    const float m = fmaxf(fabsf(ga.re), fabsf(ga.im)), n = fminf(fabsf(ga.re), fabsf(ga.im));
+    if (!(m > 1e-35f)) return false;
+    const float rm = __frcp_rn(m), q = fmaf(n * rm, n * rm, 1.f), h = rsqrtf(q);
+    g = m * (q * h);
+    rg = rm * h;
+  } else {
+    const float g2 = cnorm2(ga);
+    if (!(g2 > 0.f)) return false;
+    rg = frsqrt(g2);
+    g = g2 * rg;
+  }
+  // rotation scalars from reciprocal square roots and one quotient
+  // (hardware approximations, a few ulp): c^2 + s^2 = 1 to that level, far
+  // inside the convergence test's tol = p u
+  off = g * frsqrt(al) * frsqrt(be);
+  if (!(al > Eps<float>::tiny && be > Eps<float>::tiny && off > tol)) return false;
+  const float zt = (be - al) * 0.5f * rg;
+  const float az = fabsf(zt);
+  const float q1 = 1.f + zt * zt;
+  const float t = copysignf(az > 1e15f ? __fdividef(0.5f, az) : __fdividef(1.f, az + q1 * frsqrt(q1)), zt);
+  r.c = frsqrt(1.f + t * t);
+  r.s = t * r.c;
+  r.tg = t * g;
+  r.e = C2<float>{ga.re * rg, -ga.im * rg};  // e^{-i arg gamma}
+  return r.s != 0.f;
+}
+// FP64: the angle needs FP32 accuracy only (what it leaves of gamma, 1e-7, is
+// rotated away in the next sweep); c, s and e are normalised in FP64 from FP32
+// approximations.  About 35 operations of the narrow FP64 pipe instead of 110
+// with double square roots and quotients.
+template <bool WIDE = false>
+__device__ __forceinline__ bool rot_scalars(double al, double be, C2<double> ga, double tol, Rot<double>& r,
+                                            float& off) {
+  off = 0.f;
+  if (!(al > Eps<double>::tiny && be > Eps<double>::tiny)) return false;
+  // scaled by the power of two that brings the larger norm to [1, 2)
+  const int ha = __double2hiint(al), hb = __double2hiint(be);
+  const int ex = max(ha, hb) >> 20;
+  if (ex <= 0 || ex >= 2046) return false;  // overflow: reported with the norms
+  const double sc = __hiloint2double((2046 - ex) << 20, 0), back = __hiloint2double(ex << 20, 0);
+  const double as = al * sc, bs = be * sc, gr = ga.re * sc, gi = ga.im * sc;
+  const double g2 = fma(gi, gi, gr * gr), lim = tol * (as * bs);
+  if (!(g2 > tol * lim) || !(g2 > 0.0)) return false;
+  off = g2 * 16.0 > lim ? 1.f : 0.f;
+  const float d = (float)(bs - as), fr = fabsf((float)gr), fi = fabsf((float)gi);
+  const float m = fmaxf(fr, fi), q = fminf(fr, fi);
+  if (m > 1e-30f) {
+    const float rm = __frcp_rn(m), qm = q * rm, h1 = rsqrtf(fmaf(qm, qm, 1.f));
+    const float rg0 = rm * h1;  // 1 / |gamma|
+    const float zt = d * 0.5f * rg0, az = fabsf(zt);
+    const float t = copysignf(az > 1e15f ? __fdividef(0.5f, az) : __frcp_rn(az + sqrtf(fmaf(zt, zt, 1.f))), zt);
+    const double td = (double)t;
+    r.c = rsqrt_from(fma(td, td, 1.0), (double)rsqrtf(fmaf(t, t, 1.f)));
+    r.s = td * r.c;
+    const double rg = rsqrt_from(g2, (double)rg0);
+    r.tg = td * (g2 * rg) * back;
+    r.e = C2<double>{gr * rg, -gi * rg};
+    return r.s != 0.0;
+  }
+  // gamma below FP32's range beside the larger norm (columns 1e-30 apart and more)
+  const double rg = rsqrt(g2), zt = (bs - as) * 0.5 * rg, az = fabs(zt);
+  const double t = copysign(az > 1e15 ? 0.5 / az : 1.0 / (az + sqrt(fma(zt, zt, 1.0))), zt);
+  r.c = rsqrt(fma(t, t, 1.0));
+  r.s = t * r.c;
+  r.tg = t * (g2 * rg) * back;
+  r.e = C2<double>{gr * rg, -gi * rg};
+  return r.s != 0.0;
+}
+
+// One-sided (Hestenes) Jacobi on the pe (even) columns of L (p rows, ld LDL) in
+// shared memory; with EXT the rotations are applied to V (pe rows, ld ldv) too.
+// One column pair per group of tpp threads (at most tpp_max, fewer where the
+// pe/2 pairs of a round need more groups; 4..32), round-robin ordering.  FP64:
+// the squared norms (nrm, pe values) are formed at each sweep's start and
+// carried through its rotations, so that a pair costs 4 operations a row on the
+// narrow FP64 pipe instead of 8; a norm that cancels away is formed anew by the
+// next sweep, which such a rotation always brings.  (FP32, latency-bound, loses
+// by it: leaf Jacobi 1.12 -> 1.16 ms at n = 32768.)  Ends when a sweep rotates nothing, or when its largest rotated ratio
+// is below sqrt(tol) / 4: by quadratic convergence the next sweep's ratios stay
+// below tol.  Every thread of the CTA; true if it converged.
+template <typename T, int P_T, int NT, bool EXT>
+__device__ __forceinline__ bool jacobi_sweeps(C2<T>* Lm, int LDL, int p, C2<T>* V, int ldv, int pe, T tol,
+                                              int max_sweeps, int tpp_max, T* nrm, int& nsweeps) {
   const int tid = threadIdx.x, warp = tid >> 5;
   __shared__ int sh_rot[2];
-  __shared__ unsigned sh_off[2];  // per sweep parity: largest |gamma| / sqrt(alpha beta) rotated (float bits)
-  __shared__ int sh_k;
-  (void)t_b;
-  // ---------------------------------------------------------------- 2. Jacobi
-  // one column pair per group of tpp threads (at most the tuning table's
-  // width for this class, fewer where the pe/2 pairs of a round need more
-  // groups; 4..32); round-robin ordering over pe columns
-  const int pe = K + (K & 1);
-  const T tol = T(p) * Eps<T>::u;
+  __shared__ unsigned sh_off[2];  // per sweep parity: largest ratio rotated (float bits)
   constexpr int JH = (P_T / 2 + NT / 4 - 1) / (NT / 4);  // pairs per group at most
-  int tpp = a.jacobi_tpp[factor_class(P_T)];
+  constexpr bool CARRY = sizeof(T) == 8;
+  int tpp = tpp_max;
   while (tpp > 4 && tpp * (pe / 2) > NT) tpp >>= 1;
   const int jng = NT / tpp;
   const int jg = tid / tpp, jl = tid & (tpp - 1);
@@ -559,11 +663,24 @@ __device__ __forceinline__ void jacobi_rank_q(const PairArgs<T>& a, int side, in
     sh_off[1] = 0u;
   }
   __syncthreads();
-  bool conv = pe < 2;
-  int nsweeps = 0;
-  for (int sweep = 0; sweep < a.max_sweeps && pe >= 2; ++sweep) {
+  nsweeps = 0;
+  if (pe < 2) return true;
+  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
     ++nsweeps;
     const int sp = sweep & 1;
+    if constexpr (CARRY) {
+      const int grp = tid >> 3, gl = tid & 7;
+      for (int jb = 0; jb < pe; jb += NT / 8) {
+        const int j = jb + grp;
+        T s = T(0);
+        if (j < pe)
+          for (int r = gl; r < p; r += 8) s = nmac(s, Lm[j * LDL + r]);
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (j < pe && gl == 0) nrm[j] = s;
+      }
+      __syncthreads();
+    }
     // round-robin positions of this group's pairs in round 0; each round
     // moves every position but the fixed one (index 0) by one place
     int ia[JH], ib[JH];
@@ -580,50 +697,51 @@ __device__ __forceinline__ void jacobi_rank_q(const PairArgs<T>& a, int side, in
         // warps with an active group run the reductions converged (full mask)
         if ((warp * 32) / tpp + h * jng < pe / 2) {
           const bool act = kk < pe / 2;
-          C2<T>* ca = Lm + (act ? ia[h] : 0) * LDL;
-          C2<T>* cb = Lm + (act ? ib[h] : 0) * LDL;
-          T al = T(0), be = T(0);
+          const int ja = act ? ia[h] : 0, jb = act ? ib[h] : 0;
+          C2<T>* ca = Lm + ja * LDL;
+          C2<T>* cb = Lm + jb * LDL;
           C2<T> ga = czero<T>();
+          T al = T(0), be = T(0);
+          if constexpr (CARRY) {
+            al = nrm[ja];
+            be = nrm[jb];
+            __syncwarp();  // read by the whole group before its first lane writes them
+          }
           if (act)
             for (int r = jl; r < p; r += tpp) {
               const C2<T> xa = ca[r], xb = cb[r];
-              al = nmac(al, xa);
-              be = nmac(be, xb);
+              if constexpr (!CARRY) {
+                al = nmac(al, xa);
+                be = nmac(be, xb);
+              }
               ga = cmacc(ga, xb, xa);  // + conj(xa) * xb
             }
           for (int o = 1; o < tpp; o <<= 1) {
-            al += __shfl_xor_sync(0xffffffffu, al, o);
-            be += __shfl_xor_sync(0xffffffffu, be, o);
+            if constexpr (!CARRY) {
+              al += __shfl_xor_sync(0xffffffffu, al, o);
+              be += __shfl_xor_sync(0xffffffffu, be, o);
+            }
             ga.re += __shfl_xor_sync(0xffffffffu, ga.re, o);
             ga.im += __shfl_xor_sync(0xffffffffu, ga.im, o);
           }
-          const T g2 = cnorm2(ga);
-          // rotate unless the pair is orthogonal to tol (relative)
-          // rotation scalars from reciprocal square roots and one quotient
-          // (hardware approximations in FP32, a few ulp): c^2 + s^2 = 1 to
-          // that level, far inside the convergence test's tol = p u
-          const T rg = frsqrt(g2);
-          const T off = g2 * rg * frsqrt(al) * frsqrt(be);  // |gamma| / sqrt(alpha beta)
-          if (act && al > Eps<T>::tiny && be > Eps<T>::tiny && g2 > T(0) && off > tol) {
-            const T zt = (be - al) * T(0.5) * rg;
-            const T az = fabs(zt);
-            const T q1 = T(1) + zt * zt;
-            const T t = (zt >= T(0) ? T(1) : T(-1)) *
-                        (az > T(1e15) ? fdiv(T(0.5), az) : fdiv(T(1), az + q1 * frsqrt(q1)));
-            const T c = frsqrt(T(1) + t * t);
-            const T s = t * c;
-            if (s != T(0)) {
-              const C2<T> e = C2<T>{ga.re * rg, -ga.im * rg};  // e^{-i arg gamma}
-              for (int r = jl; r < p; r += tpp) {
-                const C2<T> xa = ca[r];
-                const C2<T> eb = cmul(e, cb[r]);
-                ca[r] = C2<T>{c * xa.re - s * eb.re, c * xa.im - s * eb.im};
-                cb[r] = C2<T>{s * xa.re + c * eb.re, s * xa.im + c * eb.im};
+          Rot<T> q;
+          float off;
+          if (act && rot_scalars<EXT>(al, be, ga, tol, q, off)) {
+            auto turn = [&](C2<T>& ra, C2<T>& rb) {
+              const C2<T> xa = ra, eb = cmul(q.e, rb);
+              ra = C2<T>{q.c * xa.re - q.s * eb.re, q.c * xa.im - q.s * eb.im};
+              rb = C2<T>{q.s * xa.re + q.c * eb.re, q.s * xa.im + q.c * eb.im};
+            };
+            for (int r = jl; r < p; r += tpp) turn(ca[r], cb[r]);
+            if constexpr (EXT)
+              for (int r = jl; r < pe; r += tpp) turn(V[ja * ldv + r], V[jb * ldv + r]);
+            if (jl == 0) {
+              if constexpr (CARRY) {
+                nrm[ja] = al - q.tg;
+                nrm[jb] = be + q.tg;
               }
-              if (jl == 0) {
-                sh_rot[sp] = 1;
-                atomicMax(&sh_off[sp], __float_as_uint((float)off));
-              }
+              sh_rot[sp] = 1;
+              atomicMax(&sh_off[sp], __float_as_uint(off));
             }
           }
           if (act) {
@@ -639,16 +757,178 @@ __device__ __forceinline__ void jacobi_rank_q(const PairArgs<T>& a, int side, in
       }
     }
     const int rot = sh_rot[sp];
-    // quadratic convergence: once the largest rotated off-diagonal ratio of a
-    // sweep is below sqrt(tol) / 4, the next sweep's ratios stay below tol,
-    // so that confirming sweep is not run
-    const T offmax = (T)__uint_as_float(sh_off[sp]);
+    const float offmax = __uint_as_float(sh_off[sp]);
     __syncthreads();
-    if (rot == 0 || offmax * offmax * T(16) <= tol) {
-      conv = true;
-      break;
+    // FP64: offmax is 1 where a ratio exceeded sqrt(tol) / 4, else 0
+    if (rot == 0 || (sizeof(T) == 4 ? offmax * offmax * 16.f <= (float)tol : offmax == 0.f)) return true;
+  }
+  return false;
+}
+
+// FP64: L turned by the right singular vectors that an FP32 Jacobi finds, so
+// that the FP64 sweeps start from columns orthogonal to ~1e-6 and two of them
+// are left (of 5.6).  V (FP32, accumulated rotations) is unitary to ~1e-6; L is
+// multiplied by its polar factor V (I + E)^{-1/2} = V (I - F), E = V^* V - I, F =
+// E/2 - 3/8 E^2 (E^3 is below 1e-18; E^2 in FP32 to 1e-19), unitary to FP64
+// rounding: L' = Y - Y F, Y = L V.  About 12 p K^2 FP64 operations, less than a
+// sweep.  work: at least pe LDL + pe^2/2 entries.
+template <int P_T, int NT>
+__device__ __forceinline__ void jacobi_precondition(C2<double>* Lm, int LDL, int p, int pe, C2<double>* work,
+                                                    int tpp_max) {
+  const int tid = threadIdx.x;
+  C2<double>* Y = work;
+  C2<float>* V = reinterpret_cast<C2<float>*>(work + pe * LDL);  // pe x pe, ld pe
+  C2<float>* L32 = reinterpret_cast<C2<float>*>(work);           // over Y, ld LDL
+  // scaled by the power of two that brings the largest entry near 1
+  __shared__ int sh_ex;
+  if (tid == 0) sh_ex = 0;
+  __syncthreads();
+  int ex = 0;
+  for (int i = tid; i < pe * p; i += NT) {
+    const C2<double> v = Lm[(i / p) * LDL + i % p];
+    ex = max(ex, max((__double2hiint(v.re) >> 20) & 0x7ff, (__double2hiint(v.im) >> 20) & 0x7ff));
+  }
+  atomicMax(&sh_ex, ex);
+  __syncthreads();
+  ex = sh_ex;
+  if (ex <= 1 || ex >= 2045) return;  // zero or not finite
+  __syncthreads();
+  if (tid == 0) sh_ex = 0;  // then the largest |E| (its bits)
+  const double sc = __hiloint2double((2046 - ex) << 20, 0);
+  for (int i = tid; i < pe * p; i += NT) {
+    const C2<double> v = Lm[(i / p) * LDL + i % p];
+    L32[(i / p) * LDL + i % p] = C2<float>{(float)(v.re * sc), (float)(v.im * sc)};
+  }
+  for (int i = tid; i < pe * pe; i += NT) V[i] = C2<float>{i / pe == i % pe ? 1.f : 0.f, 0.f};
+  __syncthreads();
+  int ns;
+  jacobi_sweeps<float, P_T, NT, true>(L32, LDL, p, V, pe, pe, (float)p * Eps<float>::u, 12, tpp_max, nullptr, ns);
+  __syncthreads();
+  // four rows of one column per thread: V's entries are converted once for four products
+  const int nrt = (p + 3) >> 2;
+  for (int i = tid; i < nrt * pe; i += NT) {
+    const int r = 4 * (i % nrt), j = i / nrt;
+    C2<double> s[4] = {czero<double>(), czero<double>(), czero<double>(), czero<double>()};
+    for (int l = 0; l < pe; ++l) {
+      const C2<float> v = V[j * pe + l];
+      const C2<double> vd{(double)v.re, (double)v.im};
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (r + u < p) s[u] = cmac_nc(s[u], Lm[l * LDL + r + u], vd);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (r + u < p) Y[j * LDL + r + u] = s[u];
+  }
+  __syncthreads();
+  // E by 2 x 2 tiles (j, j + 1) x (k, k + 1)
+  constexpr int ET = (P_T / 2 * (P_T / 2) + NT - 1) / NT;  // tiles per thread at most
+  C2<double> E[ET][4];
+  const int ht = pe >> 1;
+#pragma unroll
+  for (int h = 0; h < ET; ++h) {
+    const int i = tid + h * NT, j = 2 * (i % ht), k = 2 * (i / ht);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) E[h][u] = czero<double>();
+    if (i < ht * ht)
+      for (int l = 0; l < pe; ++l) {
+        const auto at = [&](int col) {
+          const C2<float> v = V[col * pe + l];
+          return C2<double>{(double)v.re, (double)v.im};
+        };
+        const C2<double> a0 = at(j), a1 = at(j + 1), b0 = at(k), b1 = at(k + 1);
+        E[h][0] = cmacc(E[h][0], b0, a0);  // + conj(a) b
+        E[h][1] = cmacc(E[h][1], b0, a1);
+        E[h][2] = cmacc(E[h][2], b1, a0);
+        E[h][3] = cmacc(E[h][3], b1, a1);
+      }
+  }
+  __syncthreads();
+  C2<float>* E32 = V;  // V has been read
+  float emax = 0.f;
+#pragma unroll
+  for (int h = 0; h < ET; ++h) {
+    const int i = tid + h * NT, j = 2 * (i % ht), k = 2 * (i / ht);
+    if (i < ht * ht)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int jj = j + (u & 1), kk = k + (u >> 1);
+        if (jj == kk) E[h][u].re -= 1.0;
+        const C2<float> e{(float)E[h][u].re, (float)E[h][u].im};
+        E32[kk * pe + jj] = e;
+        emax = fmaxf(emax, fmaxf(fabsf(e.re), fabsf(e.im)));
+      }
+  }
+  atomicMax(&sh_ex, __float_as_int(emax));
+  __syncthreads();
+  // not unitary enough for the expansion (not seen; NaN and infinity order
+  // above): L stays as it is, and the FP64 sweeps do all the work
+  if (__int_as_float(sh_ex) > 2e-5f || sh_ex < 0 || sh_ex >= 0x7f800000) return;
+#pragma unroll
+  for (int h = 0; h < ET; ++h) {
+    const int i = tid + h * NT, j = 2 * (i % ht), k = 2 * (i / ht);
+    if (i < ht * ht)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int jj = j + (u & 1), kk = k + (u >> 1);
+        C2<float> s = czero<float>();
+        for (int l = 0; l < pe; ++l) s = cmacc(s, E32[kk * pe + l], E32[jj * pe + l]);  // E is Hermitian
+        Lm[kk * LDL + jj] =
+            C2<double>{fma(-0.375, (double)s.re, 0.5 * E[h][u].re), fma(-0.375, (double)s.im, 0.5 * E[h][u].im)};
+      }
+  }
+  __syncthreads();
+  // L' = Y - Y F, held until every thread has read F
+  constexpr int YT = (P_T / 4 * P_T + NT - 1) / NT;
+  C2<double> o[YT][4];
+#pragma unroll
+  for (int h = 0; h < YT; ++h) {
+    const int i = tid + h * NT, r = 4 * (i % nrt), j = i / nrt;
+    if (i < nrt * pe) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) o[h][u] = r + u < p ? Y[j * LDL + r + u] : czero<double>();
+      for (int l = 0; l < pe; ++l) {
+        const C2<double> f = Lm[j * LDL + l];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (r + u < p) o[h][u] = cnmac(o[h][u], f, Y[l * LDL + r + u]);
+      }
     }
   }
+  __syncthreads();
+#pragma unroll
+  for (int h = 0; h < YT; ++h) {
+    const int i = tid + h * NT, r = 4 * (i % nrt), j = i / nrt;
+    if (i < nrt * pe)
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (r + u < p) Lm[j * LDL + r + u] = o[h][u];
+  }
+  __syncthreads();
+}
+
+// Steps 2-4 of a pair (Jacobi on the K leading columns of L in shared memory,
+// the rank from the tail sums, Q), shared by pair_kernel and
+// gram_jacobi_kernel.  work: free shared memory of work_n entries (FP64's
+// preconditioner; none in FP32).
+template <typename T, int P_T, int NT>
+__device__ __forceinline__ void jacobi_rank_q(const PairArgs<T>& a, int side, int pid, int p, int LDL, int K,
+                                              double E_K, int kcap, int lvl, C2<T>* Lm, double* sig2, int* ord,
+                                              int32_t* rank_out, double* sig_out, long long t_b, C2<T>* work,
+                                              int work_n) {
+  const int tid = threadIdx.x;
+  __shared__ int sh_k;
+  (void)t_b;
+  (void)work;
+  (void)work_n;
+  const int pe = K + (K & 1);
+  const int tpp = a.jacobi_tpp[factor_class(P_T)];
+  if constexpr (sizeof(T) == 8 && P_T <= 64)
+    if (pe >= 4 && pe * LDL + (pe * pe + 1) / 2 <= work_n)
+      jacobi_precondition<P_T, NT>(Lm, LDL, p, pe, work, tpp);
+  int nsweeps = 0;
+  const bool conv = jacobi_sweeps<T, P_T, NT, false>(Lm, LDL, p, nullptr, 0, pe, T(p) * Eps<T>::u, a.max_sweeps, tpp,
+                                                     reinterpret_cast<T*>(sig2), nsweeps);
   if (!conv && tid == 0) atomicOr(a.status, kStatusNoConv);
   DH2_PROF_T(t_c);
   DH2_PROF_ADD(1, t_c - t_b);
@@ -660,6 +940,7 @@ __device__ __forceinline__ void jacobi_rank_q(const PairArgs<T>& a, int side, in
 
   // ---------------------------------------------------------------- 3. rank
   const int grp = tid >> 3, gl = tid & 7;
+  __syncthreads();  // the carried norms share sig2's place
   for (int jb = 0; jb < K; jb += NT / 8) {
     const int j = jb + grp;
     T s = T(0);
@@ -754,13 +1035,16 @@ constexpr int gram_min_blocks() {
   return NT >= 256 ? 3 : NT >= 192 ? DH2_GRAM_MINB192 : NT >= 160 ? DH2_GRAM_MINB160 : DH2_GRAM_MINB128;
 }
 
+// FP64: 4 CTAs at 128 threads (128 registers, a few spills) and 2 at 160 and 192
+// keep the FP64 pipe fed between the barriers of a round or step (leaf factors at
+// n = 8192, 128 threads: 2 CTAs 30.9 ms, 3 26.9, 4 25.8)
 template <int NT, typename T>
 constexpr int pair_min_blocks() {
   return sizeof(T) == 4 ? (NT >= 256   ? DH2_PAIR_MINB
                            : NT >= 192 ? DH2_PAIR_MINB192
                            : NT >= 160 ? DH2_PAIR_MINB160
                                        : DH2_PAIR_MINB128)
-                        : (NT >= 160 ? 1 : 2);
+                        : (NT >= 256 ? 1 : NT >= 160 ? 2 : 4);
 }
 
 template <typename T, int P_T, bool FROM_R, int NT, bool GRAM = false>
@@ -938,6 +1222,10 @@ __global__ void __launch_bounds__(NT, (GRAM ? gram_min_blocks<NT>() : pair_min_b
   // (beta, 0, ..., 0) on the columns {r} u chunk, beta = -e^{i arg alpha} |x|;
   // the chunk part x is the reflection's vector (vbuf[slot]).  Called by a
   // whole warp; only the quarter holding row r (mine) works.
+  // eu: entries of a thread in use (FP64: the pairs past the chunk's last column
+  // are zero and left out; FP32, latency-bound, runs all E)
+  int eu = E;
+  auto used = [&](int u) { return sizeof(T) == 4 || u < eu; };
   auto publish = [&](int r, const C2<T> (&x)[E], bool mine, int slot) {
     if (!mine) return;
     const unsigned qmask = ((1u << LQT) - 1u) << (lane & (32 - LQT));
@@ -952,10 +1240,11 @@ __global__ void __launch_bounds__(NT, (GRAM ? gram_min_blocks<NT>() : pair_min_b
     for (int u = 0; u < E; u += 2) store_c2x2(vbuf + slot * C + ccol(u), x[u], x[u + 1]);
     T s0 = T(0), s1 = T(0);
 #pragma unroll
-    for (int u = 0; u < E; u += 2) {
-      s0 = nmac(s0, x[u]);
-      if (u + 1 < E) s1 = nmac(s1, x[u + 1]);
-    }
+    for (int u = 0; u < E; u += 2)
+      if (used(u)) {
+        s0 = nmac(s0, x[u]);
+        if (u + 1 < E) s1 = nmac(s1, x[u + 1]);
+      }
     s0 += s1;
 #pragma unroll
     for (int o = 1; o < LQT; o <<= 1) s0 += __shfl_xor_sync(qmask, s0, o);
@@ -967,7 +1256,7 @@ __global__ void __launch_bounds__(NT, (GRAM ? gram_min_blocks<NT>() : pair_min_b
         const T xn = xn2 * frsqrt(xn2);
         Lm[r * LDL + r] = C2<T>{-ph.re * xn, -ph.im * xn};
         sh_v0[slot] = C2<T>{ph.re * (an + xn), -ph.im * (an + xn)};
-        sh_tau[slot] = fdiv(T(1), xn * (xn + an));
+        sh_tau[slot] = frcp(xn * (xn + an));
         sh_skip[slot] = 0;
       }
     }
@@ -987,7 +1276,11 @@ __global__ void __launch_bounds__(NT, (GRAM ? gram_min_blocks<NT>() : pair_min_b
     for (int u = 0; u < E; u += 2) load_c2x2(xs + ccol(u), x[u], x[u + 1]);
     C2<T> wa[4] = {czero<T>(), czero<T>(), czero<T>(), czero<T>()};
 #pragma unroll
-    for (int u = 0; u < E; ++u) wa[u & 3] = cmacc(wa[u & 3], c[u], x[u]);
+    for (int u = 0; u < E; u += 2)
+      if (used(u)) {
+        wa[u & 3] = cmacc(wa[u & 3], c[u], x[u]);
+        wa[(u + 1) & 3] = cmacc(wa[(u + 1) & 3], c[u + 1], x[u + 1]);
+      }
     C2<T> w = cadd(cadd(wa[0], wa[1]), cadd(wa[2], wa[3]));
 #pragma unroll
     for (int o = 1; o < LQT; o <<= 1) {
@@ -997,7 +1290,11 @@ __global__ void __launch_bounds__(NT, (GRAM ? gram_min_blocks<NT>() : pair_min_b
     w = cadd(w, cmul(lrj, v0));
     const C2<T> tw = C2<T>{tau * w.re, tau * w.im};
 #pragma unroll
-    for (int u = 0; u < E; ++u) c[u] = cnmac(c[u], tw, x[u]);
+    for (int u = 0; u < E; u += 2)
+      if (used(u)) {
+        c[u] = cnmac(c[u], tw, x[u]);
+        c[u + 1] = cnmac(c[u + 1], tw, x[u + 1]);
+      }
     if (lq == 0) Lm[j * LDL + r] = csub(lrj, cmulc(tw, v0));
   };
 
@@ -1071,6 +1368,7 @@ __global__ void __launch_bounds__(NT, (GRAM ? gram_min_blocks<NT>() : pair_min_b
 #pragma unroll
       for (int u = 0; u < E; ++u) ch[s][u] = r < p ? Xs[ccol(u) * LDL + r] : czero<T>();
     }
+    eu = 2 * ((min(C, N - j0) + 2 * LQT - 1) / (2 * LQT));
     if (warp == 0) publish(0, ch[0], lrow(0) == 0, 0);
     __syncthreads();
     const int j0n = j0 + C;
@@ -1259,7 +1557,7 @@ __global__ void __launch_bounds__(NT, (GRAM ? gram_min_blocks<NT>() : pair_min_b
           const C2<T> ph = an2 > Eps<T>::tiny ? C2<T>{al.re * ra, al.im * ra} : C2<T>{T(1), T(0)};
           Lm[i * LDL + pv] = C2<T>{-ph.re * xn, -ph.im * xn};
           sh_v0[0] = C2<T>{ph.re * (an + xn), -ph.im * (an + xn)};
-          sh_tau[0] = fdiv(T(1), xn * (xn + an));
+          sh_tau[0] = frcp(xn * (xn + an));
           sh_skip[0] = 0;
         }
       }
@@ -1334,7 +1632,8 @@ __global__ void __launch_bounds__(NT, (GRAM ? gram_min_blocks<NT>() : pair_min_b
     }
   }
   __syncthreads();
-  jacobi_rank_q<T, P_T, NT>(a, side, pid, p, LDL, K, E_K, kcap, lvl, Lm, sig2, ord, rank_out, sig_out, t_b);
+  jacobi_rank_q<T, P_T, NT>(a, side, pid, p, LDL, K, E_K, kcap, lvl, Lm, sig2, ord, rank_out, sig_out, t_b,
+                            Lm + (int64_t)P * LDL, XTRA * LDL);
 }
 
 // Steps 2-4 of the leaf pairs of a mixed-mode launch list, after the
@@ -1375,7 +1674,7 @@ __global__ void __launch_bounds__(NT, MINB)
   t_b = clock64();
 #endif
   jacobi_rank_q<float, P_T, NT>(a, side, pid, p, LDL, K, E_K, a.kcap[side][pid], a.level[side][pid], Lm, sig2, ord,
-                                rank_out, sig_out, t_b);
+                                rank_out, sig_out, t_b, nullptr, 0);
 }
 
 // R_tc = Q^* A for the pairs of one launch (Section 6, R recursion: R_tc =
