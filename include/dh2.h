@@ -466,9 +466,9 @@ enum {
   DH2_KC_CLASSIFY = 17,     /* row classes of a level's non-leaf pairs                           */
   DH2_KC_EXPAND = 18,       /* expansion of non-leaf column bases (Eq. nested)                   */
   DH2_KC_PROJECT = 19,      /* coupling matrices S_b                                             */
-  DH2_KC_LEAF_GRAM = 20,    /* + leaf row class 0..3: tensor-core Gram matrices (MIXED_BF16X3)   */
+  DH2_KC_LEAF_GRAM = 20,    /* + leaf row class 0..3: Gram matrices (MIXED_BF16X3: tensor cores; FP32) */
   DH2_KC_GRAM_SCALES = 24,  /* row scales of the leaf Gram matrices (MIXED_BF16X3)               */
-  DH2_KC_LEAF_JACOBI = 25,  /* + leaf row class 0..3: Jacobi, rank and Q after the Cholesky (MIXED) */
+  DH2_KC_LEAF_JACOBI = 25,  /* + leaf row class 0..3: Jacobi, rank and Q after the Cholesky (MIXED, FP32) */
   DH2_KC_LEAF_R_TC = 29,    /* leaf R_tc = Q_tc^* G^omega_tc on the tensor cores, all classes (MIXED) */
   DH2_KC_COUNT = 32
 };

@@ -23,8 +23,7 @@ CUDA_SOURCES = ["dh2_pair.cu", "dh2_gram.cu", "dh2_rq_tc.cu", "dh2_ops.cu", "dh2
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # build-time tuning macros, read from the environment (integers; the defaults,
 # the measured best, sit beside each #ifndef in csrc/)
-TUNING_MACROS = ("DH2_PAIR_MINB", "DH2_PAIR_MINB192", "DH2_PAIR_MINB160", "DH2_PAIR_MINB128", "DH2_LQT",
-                 "DH2_HOST_PANELS", "DH2_GRAM_MINB128", "DH2_GRAM_MINB160", "DH2_GRAM_MINB192", "DH2_RQ_MINB",
+TUNING_MACROS = ("DH2_PAIR_MINB", "DH2_LQT", "DH2_HOST_PANELS", "DH2_GRAM_MINB128", "DH2_GRAM_MINB160", "DH2_GRAM_MINB192", "DH2_RQ_MINB",
                  "DH2_PROJ_MINB")
 
 

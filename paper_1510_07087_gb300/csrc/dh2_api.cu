@@ -82,7 +82,7 @@ struct Tree::Dev {
   int32_t *cluster[2], *leaf[2], *start[2], *m[2], *ncols[2], *son[2], *sonoff[2], *level[2], *kcap[2],
       *rowcap[2];
   int64_t *cmoff[2], *Roff[2], *Qoff[2], *Xoff[2], *hoff[2];
-  int64_t* gram_off[2];  // mixed modes: leaf Gram matrix offsets
+  int64_t* gram_off[2];  // Gram matrix offsets (leaf pairs; non-leaf pairs: from their level's start)
   int32_t *gcol[2], *gblk[2];
   int64_t* seg_dst[2];  // column-map segments (expanded into gcol/gblk on upload)
   int64_t* seg_begin[2];  // per pair: first segment
@@ -115,7 +115,11 @@ struct Tree::Dev {
   // host-side sizes
   int64_t npairs[2] = {0, 0}, nleaf[2] = {0, 0};
   int64_t R_elems[2] = {0, 0}, Q_elems[2] = {0, 0}, X_elems[2] = {0, 0}, h_elems[2] = {0, 0};
-  int64_t gram_elems = 0;  // both sides together
+  int64_t gram_elems = 0;  // leaf Gram matrices, both sides together
+  int64_t lvl_gram_elems = 0;  // non-leaf Gram matrices (one per column segment) of the largest level
+  std::vector<uint64_t> gseg_h;  // per level: non-leaf pairs' column segments, code << 32 | segment
+  std::vector<int64_t> gseg_begin, gseg_count;
+  uint64_t* gseg = nullptr;
   int64_t S_elems = 0, near_elems = 0, bmax_elems = 0;
   int64_t nadm = 0, ninadm = 0;
   int64_t nleaf_codes = 0;
@@ -284,6 +288,7 @@ dh2_status upload_tree(Tree& tr) {
   add32(std::vector<int32_t>(tr.level), &D->clevel);
   D->max_leaf = tr.max_leaf;
 
+  std::vector<int64_t> lvl_gram(tr.depth + 1, 0);  // both sides of a level share its Gram buffer
   for (int sd = 0; sd < 2; ++sd) {
     Side& S = tr.side[sd];
     const int64_t np = (int64_t)S.pairs.size();
@@ -317,6 +322,9 @@ dh2_status upload_tree(Tree& tr) {
         kc[p] = (int32_t)std::min<int64_t>(rc[p], P.ncols);
         xo[p] = X_e;
         X_e += (int64_t)tr.size[P.cluster] * kc[p];
+        const int64_t mpd = (std::min(rc[p], kGramRows) + 7) & ~7;
+        go[p] = lvl_gram[P.level];
+        lvl_gram[P.level] += mpd * mpd * ((P.ncols + kGramSegCols - 1) / kGramSegCols);
       }
       ro[p] = R_e;
       R_e += (int64_t)kc[p] * P.ncols;
@@ -519,18 +527,26 @@ dh2_status upload_tree(Tree& tr) {
     for (int c = 1; c <= kLeafClasses; ++c)
       D->leaf_class_begin[c] = std::max(D->leaf_class_begin[c], D->leaf_class_begin[c - 1]);
     D->nleaf_codes = (int64_t)codes.size();
+    for (int64_t e : lvl_gram) D->lvl_gram_elems = std::max(D->lvl_gram_elems, e);
+    D->gseg_begin.assign(tr.depth + 1, 0);
+    D->gseg_count.assign(tr.depth + 1, 0);
     D->nl_code_begin.assign(tr.depth + 1, 0);
     D->nl_code_count.assign(tr.depth + 1, 0);
     D->nl_rowcap_max.assign(tr.depth + 1, 0);
     for (int l = tr.depth; l >= 0; --l) {
       D->nl_code_begin[l] = (int64_t)codes.size();
+      D->gseg_begin[l] = (int64_t)D->gseg_h.size();
       for (int sd = 0; sd < 2; ++sd)
         for (int64_t p : tr.side[sd].nonleaf_by_level[l]) {
           codes.push_back((int32_t)((sd << kCodeSideShift) | (int32_t)p));
+          const int64_t nseg = (tr.side[sd].pairs[p].ncols + kGramSegCols - 1) / kGramSegCols;
+          for (int64_t g = 0; g < nseg; ++g) D->gseg_h.push_back(((uint64_t)(uint32_t)codes.back() << 32) | (uint64_t)g);
           D->nl_rowcap_max[l] = std::max(D->nl_rowcap_max[l], D->rowcap_h[sd][p]);
         }
       D->nl_code_count[l] = (int64_t)codes.size() - D->nl_code_begin[l];
+      D->gseg_count[l] = (int64_t)D->gseg_h.size() - D->gseg_begin[l];
     }
+    bufs.push_back({D->gseg_h.data(), bytes_of(D->gseg_h), (void**)&D->gseg});
     // R tiles of 32 columns per pair, in the order of the codes
     std::vector<int64_t> tiles;
     auto add_tiles = [&](int32_t code) {
@@ -729,8 +745,7 @@ void fill_args(dh2_matrix* M, const dh2_compress_params& cp, PairArgs<T>& pa, No
   pa.ld = M->ld;
   pa.invw = M->invw;
   pa.eps2 = M->eps2;
-  pa.H = nullptr;  // set by run_compress in the mixed modes
-  pa.L4 = nullptr;
+  pa.H = pa.L4 = pa.Hl = nullptr;  // set by run_compress in the FP32 and mixed modes
   for (int sd = 0; sd < 2; ++sd) {
     pa.hoff[sd] = D->gram_off[sd];
     pa.rank_ovr[sd] = nullptr;  // set by run_compress when ranks are given
@@ -928,6 +943,11 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
   std::vector<std::vector<uint64_t>> nl_tiles(maxdepth + 1);
   size_t args_bytes = align256(sizeof(PairArgs<T>) * nprob) + align256(sizeof(NormsArgs<T>) * nprob);
   size_t codes_bytes = 0;
+  // FP32 and mixed modes: the column segments of a level's pairs (Gram matrices)
+  constexpr bool f32 = sizeof(T) == 4;
+  std::vector<std::vector<uint64_t>> gsegs(maxdepth + 1);
+  std::vector<const uint64_t*> d_gseg(maxdepth + 1, nullptr);
+  std::vector<int64_t> n_gseg(maxdepth + 1, 0);
   if (nprob > 1) {
     struct LC {
       int cls;
@@ -948,6 +968,12 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
         for (int sd = 0; sd < 2; ++sd)
           for (int64_t p : tr.side[sd].nonleaf_by_level[l])
             nl_codes[l].push_back(((uint32_t)i << kCodeProbShift) | ((uint32_t)sd << kCodeSideShift) | (uint32_t)p);
+      if (f32) {
+        const Tree::Dev* D = tr.dev;
+        for (int l = 0; l <= tr.depth; ++l)
+          for (int64_t q = D->gseg_begin[l]; q < D->gseg_begin[l] + D->gseg_count[l]; ++q)
+            gsegs[l].push_back(D->gseg_h[q] | ((uint64_t)i << (32 + kCodeProbShift)));
+      }
       for (size_t b = 0; b < tr.blocks.size(); ++b)
         if (tr.blocks[b].adm) norm_codes.push_back(((uint32_t)i << 26) | (uint32_t)b);
     }
@@ -993,7 +1019,7 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
     codes_bytes = align256(4 * leaf_codes.size()) + align256(4 * norm_codes.size()) + align256(8 * leaf_tiles.size()) +
                   align256(8 * pieces.size()) + align256(8 * pbegin.size());
     for (int l = 0; l <= maxdepth; ++l)
-      codes_bytes += align256(4 * nl_codes[l].size()) + align256(8 * nl_tiles[l].size());
+      codes_bytes += align256(4 * nl_codes[l].size()) + align256(8 * nl_tiles[l].size()) + align256(8 * gsegs[l].size());
   }
   // per level: the non-leaf codes sorted into row-count classes
   int64_t nl_max = 0;
@@ -1033,21 +1059,24 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
       }
     for (const HList& L : hl) host_bytes += align256(4 * L.codes->size()) + align256(8 * L.tiles.size());
   }
-  // mixed modes: the leaf Gram matrices (double-float, mp x mp per leaf pair)
-  // and the window sums of the pairs with more than one window, per problem
+  // FP32 and mixed modes: the leaf Gram matrices (double-float, mp x mp per leaf
+  // pair) and those of the largest level, per problem; mixed modes: the block
+  // maxima the leaf slices are scaled by
   const bool mixed = mode_mixed(cp.mode);
-  std::vector<size_t> gram_h_off(nprob, 0), gram_l_off(nprob, 0), gram_m_off(nprob, 0);
+  std::vector<size_t> gram_h_off(nprob, 0), gram_l_off(nprob, 0), gram_m_off(nprob, 0), gram_lvl_off(nprob, 0);
   size_t gram_bytes = 0;
-  if (mixed) {
-    gram_bytes = align256(sizeof(GramArgs) * nprob);
+  if (f32) {
+    if (mixed) gram_bytes = align256(sizeof(GramArgs) * nprob);
     for (int i = 0; i < nprob; ++i) {
       const Tree::Dev* D = Ms[i]->tree->tr.dev;
       gram_h_off[i] = gram_bytes;
       if (!Ms[i]->gram) gram_bytes += align256(sizeof(float4) * (size_t)D->gram_elems);  // else kept by the matrix
       gram_l_off[i] = gram_bytes;  // Cholesky factors: over H, or beside the kept Gram matrices
       if (Ms[i]->gram) gram_bytes += align256(sizeof(float4) * (size_t)D->gram_elems);
+      gram_lvl_off[i] = gram_bytes;
+      gram_bytes += align256(sizeof(float4) * (size_t)D->lvl_gram_elems);
       gram_m_off[i] = gram_bytes;
-      gram_bytes += align256(sizeof(float) * (size_t)D->bmax_elems);
+      if (mixed) gram_bytes += align256(sizeof(float) * (size_t)D->bmax_elems);
     }
   }
   // ranks given instead of the truncation rule (one problem only)
@@ -1146,14 +1175,16 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
   }
   GramArgs* d_ga = (GramArgs*)gram_base;
   std::vector<GramArgs> gas;
+  for (int i = 0; i < nprob && f32; ++i) {
+    pas[i].H = Ms[i]->gram ? (float4*)Ms[i]->gram : (float4*)(gram_base + gram_h_off[i]);
+    pas[i].L4 = Ms[i]->gram ? (float4*)(gram_base + gram_l_off[i]) : pas[i].H;
+    pas[i].Hl = (float4*)(gram_base + gram_lvl_off[i]);
+  }
   if (mixed) {
     gas.resize(nprob);
     for (int i = 0; i < nprob; ++i) {
       const Tree::Dev* D = Ms[i]->tree->tr.dev;
       const dh2_matrix* M = Ms[i];
-      float4* Hbuf = Ms[i]->gram ? (float4*)Ms[i]->gram : (float4*)(gram_base + gram_h_off[i]);
-      pas[i].H = Hbuf;
-      pas[i].L4 = Ms[i]->gram ? (float4*)(gram_base + gram_l_off[i]) : Hbuf;
       GramArgs& g = gas[i];
       for (int sd = 0; sd < 2; ++sd) {
         g.start[sd] = D->start[sd];
@@ -1176,7 +1207,7 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
       nas[i].bmax = (float*)(gram_base + gram_m_off[i]);
       g.G = (const C2<float>*)M->G;
       g.ld = M->ld;
-      g.H = Hbuf;
+      g.H = pas[i].H;
       g.status = M->status;
       g.spin_limit = (uint32_t)std::min<int64_t>(std::max<int64_t>(cp.spin_limit, 0), (int64_t)UINT32_MAX);
     }
@@ -1229,6 +1260,8 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
     for (int l = 0; l <= maxdepth; ++l) {
       d_nltiles[l] = up64(nl_tiles[l]);
       n_nltiles[l] = (int64_t)nl_tiles[l].size();
+      d_gseg[l] = up64(gsegs[l]);
+      n_gseg[l] = (int64_t)gsegs[l].size();
     }
   } else {
     const Tree& tr = Ms[0]->tree->tr;
@@ -1255,6 +1288,8 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
     for (int l = 0; l <= tr.depth; ++l) {
       d_nltiles[l] = (const uint64_t*)D->tiles + D->nl_tile_begin[l];
       n_nltiles[l] = D->nl_tile_count[l];
+      d_gseg[l] = D->gseg + D->gseg_begin[l];
+      n_gseg[l] = D->gseg_count[l];
     }
   }
   if (hs) {
@@ -1333,8 +1368,9 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
     }
   };
   // leaf factors and R of one launch list per size class
-  // leaf factorisations of one size class: the streamed LQ, or in the mixed
-  // modes the tensor-core Gram matrices and their pivoted Cholesky
+  // leaf factorisations of one size class: FP64 (and FP32 above kGramRows rows)
+  // the streamed LQ; FP32 Gram matrices in integers, the mixed modes on the
+  // tensor cores, and their pivoted Cholesky
   // events around the Gram and factor launches of each class (mixed modes,
   // device input): the leaf phase split into its two kernels
   cudaEvent_t kev[4 * kLeafClasses] = {};
@@ -1351,10 +1387,18 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
         if (timed) cudaEventRecord(kev[4 * c + 1], st);
         // pivoted Cholesky, then Jacobi, rank and Q
         if (timed) cudaEventRecord(kev[4 * c + 2], st);
-        ok_launch &= launch_pair_kernel_gram(reinterpret_cast<const PairArgs<float>*>(d_pa), codes, n, P, st);
+        ok_launch &= launch_pair_kernel_gram(d_pa, codes, n, P, false, st);
         counted(DH2_KC_LEAF_FACTOR + c, true);
         counted(DH2_KC_LEAF_JACOBI + c, true);
         if (timed) cudaEventRecord(kev[4 * c + 3], st);
+        return;
+      }
+      if (cls_maxm[c] <= kGramRows) {
+        ok_launch &= launch_gram_i64(d_pa, codes, nullptr, n, P, st);
+        counted(DH2_KC_LEAF_GRAM + c, true);
+        ok_launch &= launch_pair_kernel_gram(d_pa, codes, n, P, false, st);
+        counted(DH2_KC_LEAF_FACTOR + c, true);
+        counted(DH2_KC_LEAF_JACOBI + c, true);
         return;
       }
     }
@@ -1534,8 +1578,22 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
       launch_classify<T>(d_pa, d_nl[l], n, d_cls, d_cnt, st);
       counted(DH2_KC_CLASSIFY, true);
       const int Pc[4] = {32, 48, 64, P_level[l]};
+      // FP32: pairs of at most kGramRows rows from the Gram matrices of their
+      // column segments; the LQ launches take the others
+      const int c_lq = f32 ? 3 : 0;
+      if constexpr (f32) {
+        ok_launch &= launch_gram_i64(d_pa, nullptr, d_gseg[l], (int)n_gseg[l], P_level[l], st);
+        counted(DH2_KC_LEVEL_FACTOR, true);
+        for (int c = 0; c < 3; ++c) {
+          if (c > 0 && Pc[c - 1] >= P_level[l]) break;  // no pair of this level has more rows
+          ok_launch &= launch_pair_kernel_gram(d_pa, d_cls + (int64_t)c * n, n, std::min(Pc[c], std::max(P_level[l], 2)),
+                                               true, st, d_cnt + c);
+          counted(DH2_KC_LEVEL_FACTOR + c, true);
+          counted(DH2_KC_LEVEL_FACTOR + c, true);
+        }
+      }
       // wide pairs: their column segments' factors first, by row class
-      const int nsg = (int)seg_lists[l].size();
+      const int nsg = P_level[l] > (f32 ? kGramRows : 0) ? (int)seg_lists[l].size() : 0;
       if (nsg > 0) {
         if (cudaMemsetAsync(d_seg_cnt[l], 0, 4 * sizeof(int), st) != cudaSuccess) {
           cudaGetLastError();
@@ -1543,14 +1601,14 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
         }
         launch_classify_seg<T>(d_pa, d_seg[l], nsg, d_seg_cls[l], d_seg_cnt[l], st);
         counted(DH2_KC_CLASSIFY, true);
-        for (int c = 0; c < 4; ++c) {
+        for (int c = c_lq; c < 4; ++c) {
           if (c > 0 && Pc[c - 1] >= P_level[l]) break;
           ok_launch &= launch_pair_kernel<T>(d_pa, nullptr, nsg, std::min(Pc[c], std::max(P_level[l], 2)), true, st,
                                              d_seg_cnt[l] + c, d_seg_cls[l] + (int64_t)c * nsg);
           counted(DH2_KC_LEVEL_FACTOR + c, true);
         }
       }
-      for (int c = 0; c < 4; ++c) {
+      for (int c = c_lq; c < 4; ++c) {
         if (c > 0 && Pc[c - 1] >= P_level[l]) break;  // no pair of this level has more rows
         ok_launch &= launch_pair_kernel<T>(d_pa, d_cls + (int64_t)c * n, n, std::min(Pc[c], std::max(P_level[l], 2)),
                                            true, st, d_cnt + c);

@@ -194,9 +194,12 @@ struct PairArgs {
   double* sig[2];                     // per pair P values (descending)
   int32_t* rank[2];
   const double* eps2;                 // per level eps_l^2
-  const float4* H;                    // mixed modes: leaf Gram matrices (see GramArgs)
-  float4* L4;                         // mixed modes: leaf Cholesky factors, pair at L4 + its Gram offset (FP32 complex, ld p)
-  const int64_t* hoff[2];             // mixed modes: per pair, first entry of its Gram matrix in H
+  float4* H;                          // FP32 and mixed modes: leaf Gram matrices (see GramArgs)
+  float4* L4;                         // and leaf Cholesky factors, pair at L4 + its Gram offset (FP32 complex, ld p)
+  // per pair, first entry of its Gram matrix: a leaf pair's in H, a non-leaf
+  // pair's (one per column segment, mp x mp each) in Hl, from its level's start
+  const int64_t* hoff[2];
+  float4* Hl;
   const int32_t* rank_ovr[2];         // per pair a rank replacing the truncation rule (< 0: the rule), or NULL
   int32_t max_sweeps;
   int32_t jacobi_tpp[5];              // per factor class: most threads per Jacobi column pair (TuneTable)
@@ -224,11 +227,22 @@ template <typename T>
 bool launch_pair_kernel(const PairArgs<T>* args_dev, const uint32_t* codes, int nblocks, int P, bool from_r,
                         cudaStream_t st, const int* count = nullptr, const uint64_t* segs = nullptr);
 
-// The leaf factorisation of the mixed modes: the pair kernel with steps 1
-// and 1b replaced by the pivoted Cholesky of the leaf's Gram matrix H
-// (launch_gram before it); leaves of at most 64 rows.
-bool launch_pair_kernel_gram(const PairArgs<float>* args_dev, const uint32_t* codes, int nblocks, int P,
-                             cudaStream_t st);
+// The factorisation from Gram matrices (FP32 and mixed modes, pairs of at most
+// kGramRows rows): the pair kernel with steps 1 and 1b replaced by the pivoted
+// Cholesky of H (launch_gram or launch_gram_i64 before it), then Jacobi, rank
+// and Q.  Non-leaf pairs (from_r): H summed over the pair's column segments;
+// count as for launch_pair_kernel.
+constexpr int kGramRows = 64;
+bool launch_pair_kernel_gram(const PairArgs<float>* args_dev, const uint32_t* codes, int nblocks, int P, bool from_r,
+                             cudaStream_t st, const int* count = nullptr);
+
+// H = A A^* from products of fixed-point integers on the integer pipe, FP32
+// mode's leaf pairs (codes) or a level's pairs by segments of kGramSegCols
+// columns (segs: code << 32 | segment; pairs above kGramRows rows are left to
+// the LQ launches).  P: most rows of the list.
+constexpr int kGramSegCols = 256;
+bool launch_gram_i64(const PairArgs<float>* args_dev, const uint32_t* codes, const uint64_t* segs, int n, int P,
+                     cudaStream_t st);
 
 // R = Q^* A for the pairs of a pair-kernel launch, after it, by tiles of 32
 // columns, tiles[i] = launch code << 32 | first column (P as for the pair

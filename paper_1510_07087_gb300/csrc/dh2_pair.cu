@@ -345,8 +345,9 @@ __device__ __forceinline__ Df df_shfl_xor(Df x, int o) {
 }
 
 // ---------------------------------------------------------------- 1'. pivoted Cholesky of a Gram matrix
-// H = A A^* of a leaf pair from the tensor-core Gram kernel (double-float,
-// column-major, ld mp = p rounded up to 8) is factored by left-looking
+// H = A A^* of a pair from the Gram kernels (double-float, column-major, ld mp =
+// p rounded up to 8; a non-leaf pair's as nparts matrices, one per column
+// segment, summed as they are read) is factored by left-looking
 // Cholesky with diagonal pivoting in double-float arithmetic:
 // H = L L^* + (Schur complement), stopping at the first K whose Schur
 // complement has trace E_K <= tau (= drop eps_l^2).  Since L L^* = A A^*, the
@@ -363,19 +364,22 @@ __device__ __forceinline__ Df df_shfl_xor(Df x, int o) {
 // Rows: LPR threads per row.
 template <typename T, int NT, int LPR>
 __device__ void gram_cholesky(const PairArgs<T>& a, int side, int pid, int p, int P, int row, int q,
-                              bool live, double tau, C2<T>* Lg, float4* Hs, float* dhi, float* dlo, int* piv,
-                              int* pcol, int& K, double& E_K) {
+                              bool live, double tau, const float4* Hin, int nparts, C2<T>* Lg, float4* Hs, float* dhi,
+                              float* dlo, int* piv, int* pcol, int& K, double& E_K) {
   const int tid = threadIdx.x, lane = tid & 31;
   const int mp = (p + 7) & ~7;
   DH2_PROF_T(t_h0);
-  const float4* Hin = a.H + a.hoff[side][pid];
   // the scale from the largest diagonal entry (warp 0), then H is read,
   // scaled (a power of two: exact) and stored in one pass that also fills the
   // Schur diagonal
   __shared__ int sh_se;
   if ((tid >> 5) == 0) {
     float hmax = 0.f;
-    for (int r = lane; r < p; r += 32) hmax = fmaxf(hmax, Hin[r + (int64_t)r * mp].x);
+    for (int r = lane; r < p; r += 32) {
+      float h = 0.f;
+      for (int s = 0; s < nparts; ++s) h += Hin[r + (int64_t)r * mp + (int64_t)s * mp * mp].x;
+      hmax = fmaxf(hmax, h);
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) hmax = fmaxf(hmax, __shfl_xor_sync(0xffffffffu, hmax, o));
     int eh = 0;
@@ -389,7 +393,12 @@ __device__ void gram_cholesky(const PairArgs<T>& a, int side, int pid, int p, in
 #pragma unroll 4
   for (int idx = tid; idx < p * p; idx += NT) {
     const int r = idx % p, c = idx / p;
-    const float4 h = __ldg(Hin + r + (int64_t)c * mp);
+    float4 h = __ldg(Hin + r + (int64_t)c * mp);
+    for (int s = 1; s < nparts; ++s) {
+      const float4 g = __ldg(Hin + r + (int64_t)c * mp + (int64_t)s * mp * mp);
+      const Df re = df_add(Df{h.x, h.y}, Df{g.x, g.y}), im = df_add(Df{h.z, h.w}, Df{g.z, g.w});
+      h = make_float4(re.hi, re.lo, im.hi, im.lo);
+    }
     const float4 hs = make_float4(h.x * sc, h.y * sc, h.z * sc, h.w * sc);
     Hs[r + c * P] = hs;
     if (r == c) {
@@ -526,21 +535,12 @@ __device__ void gram_cholesky(const PairArgs<T>& a, int side, int pid, int p, in
 #endif
 }
 
-// P_T: largest factor size of the instantiation (32, 48, 64 or 128 rows).
-// NT: threads per CTA: 4 per row of P_T for the leaf sizes (128, 192, 256),
-// 256 for P_T = 128.  Every thread holds 16 chunk entries, so the chunk is
+// P_T: largest factor size of the instantiation (32, 40, 48, 64 or 128 rows; FP32
+// pairs of at most kGramRows rows go by Gram matrices).  NT: threads per CTA: 4
+// per row of P_T up to 64 rows (128 to 256), 256 for P_T = 128.  Every thread holds 16 chunk entries, so the chunk is
 // 64 columns wide for the three leaf sizes.
 #ifndef DH2_PAIR_MINB
 #define DH2_PAIR_MINB 3  // CTAs per SM at 256 threads (FP32)
-#endif
-#ifndef DH2_PAIR_MINB192
-#define DH2_PAIR_MINB192 4  // at 192 threads
-#endif
-#ifndef DH2_PAIR_MINB160
-#define DH2_PAIR_MINB160 5  // at 160 threads
-#endif
-#ifndef DH2_PAIR_MINB128
-#define DH2_PAIR_MINB128 6  // at 128 threads
 #endif
 #ifndef DH2_LQT
 #define DH2_LQT 8  // threads per row in the streamed LQ (4 or 8)
@@ -1018,8 +1018,7 @@ __device__ __forceinline__ void jacobi_rank_q(const PairArgs<T>& a, int side, in
 // CTAs per SM of the pivoted Cholesky of a Gram matrix (pair_kernel with
 // GRAM): its shared memory is H alone (P x P double-float complex), so the
 // register file sets the limit for the classes up to 48 rows.  8 / 7 / 5 CTAs
-// (64 / 56 / 64 registers, no spills) against the 6 / 5 / 4 of the LQ pair
-// kernel: the Cholesky waits on a barrier per pivot step, and more pairs per
+// (64 / 56 / 64 registers, no spills) against 6 / 5 / 4: the Cholesky waits on a barrier per pivot step, and more pairs per
 // SM fill those waits (measured: factor phase 4.50 -> 4.19 ms at n = 32768)
 #ifndef DH2_GRAM_MINB128
 #define DH2_GRAM_MINB128 8
@@ -1040,10 +1039,7 @@ constexpr int gram_min_blocks() {
 // n = 8192, 128 threads: 2 CTAs 30.9 ms, 3 26.9, 4 25.8)
 template <int NT, typename T>
 constexpr int pair_min_blocks() {
-  return sizeof(T) == 4 ? (NT >= 256   ? DH2_PAIR_MINB
-                           : NT >= 192 ? DH2_PAIR_MINB192
-                           : NT >= 160 ? DH2_PAIR_MINB160
-                                       : DH2_PAIR_MINB128)
+  return sizeof(T) == 4 ? DH2_PAIR_MINB
                         : (NT >= 256 ? 1 : NT >= 160 ? 2 : 4);
 }
 
@@ -1060,7 +1056,7 @@ __global__ void __launch_bounds__(NT, (GRAM ? gram_min_blocks<NT>() : pair_min_b
   constexpr int C = LQT * E;         // chunk width (16 * NT / P_T)
   static_assert(LPR >= 1 && LPR <= 32 && S >= 1 && S * E == 16, "16 chunk entries per thread");
   constexpr int XTRA = GRAM ? 0 : C;  // columns after L: the staged chunk of A (none from a Gram matrix)
-  static_assert(!GRAM || (!FROM_R && sizeof(T) == 4), "Gram factors: FP32 leaf pairs");
+  static_assert(!GRAM || sizeof(T) == 4, "Gram factors: FP32");
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ C2<T> sh_v0[2];
   __shared__ T sh_tau[2];
@@ -1138,7 +1134,7 @@ __global__ void __launch_bounds__(NT, (GRAM ? gram_min_blocks<NT>() : pair_min_b
   // [L_1 ... L_S]): a segment CTA factors its columns; the pair's own CTA
   // then factors the segments' factors instead of Ghat_tc
   C2<T>* seg_out = nullptr;
-  if (FROM_R) {
+  if (FROM_R && !GRAM) {
     const int64_t so = a.seg_off[side] ? a.seg_off[side][pid] : -1;
     if (seg >= 0) {
       if (so < 0 || p > P || p > P_T || p == 0) return;  // reported by the pair's own CTA
@@ -1187,8 +1183,12 @@ __global__ void __launch_bounds__(NT, (GRAM ? gram_min_blocks<NT>() : pair_min_b
   double E_K = 0.0;  // energy left out of them
   long long t_b = 0;  // start of the Jacobi step (profile build)
   if constexpr (GRAM) {
-    gram_cholesky<T, NT, LPR>(a, side, pid, p, P, row, q, live, drop * a.eps2[lvl],
-                              reinterpret_cast<C2<T>*>(a.L4 + a.hoff[side][pid]), Hs, nu, dlo, piv, pcol, K, E_K);
+    // (a non-leaf pair's L goes over its first segment's H, read by then)
+    const float4* Hin = (FROM_R ? a.Hl : a.H) + a.hoff[side][pid];
+    gram_cholesky<T, NT, LPR>(a, side, pid, p, P, row, q, live, drop * a.eps2[lvl], Hin,
+                              FROM_R ? (N + kGramSegCols - 1) / kGramSegCols : 1,
+                              reinterpret_cast<C2<T>*>((FROM_R ? a.Hl : a.L4) + a.hoff[side][pid]), Hs, nu, dlo, piv,
+                              pcol, K, E_K);
 #if DH2_PROF_ON
     t_b = clock64();
 #endif
@@ -1612,7 +1612,7 @@ __global__ void __launch_bounds__(NT, (GRAM ? gram_min_blocks<NT>() : pair_min_b
     // L (columns < K) is in the factor buffer; a zero column pads it to
     // even width; K and E_K go to the singular-value record, and
     // gram_jacobi_kernel takes it from there
-    C2<T>* Lg = reinterpret_cast<C2<T>*>(a.L4 + a.hoff[side][pid]);
+    C2<T>* Lg = reinterpret_cast<C2<T>*>((FROM_R ? a.Hl : a.L4) + a.hoff[side][pid]);
     if (K & 1)
       for (int i = tid; i < p; i += NT) Lg[(int64_t)K * p + i] = czero<T>();
     if (tid == 0) {
@@ -1636,15 +1636,17 @@ __global__ void __launch_bounds__(NT, (GRAM ? gram_min_blocks<NT>() : pair_min_b
                             Lm + (int64_t)P * LDL, XTRA * LDL);
 }
 
-// Steps 2-4 of the leaf pairs of a mixed-mode launch list, after the
-// pivoted Cholesky of their Gram matrices (pair_kernel<..., GRAM>): L (p x K,
+// Steps 2-4 of the pairs of a launch list, after the pivoted Cholesky of their
+// Gram matrices (pair_kernel<..., GRAM>): L (p x K,
 // ld p, columns < K rounded up to even) from the factor buffer L4, K and E_K
 // from its singular-value record.  Only L is held in shared memory, so that
 // more pairs run side by side than in the Cholesky, whose shared memory holds
 // all of H.
-template <int P_T, int NT, int MINB>
+template <int P_T, int NT, int MINB, bool FROM_R>
 __global__ void __launch_bounds__(NT, MINB)
-    gram_jacobi_kernel(const PairArgs<float>* __restrict__ args, const uint32_t* __restrict__ codes, const int P) {
+    gram_jacobi_kernel(const PairArgs<float>* __restrict__ args, const uint32_t* __restrict__ codes, const int P,
+                       const int* __restrict__ count) {
+  if (FROM_R && (int)blockIdx.x >= *count) return;
   extern __shared__ __align__(16) unsigned char smem[];
   const int LDL = P + 1;
   C2<float>* Lm = reinterpret_cast<C2<float>*>(smem);
@@ -1658,7 +1660,7 @@ __global__ void __launch_bounds__(NT, MINB)
   const int side = (int)((code >> kCodeSideShift) & 1u);
   const int pid = (int)(code & kCodePairMask);
   if (!DH2_IN(pid, c_lim.npairs[side], 14, pid)) return;
-  const int p = a.m[side][pid];
+  const int p = FROM_R ? a.rank[side][a.son[side][2 * pid]] + a.rank[side][a.son[side][2 * pid + 1]] : a.m[side][pid];
   const int N = a.ncols[side][pid];
   if (p > P || p > P_T || p == 0 || N == 0) return;  // rank and record already written by the Cholesky launch
   int32_t* rank_out = a.rank[side] + pid;
@@ -1666,7 +1668,7 @@ __global__ void __launch_bounds__(NT, MINB)
   const int K = (int)sig_out[kSigValues];
   const double E_K = sig_out[kSigValues + 1];
   const int pe = K + (K & 1);
-  const C2<float>* Lg = reinterpret_cast<const C2<float>*>(a.L4 + a.hoff[side][pid]);
+  const C2<float>* Lg = reinterpret_cast<const C2<float>*>((FROM_R ? a.Hl : a.L4) + a.hoff[side][pid]);
   for (int i = tid; i < pe * p; i += NT) Lm[(i / p) * LDL + i % p] = Lg[i];
   __syncthreads();
   long long t_b = 0;
@@ -1675,6 +1677,249 @@ __global__ void __launch_bounds__(NT, MINB)
 #endif
   jacobi_rank_q<float, P_T, NT>(a, side, pid, p, LDL, K, E_K, a.kcap[side][pid], a.level[side][pid], Lm, sig2, ord,
                                 rank_out, sig_out, t_b, nullptr, 0);
+}
+
+// ---------------------------------------------------------------- 1''. Gram matrices in integers
+// H = A A^* of a pair (FROM_R: of one segment of kGramSegCols columns of a
+// non-leaf pair) for the pivoted Cholesky.  Squaring needs H to about twice FP32's
+// precision; a streamed LQ avoids the squaring, but runs p reflections, one
+// barrier chain each, per 64 columns.  Here each row of A is written in fixed
+// point, q = rint(a 2^(b - e)) with every |re|, |im| of the row below 2^e, and
+// the products are summed exactly in 64-bit integers (IMAD.WIDE, 32 lanes per
+// clock and SM: four per complex product, against 36 FP32 operations in
+// double-float and sixteen for the reflections of an LQ).  b: the sum of N
+// columns stays below 2^62; 27 bits up to 128 columns, 26 to 512, 25 to 2048: a
+// backward error of 2^-(b+1) of each row's largest entry, below FP32's own
+// rounding of the LQ.  A chunk of 64 columns that raises a row's e shifts the sums
+// it enters (their dropped bits lie below the new resolution).
+// Threads: 4 x 4 tiles of the lower triangle, the columns of a chunk dealt to
+// G = NT / tiles threads per tile, summed at the end.
+// n = 8192, eps 1e-6, FP32 (leaf factors): streamed LQ with its Jacobi 2.32 ms;
+// this 0.58 ms, Cholesky 0.32, Jacobi 0.60 (with divisions in the staging and no
+// prefetch 1.12 ms).  Bound by issue: staging, scan and conversion, ~250 per 32
+// entries; the integer products are a fifth of it.  Singular values lie half as
+// far from FP64's as the LQ's (mean 2.3e-7 against 4.1e-7 of the largest).
+__host__ __device__ constexpr int gram_i64_ld(int p) {  // rows in fours, an odd number of them: staging by columns spreads over the banks
+  return ((p + 3) / 4 | 1) * 4;
+}
+constexpr int kGramI64Chunk = 64;
+template <bool FROM_R, int NT>
+__global__ void __launch_bounds__(NT, NT <= 128 ? 4 : 3)
+    gram_i64_kernel(const PairArgs<float>* __restrict__ args, const uint32_t* __restrict__ codes,
+                    const uint64_t* __restrict__ segs, const int P) {
+  constexpr int CW = kGramI64Chunk, NW = NT / 32;
+  extern __shared__ __align__(16) unsigned char smem[];
+  // two chunks, column jj from jj * LD: A's stored entries as float2, then q in place
+  int2* const buf = reinterpret_cast<int2*>(smem);
+  __shared__ int rexp[kGramRows], rdel[kGramRows], rmax[kGramRows];
+  __shared__ int cgc[2][CW];
+  __shared__ float cwt[2][CW];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t code = FROM_R ? (uint32_t)(segs[blockIdx.x] >> 32) : codes[blockIdx.x];
+  const int seg = FROM_R ? (int)(uint32_t)segs[blockIdx.x] : 0;
+  const int side = (int)((code >> kCodeSideShift) & 1u);
+  const int pid = (int)(code & kCodePairMask);
+  const PairArgs<float>& a = args[code >> kCodeProbShift];
+  if (!DH2_IN(pid, c_lim.npairs[side], 9, pid)) return;
+  int N = a.ncols[side][pid];
+  Source<float, FROM_R> src;
+  src.side = side;
+  src.pid = pid;
+  int p;
+  if constexpr (FROM_R) {
+    const int s0 = a.son[side][2 * pid], s1 = a.son[side][2 * pid + 1];
+    if (!DH2_IN(s0, c_lim.npairs[side], 12, pid) || !DH2_IN(s1, c_lim.npairs[side], 13, pid)) return;
+    src.k1 = a.rank[side][s0];
+    p = src.k1 + a.rank[side][s1];
+    src.off0 = a.sonoff[side][2 * pid] + seg * kGramSegCols;
+    src.off1 = a.sonoff[side][2 * pid + 1] + seg * kGramSegCols;
+    src.ld0 = a.kcap[side][s0];
+    src.ld1 = a.kcap[side][s1];
+    src.roff0 = a.Roff[side][s0];
+    src.roff1 = a.Roff[side][s1];
+    src.R0 = a.R[side] + src.roff0;
+    src.R1 = a.R[side] + src.roff1;
+    N = min(kGramSegCols, N - seg * kGramSegCols);
+  } else {
+    p = a.m[side][pid];
+    src.r0 = a.start[side][pid];
+    src.cmo = a.cmoff[side][pid];
+    src.gcol = a.gcol[side] + src.cmo;
+    src.colw = a.colw[side] + src.cmo;
+    src.G = a.G;
+    src.ld = a.ld;
+    src.entry = a.entry;
+    src.gen = a.gen;
+  }
+  if (p > P || p > kGramRows || p == 0 || N <= 0) return;  // p > kGramRows: an LQ launch's (FROM_R), or reported by the factor launch
+  const int mp = (p + 7) & ~7;
+  float4* Hout = (FROM_R ? a.Hl + (int64_t)seg * mp * mp : a.H) + a.hoff[side][pid];
+  const int LD = gram_i64_ld(p), nt = (p + 3) >> 2, ntile = nt * (nt + 1) / 2;
+  const int G = NT / ntile, grp = tid / ntile;  // column groups (ntile <= NT)
+  int ti, tj;                                   // this thread's tile, ti >= tj
+  {
+    const int t = tid % ntile;
+    ti = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
+    while (ti * (ti + 1) / 2 > t) --ti;
+    while ((ti + 1) * (ti + 2) / 2 <= t) ++ti;
+    tj = t - ti * (ti + 1) / 2;
+  }
+  const int lg = 32 - __clz(N - 1 | 1);  // N <= 2^lg
+  const int b = min(27, (61 - lg) >> 1);  // (27: 2^(b - e) stays finite)
+  long long ar[4][4], ai[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) ar[i][j] = ai[i][j] = 0;
+  if (tid < kGramRows) rexp[tid] = -1000;
+  for (int i = tid; i < 2 * CW * (LD - p); i += NT) buf[(i / (LD - p)) * LD + p + i % (LD - p)] = make_int2(0, 0);
+  bool bad = false;
+  const int RG = (p + 31) >> 5;            // 32-row groups
+  const int r = (warp % RG) * 32 + lane;   // the row this thread scans and converts
+  const int c0 = warp / RG, cs = NW / RG;  // its columns c0, c0 + cs, ... (warps past cs * RG idle)
+  const bool scan = r < p && c0 < cs;
+  const bool gen = !FROM_R && src.gen;
+  const bool down = FROM_R || side == 0;  // consecutive threads on the contiguous direction
+  // the column table of a chunk, and its entries: by cp.async, under the
+  // products of the chunk before; generated ones are computed (with their weight)
+  auto table = [&](int j0, int s) {
+    if (!FROM_R && tid < min(CW, N - j0)) src.colinfo(j0 + tid, cgc[s][tid], cwt[s][tid]);
+  };
+  auto entries = [&](int j0, int s) {
+    const int cw = min(CW, N - j0);
+    C2<float>* X = reinterpret_cast<C2<float>*>(buf + s * CW * LD);
+    for (Walk2 it(tid, NT, down ? p : cw); it.g < (down ? cw : p); it.next()) {
+      const int rr = down ? it.f : it.g, jj = down ? it.g : it.f;
+      C2<float>* o = X + jj * LD + rr;
+      if (gen) {
+        *o = src.leaf_at(rr, cgc[s][jj], 1.f);
+      } else {
+        const C2<float>* g = FROM_R ? src.sons_ptr(rr, j0 + jj) : src.leaf_ptr(rr, cgc[s][jj]);
+        if (g) cp_async<sizeof(C2<float>)>(o, g);
+        else *o = czero<float>();
+      }
+    }
+    cp_async_commit();
+  };
+  table(0, 0);
+  __syncthreads();
+  entries(0, 0);
+  for (int j0 = 0, s = 0; j0 < N; j0 += CW, s ^= 1) {
+    const int cw = min(CW, N - j0);
+    const bool more = j0 + CW < N;
+    int2* Xs = buf + s * CW * LD;
+    if (tid < kGramRows) rmax[tid] = 0;
+    if (more) table(j0 + CW, s ^ 1);
+    cp_async_wait_all();
+    __syncthreads();  // this chunk has landed; the other buffer's products are done
+    if (more && !gen) entries(j0 + CW, s ^ 1);
+    if (scan) {
+      int m = 0;  // largest |re|, |im| as bits (NaN and infinity above every finite value)
+      for (int j = c0; j < cw; j += cs) {
+        const int2 v = Xs[j * LD + r];
+        const float w = FROM_R ? 1.f : cwt[s][j];
+        m = max(m, max(__float_as_int(__int_as_float(v.x) * w) & 0x7fffffff,
+                       __float_as_int(__int_as_float(v.y) * w) & 0x7fffffff));
+      }
+      bad |= m >= 0x7f800000;
+      atomicMax(&rmax[r], min(m, 0x7f7fffff));
+    }
+    __syncthreads();
+    bool moved = false;
+    if (tid < p) {
+      // below 2^e; rows below 2^-100 are zero to FP32's products anyway
+      const int e = max((rmax[tid] >> 23) - 126, -100), old = rexp[tid];
+      rdel[tid] = j0 > 0 && e > old ? e - old : 0;
+      moved = rdel[tid] > 0;
+      rexp[tid] = max(e, old);
+    }
+    moved = __syncthreads_or(moved);
+    if (scan) {
+      const float sc = __int_as_float((b - rexp[r] + 127) << 23);  // b - e in [-101, 127]
+      // (a product with 2^(b - e) is exact: the order of the factors leaves q the same)
+      const float cj = !FROM_R && side == 1 && !gen ? -1.f : 1.f;  // A = G^* (generated entries: already conjugated)
+      for (int j = c0; j < cw; j += cs) {
+        const int2 v = Xs[j * LD + r];
+        const float w = FROM_R ? 1.f : cwt[s][j];
+        Xs[j * LD + r] = make_int2(__float2int_rn(__int_as_float(v.x) * w * sc),
+                                   __float2int_rn(__int_as_float(v.y) * w * sc * cj));
+      }
+    }
+    if (moved && grp < G) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int sh = min(63, (4 * ti + i < p ? rdel[4 * ti + i] : 0) + (4 * tj + j < p ? rdel[4 * tj + j] : 0));
+          ar[i][j] >>= sh;
+          ai[i][j] >>= sh;
+        }
+    }
+    __syncthreads();
+    if (grp < G)
+      for (int jj = grp; jj < cw; jj += G) {
+        const int4* xp = reinterpret_cast<const int4*>(Xs + jj * LD + 4 * ti);
+        const int4* yp = reinterpret_cast<const int4*>(Xs + jj * LD + 4 * tj);
+        const int4 x01 = xp[0], x23 = xp[1], y01 = yp[0], y23 = yp[1];
+        const int xr[4] = {x01.x, x01.z, x23.x, x23.z}, xi[4] = {x01.y, x01.w, x23.y, x23.w};
+        const int yr[4] = {y01.x, y01.z, y23.x, y23.z}, yi[4] = {y01.y, y01.w, y23.y, y23.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int nr = -xr[i];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {  // x conj(y)
+            ar[i][j] += (long long)xr[i] * yr[j];
+            ai[i][j] += (long long)xi[i] * yr[j];
+            ar[i][j] += (long long)xi[i] * yi[j];
+            ai[i][j] += (long long)nr * yi[j];
+          }
+        }
+      }
+    if (more && gen) entries(j0 + CW, s ^ 1);
+  }
+  // the groups' sums, through the staging buffer (16 entries per tile)
+  longlong2* red = reinterpret_cast<longlong2*>(smem);
+  for (int g = 1; g < G; ++g) {
+    __syncthreads();
+    if (grp == g)
+#pragma unroll
+      for (int u = 0; u < 16; ++u) red[u * ntile + tid % ntile] = make_longlong2(ar[u >> 2][u & 3], ai[u >> 2][u & 3]);
+    __syncthreads();
+    if (grp == 0)
+#pragma unroll
+      for (int u = 0; u < 16; ++u) {
+        const longlong2 v = red[u * ntile + tid];
+        ar[u >> 2][u & 3] += v.x;
+        ai[u >> 2][u & 3] += v.y;
+      }
+  }
+  if (__syncthreads_or(bad)) {  // non-finite entries: reported, H zero
+    if (tid == 0) atomicOr(a.status, kStatusNaN);
+    for (int i = tid; i < mp * mp; i += NT) Hout[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    return;
+  }
+  if (grp == 0) {
+    auto to_df = [](long long v, int ex) {
+      const float hi = __ll2float_rn(v);
+      const float lo = __ll2float_rn(v - __float2ll_rn(hi));
+      // 2^ex in two factors (either may lie outside the normal range alone)
+      const int h = ex >> 1;
+      const float s0 = __int_as_float((h + 127) << 23), s1 = __int_as_float((ex - h + 127) << 23);
+      return make_float2(hi * s0 * s1, lo * s0 * s1);
+    };
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int rr = 4 * ti + i, cc = 4 * tj + j;
+        if (rr < p && cc <= rr) {
+          const int ex = rexp[rr] + rexp[cc] - 2 * b;
+          const float2 re = to_df(ar[i][j], ex), im = to_df(ai[i][j], ex);
+          Hout[rr + (int64_t)cc * mp] = make_float4(re.x, re.y, im.x, im.y);
+          if (cc != rr) Hout[cc + (int64_t)rr * mp] = make_float4(re.x, re.y, -im.x, -im.y);
+        }
+      }
+  }
 }
 
 // R_tc = Q^* A for the pairs of one launch (Section 6, R recursion: R_tc =
@@ -2188,55 +2433,90 @@ template <typename T>
 bool launch_pair_kernel(const PairArgs<T>* args, const uint32_t* codes, int nblocks, int P, bool from_r,
                         cudaStream_t st, const int* count, const uint64_t* segs) {
   if (nblocks <= 0) return true;
-  if (!from_r) {
-    if (P <= 32) return launch_one<T, 32, false, 128>(args, codes, nblocks, P, st, count);
-    if (P <= 40) return launch_one<T, 40, false, 160>(args, codes, nblocks, P, st, count);
-    if (P <= 48) return launch_one<T, 48, false, 192>(args, codes, nblocks, P, st, count);
-    if (P <= 64) return launch_one<T, 64, false, 256>(args, codes, nblocks, P, st, count);
-    return launch_one<T, 128, false, 256>(args, codes, nblocks, P, st, count);
+  // FP32 pairs of at most kGramRows rows are factored from Gram matrices
+  if constexpr (sizeof(T) == 8) {
+    if (!from_r) {
+      if (P <= 32) return launch_one<T, 32, false, 128>(args, codes, nblocks, P, st, count);
+      if (P <= 40) return launch_one<T, 40, false, 160>(args, codes, nblocks, P, st, count);
+      if (P <= 48) return launch_one<T, 48, false, 192>(args, codes, nblocks, P, st, count);
+      if (P <= 64) return launch_one<T, 64, false, 256>(args, codes, nblocks, P, st, count);
+    } else {
+      if (P <= 32) return launch_one<T, 32, true, 128>(args, codes, nblocks, P, st, count, segs);
+      if (P <= 48) return launch_one<T, 48, true, 192>(args, codes, nblocks, P, st, count, segs);
+      if (P <= 64) return launch_one<T, 64, true, 256>(args, codes, nblocks, P, st, count, segs);
+    }
   }
-  if (P <= 32) return launch_one<T, 32, true, 128>(args, codes, nblocks, P, st, count, segs);
-  if (P <= 48) return launch_one<T, 48, true, 192>(args, codes, nblocks, P, st, count, segs);
-  if (P <= 64) return launch_one<T, 64, true, 256>(args, codes, nblocks, P, st, count, segs);
+  if (!from_r) return launch_one<T, 128, false, 256>(args, codes, nblocks, P, st, count);
   return launch_one<T, 128, true, 256>(args, codes, nblocks, P, st, count, segs);
+}
+
+template <bool FROM_R, int NT>
+bool launch_i64(const PairArgs<float>* args, const uint32_t* codes, const uint64_t* segs, int n, int P,
+                cudaStream_t st) {
+  auto kern = gram_i64_kernel<FROM_R, NT>;
+  const size_t smem = 2 * (size_t)kGramI64Chunk * gram_i64_ld(P) * sizeof(int2);
+  if (!set_smem(kern, smem)) return false;
+  kern<<<n, NT, smem, st>>>(args, codes, segs, P);
+  return true;
+}
+bool launch_gram_i64(const PairArgs<float>* args, const uint32_t* codes, const uint64_t* segs, int n, int P,
+                     cudaStream_t st) {
+  if (n <= 0) return true;
+  P = std::min(P, kGramRows);
+  // 55 tiles at 40 rows fill 110 of 128 threads; 78 at 48 rows 156 of 160, 136 at 64
+  if (P <= 40) return segs ? launch_i64<true, 128>(args, codes, segs, n, P, st) : launch_i64<false, 128>(args, codes, segs, n, P, st);
+  return segs ? launch_i64<true, 160>(args, codes, segs, n, P, st) : launch_i64<false, 160>(args, codes, segs, n, P, st);
 }
 
 // The Jacobi launch of a class: NT = 4 x rows threads per CTA, or (the
 // tuning table's narrow choices) NTN, a multiple of 32 near 2 x rows, or NTM
 // near 1 x rows, with the same threads per SM (about twice or four times the
-// CTAs, so more pairs at once; at most 32 CTAs per SM).
-template <int P_T, int NT, int NTN, int NTM>
-bool launch_gram_factor(const PairArgs<float>* args, const uint32_t* codes, int nblocks, int P, cudaStream_t st) {
+// CTAs, so more pairs at once; at most 32 CTAs per SM).  A level's pairs are few:
+// 4 x rows.
+template <int P_T, int NT, int NTN, int NTM, bool FROM_R>
+bool launch_gram_factor(const PairArgs<float>* args, const uint32_t* codes, int nblocks, int P, cudaStream_t st,
+                        const int* count) {
   static_assert(NT % 32 == 0 && NTN % 32 == 0 && NTM % 32 == 0 && NTM >= P_T,
                 "whole warps (the Jacobi reductions run converged), one thread per column of the rank step");
-  if (!launch_one<float, P_T, false, NT, true>(args, codes, nblocks, P, st)) return false;
+  if (!launch_one<float, P_T, FROM_R, NT, true>(args, codes, nblocks, P, st, count)) return false;
   const size_t smem = (((size_t)P * (P + 1) * sizeof(C2<float>) + 15) & ~(size_t)15) + (size_t)P * sizeof(double) +
                       (size_t)P * sizeof(int);
   constexpr int MINB = 2048 / NT - 4;
-  const int narrow = tune_current().jacobi_narrow[factor_class(P_T)];
-  if (narrow == 2) {
-    constexpr int MB = NT * MINB / NTM < 32 ? NT * MINB / NTM : 32;
-    auto kern = gram_jacobi_kernel<P_T, NTM, MB>;
-    if (!set_smem(kern, smem)) return false;
-    kern<<<nblocks, NTM, smem, st>>>(args, codes, P);
-  } else if (narrow == 1) {
-    auto kern = gram_jacobi_kernel<P_T, NTN, NT * MINB / NTN>;
-    if (!set_smem(kern, smem)) return false;
-    kern<<<nblocks, NTN, smem, st>>>(args, codes, P);
-  } else {
-    auto kern = gram_jacobi_kernel<P_T, NT, MINB>;
-    if (!set_smem(kern, smem)) return false;
-    kern<<<nblocks, NT, smem, st>>>(args, codes, P);
+  const int narrow = FROM_R ? 0 : tune_current().jacobi_narrow[factor_class(P_T)];
+  if constexpr (!FROM_R) {
+    if (narrow == 2) {
+      constexpr int MB = NT * MINB / NTM < 32 ? NT * MINB / NTM : 32;
+      auto kern = gram_jacobi_kernel<P_T, NTM, MB, false>;
+      if (!set_smem(kern, smem)) return false;
+      kern<<<nblocks, NTM, smem, st>>>(args, codes, P, count);
+      return true;
+    }
+    if (narrow == 1) {
+      auto kern = gram_jacobi_kernel<P_T, NTN, NT * MINB / NTN, false>;
+      if (!set_smem(kern, smem)) return false;
+      kern<<<nblocks, NTN, smem, st>>>(args, codes, P, count);
+      return true;
+    }
   }
+  auto kern = gram_jacobi_kernel<P_T, NT, MINB, FROM_R>;
+  if (!set_smem(kern, smem)) return false;
+  kern<<<nblocks, NT, smem, st>>>(args, codes, P, count);
   return true;
 }
 
-bool launch_pair_kernel_gram(const PairArgs<float>* args, const uint32_t* codes, int nblocks, int P, cudaStream_t st) {
+bool launch_pair_kernel_gram(const PairArgs<float>* args, const uint32_t* codes, int nblocks, int P, bool from_r,
+                             cudaStream_t st, const int* count) {
   if (nblocks <= 0) return true;
-  if (P <= 32) return launch_gram_factor<32, 128, 64, 32>(args, codes, nblocks, P, st);
-  if (P <= 40) return launch_gram_factor<40, 160, 96, 64>(args, codes, nblocks, P, st);
-  if (P <= 48) return launch_gram_factor<48, 192, 96, 64>(args, codes, nblocks, P, st);
-  if (P <= 64) return launch_gram_factor<64, 256, 128, 64>(args, codes, nblocks, P, st);
+  if (from_r) {
+    if (P <= 32) return launch_gram_factor<32, 128, 64, 32, true>(args, codes, nblocks, P, st, count);
+    if (P <= 48) return launch_gram_factor<48, 192, 96, 64, true>(args, codes, nblocks, P, st, count);
+    if (P <= 64) return launch_gram_factor<64, 256, 128, 64, true>(args, codes, nblocks, P, st, count);
+    return false;
+  }
+  if (P <= 32) return launch_gram_factor<32, 128, 64, 32, false>(args, codes, nblocks, P, st, count);
+  if (P <= 40) return launch_gram_factor<40, 160, 96, 64, false>(args, codes, nblocks, P, st, count);
+  if (P <= 48) return launch_gram_factor<48, 192, 96, 64, false>(args, codes, nblocks, P, st, count);
+  if (P <= 64) return launch_gram_factor<64, 256, 128, 64, false>(args, codes, nblocks, P, st, count);
   return false;
 }
 
