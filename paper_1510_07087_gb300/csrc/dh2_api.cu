@@ -132,7 +132,10 @@ struct Tree::Dev {
   int64_t leaf_tile_class_begin[kLeafClasses + 1] = {};  // leaf tiles of each size class
   std::vector<int64_t> nl_tile_begin, nl_tile_count;    // per level
   std::vector<int32_t> nl_rowcap_max;                   // per level
-  std::vector<int64_t> lvl_begin[2], lvl_nl_begin[2], lvl_end[2];
+  std::vector<int64_t> lvl_nl_begin[2], lvl_end[2];
+  // per level the pairs that have father pairs (backward transformation)
+  int32_t* son_list[2];
+  std::vector<int64_t> lvl_son_begin[2], lvl_son_end[2];
   int32_t max_leaf = 0;
   std::vector<int32_t> kcap_h[2], rowcap_h[2];
   std::vector<int64_t> Qoff_h[2], Soff_h;
@@ -343,7 +346,6 @@ dh2_status upload_tree(Tree& tr) {
     D->nleaf[sd] = (int64_t)S.leaf_pairs.size();
     std::vector<int32_t> ll(S.leaf_pairs.begin(), S.leaf_pairs.end());
     // level ranges
-    D->lvl_begin[sd].assign(tr.depth + 1, 0);
     D->lvl_nl_begin[sd].assign(tr.depth + 1, 0);
     D->lvl_end[sd].assign(tr.depth + 1, 0);
     for (int l = 0; l <= tr.depth; ++l) {
@@ -356,10 +358,18 @@ dh2_status upload_tree(Tree& tr) {
         }
       if (b < 0) b = e = nb = 0;
       if (nb < 0) nb = e;
-      D->lvl_begin[sd][l] = b;
       D->lvl_nl_begin[sd][l] = nb;
       D->lvl_end[sd][l] = e;
     }
+    std::vector<int32_t> sl;
+    D->lvl_son_begin[sd].assign(tr.depth + 1, 0);
+    D->lvl_son_end[sd].assign(tr.depth + 1, 0);
+    for (int64_t p = 0; p < np; ++p) {  // levels are contiguous ranges
+      if (p == 0 || S.pairs[p].level != S.pairs[p - 1].level) D->lvl_son_begin[sd][S.pairs[p].level] = (int64_t)sl.size();
+      if (!S.pairs[p].parents.empty()) sl.push_back((int32_t)p);
+      D->lvl_son_end[sd][S.pairs[p].level] = (int64_t)sl.size();
+    }
+    add32(std::move(sl), &D->son_list[sd]);
     add32(std::move(cl), &D->cluster[sd]);
     add32(std::move(lf), &D->leaf[sd]);
     add32(std::move(st), &D->start[sd]);
@@ -2452,13 +2462,68 @@ void dh2_matrix_free(dh2_matrix* M) { matrix_release(M); }
 
 namespace {
 
+// A second stream for the nearfield product beside the transformations, with
+// its fork and join events: taken from a small pool for the time of one call's
+// launches (two threads never enqueue on one at a time), at most kSideStreams
+// per device, kept until the process ends.  Work of an earlier call still
+// running on it only delays this call's.
+constexpr int kSideStreams = 8;
+struct SideStream {
+  cudaStream_t st = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr;
+};
+std::mutex g_side_mu;
+std::vector<SideStream> g_side_idle[64];
+int g_side_made[64] = {};
+class SideLease {
+ public:
+  explicit SideLease(int dev) : dev_(dev) {
+    if (dev < 0 || dev >= 64) return;
+    std::lock_guard<std::mutex> lk(g_side_mu);
+    if (!g_side_idle[dev].empty()) {
+      s_ = g_side_idle[dev].back();
+      g_side_idle[dev].pop_back();
+    } else if (g_side_made[dev] < kSideStreams) {
+      SideStream s;
+      if (cudaStreamCreateWithFlags(&s.st, cudaStreamNonBlocking) == cudaSuccess &&
+          cudaEventCreateWithFlags(&s.fork, cudaEventDisableTiming) == cudaSuccess &&
+          cudaEventCreateWithFlags(&s.join, cudaEventDisableTiming) == cudaSuccess) {
+        g_side_idle[dev].reserve(kSideStreams);  // giving it back cannot throw
+        ++g_side_made[dev];
+        s_ = s;
+      } else {
+        cudaGetLastError();
+        if (s.fork) cudaEventDestroy(s.fork);
+        if (s.st) cudaStreamDestroy(s.st);
+      }
+    }
+  }
+  ~SideLease() {
+    if (!s_.st) return;
+    std::lock_guard<std::mutex> lk(g_side_mu);
+    g_side_idle[dev_].push_back(s_);
+  }
+  SideLease(const SideLease&) = delete;
+  SideLease& operator=(const SideLease&) = delete;
+  const SideStream& get() const { return s_; }
+
+ private:
+  int dev_;
+  SideStream s_;
+};
+// nearfield entries from which the fork and join (about 6 us) pay: the product's
+// other kernels, ~20 us and more there, are bound by latency and leave HBM idle,
+// and the nearfield leaves them registers and threads.  n = 32768, one vector: 1224 -> 1158
+// us; n = 12289, adjoint, three vectors: 411 -> 367 us
+constexpr int64_t kOverlapElems = int64_t(1) << 23;
+
 // The launches of y = G~ x (adj = 0: forward transformation on W, coupling
 // with S_b, backward on V, nearfield) or y = G~^* x (adj = 1: the sides
 // exchanged, S_b^* and G_b^*), with the coefficient vectors in buf (hx bytes
 // for x's, then y's).  Every coefficient is written before it is read.
 template <typename T>
 dh2_status matvec_launches(const dh2_matrix* M, int adj, const void* xv, void* yv, int nrhs, void* buf, size_t hx,
-                           cudaStream_t st) {
+                           bool may_overlap, cudaStream_t st) {
   Tree& tr = M->tree->tr;
   Tree::Dev* D = tr.dev;
   const int64_t n = tr.n;
@@ -2469,11 +2534,6 @@ dh2_status matvec_launches(const dh2_matrix* M, int adj, const void* xv, void* y
   C2<T>* y = (C2<T>*)yv;
   DH2_CUDA_TRY(cudaMemsetAsync(y, 0, sizeof(C2<T>) * n * nrhs, st));
   const SideView<T> Vin = side_view<T>(tr, M, si);
-  launch_mv_forward_leaf<T>(Vin, D->leaf_list[si], (int)D->nleaf[si], x, nrhs, n, xh, D->hoff[si], st);
-  for (int l = tr.depth; l >= 0; --l) {
-    const int64_t b = D->lvl_nl_begin[si][l], e = D->lvl_end[si][l];
-    if (e > b) launch_mv_forward_up<T>(Vin, D->iota[si] + b, (int)(e - b), nrhs, xh, D->hoff[si], st);
-  }
   MvArgs<T> a;
   a.V = side_view<T>(tr, M, so);
   a.W = Vin;
@@ -2493,15 +2553,41 @@ dh2_status matvec_launches(const dh2_matrix* M, int adj, const void* xv, void* y
   a.near = (const C2<T>*)M->near;
   a.G = (const C2<T>*)M->G;
   a.ld = M->ld;
+  // the nearfield on a second stream, beside the transformations (not in a
+  // caller's capture: the pool's streams would join it)
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (may_overlap && (D->near_elems < kOverlapElems || D->nadm == 0 ||
+                      cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)) {
+    cudaGetLastError();
+    may_overlap = false;
+  }
+  SideLease lease(may_overlap ? M->device : -1);
+  const SideStream& side = lease.get();
+  bool forked = false;
+  if (side.st) {
+    forked = cudaEventRecord(side.fork, st) == cudaSuccess && cudaStreamWaitEvent(side.st, side.fork, 0) == cudaSuccess;
+    if (forked) {
+      launch_mv_near<T>(a, adj != 0, nrhs, x, y, n, side.st);
+      DH2_CUDA_TRY(cudaEventRecord(side.join, side.st));
+    } else {
+      cudaGetLastError();
+    }
+  }
+  launch_mv_forward_leaf<T>(Vin, D->leaf_list[si], (int)D->nleaf[si], x, nrhs, n, xh, D->hoff[si], st);
+  for (int l = tr.depth; l >= 0; --l) {
+    const int64_t b = D->lvl_nl_begin[si][l], e = D->lvl_end[si][l];
+    if (e > b) launch_mv_forward_up<T>(Vin, D->iota[si] + b, (int)(e - b), nrhs, xh, D->hoff[si], st);
+  }
   if (adj) launch_mv_coupling_adj<T>(a, (int)D->npairs[so], nrhs, st);
   else launch_mv_coupling<T>(a, (int)D->npairs[so], nrhs, st);
   // backward transformation, top-down
   for (int l = 1; l <= tr.depth; ++l) {
-    const int64_t b = D->lvl_begin[so][l], e = D->lvl_end[so][l];
-    if (e > b) launch_mv_backward_down<T>(a, D->iota[so] + b, (int)(e - b), nrhs, st);
+    const int64_t b = D->lvl_son_begin[so][l], e = D->lvl_son_end[so][l];
+    if (e > b) launch_mv_backward_down<T>(a, D->son_list[so] + b, (int)(e - b), nrhs, st);
   }
   launch_mv_backward_leaf<T>(a, D->leaf_list[so], D->leaf_units[so], D->nleaf_units[so], nrhs, y, n, st);
-  launch_mv_near<T>(a, adj != 0, nrhs, x, y, n, st);
+  if (forked) DH2_CUDA_TRY(cudaStreamWaitEvent(st, side.join, 0));
+  else launch_mv_near<T>(a, adj != 0, nrhs, x, y, n, st);
   DH2_CUDA_TRY(cudaGetLastError());
   return DH2_OK;
 }
@@ -2516,7 +2602,7 @@ dh2_status run_matvec(const dh2_matrix* M, int adj, const void* x, void* y, int 
     cudaGetLastError();
     return DH2_ENOMEM;
   }
-  const dh2_status s = matvec_launches<T>(M, adj, x, y, nrhs, buf, hx, st);
+  const dh2_status s = matvec_launches<T>(M, adj, x, y, nrhs, buf, hx, true, st);
   cudaFreeAsync(buf, st);
   return s;
 }
@@ -2931,7 +3017,7 @@ dh2_status run_matvec_noalloc(const dh2_matrix* M, const void* xv, void* yv, int
     const dh2_status s = noalloc_scratch_address(dev, &buf);
     if (s != DH2_OK) return s;
   }
-  return matvec_launches<T>(M, 0, xv, yv, nrhs, buf, hx, st);
+  return matvec_launches<T>(M, 0, xv, yv, nrhs, buf, hx, false, st);  // (a second stream would be made by the runtime's allocator)
 }
 
 }  // namespace

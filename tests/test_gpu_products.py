@@ -62,3 +62,46 @@ def test_products_by_columns(fp64, view, n, kappa, leaf, kernel):
     for j in range(9):
         a, b = np.vdot(zs[:, j], y[:, j]), np.vdot(t[:, j], xs[:, j])
         assert abs(a - b) <= 10 * tol * gn * np.linalg.norm(xs[:, j]) * np.linalg.norm(zs[:, j])
+
+
+def test_products_on_several_streams_and_threads():
+    """The nearfield runs on a second stream beside the transformations (n large enough): products of
+    one matrix from several threads, each on a stream of its own, and the use of x and y right after
+    the call on the caller's stream give the product of a lone call (bounds as above)."""
+    import threading
+
+    D = dev()
+    n, kappa = 4200, 6.0
+    pts = random_ellipsoid(n)
+    T = D.dh2_tree_build(pts, 32, kappa)
+    perm = T.perm()
+    G = helmholtz_matrix(pts, kappa)[np.ix_(perm, perm)].astype(np.complex64)
+    assert (1.0 - T.stats().adm_fraction) * n * n > 2 ** 23
+    M = D.dh2_compress(T, colmajor(G, torch.complex64), eps=1e-4)
+    xs = torch.randn((8, n), dtype=torch.complex64, device="cuda")
+    want = torch.empty_like(xs)
+    for i in range(8):
+        D.dh2_matvec(M, xs[i], want[i])
+    torch.cuda.synchronize()
+    got = torch.zeros((8, 20, n), dtype=torch.complex64, device="cuda")
+    torch.cuda.synchronize()
+
+    def work(i):
+        st = torch.cuda.Stream()
+        with torch.cuda.stream(st):
+            for k in range(20):
+                x = xs[i] * 2.0  # made and dropped on this stream
+                y = torch.empty_like(x)
+                D.dh2_matvec(M, x, y)
+                x.zero_()
+                got[i, k] = 0.5 * y
+
+    ts = [threading.Thread(target=work, args=(i,)) for i in range(8)]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    torch.cuda.synchronize()
+    for i in range(8):
+        d = (got[i] - want[i]).norm(dim=1)
+        assert float(d.max()) <= 1e-5 * float(want[i].norm())
