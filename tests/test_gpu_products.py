@@ -71,7 +71,7 @@ def test_products_on_several_streams_and_threads():
     import threading
 
     D = dev()
-    n, kappa = 4200, 6.0
+    n, kappa = 4200, 12.0
     pts = random_ellipsoid(n)
     T = D.dh2_tree_build(pts, 32, kappa)
     perm = T.perm()
