@@ -228,14 +228,14 @@ cudaError_t dev_malloc_async(void** p, size_t bytes, cudaStream_t st) {
 // from each cluster's number of inadmissible blocks and their extent in the
 // other dimension; the device writes the lists (NearFill).  A
 // unit holds about `target` entries: at most kNearUnitMax, so that its sums pay
-// for their atomic additions, and few enough that a small matrix still gives
-// every SM tens of units (n = 8192 in FP64, eight vectors: 3.1 ms with half
-// as many, 2.95 so).
+// for their atomic additions, and so that a small matrix still gives every SM
+// some twelve of them (three waves; FP64 n = 4096, one vector: 6 per SM 193 us, 12
+// 172, 32 181; complex64 n = 4500: 47.1, 47.4, 51.1).
 constexpr int64_t kNearUnitMin = 2048, kNearUnitMax = 65536;
 void near_units_of(const Tree& tr, const std::vector<int32_t>& cnt, const std::vector<int64_t>& extent,
                    int64_t near_elems, std::vector<int32_t>& item_begin, std::vector<int32_t>& unit_begin) {
   const int32_t nc = tr.nclusters();
-  const int64_t target = std::min(kNearUnitMax, std::max(kNearUnitMin, near_elems / (152 * 32)));
+  const int64_t target = std::min(kNearUnitMax, std::max(kNearUnitMin, near_elems / (152 * 12)));
   item_begin.assign(nc + 1, 0);
   unit_begin.assign(nc + 1, 0);
   for (int32_t c = 0; c < nc; ++c) {
@@ -897,6 +897,12 @@ struct PlanState {
   std::function<cudaError_t(const void* const* G, cudaStream_t st)> set_inputs;
 };
 
+// Leaf pairs up to which one Jacobi launch takes all size classes (two waves of
+// the largest class's CTAs, 8 per SM), and non-leaf pairs of a level up to which
+// one Cholesky and one Jacobi launch take all row classes (4 per SM).
+constexpr int64_t kOneJacobi = 152 * 16;
+constexpr int kOneLevel = 152 * 4;
+
 // The compression of one or several independent problems: each phase is one
 // launch over every problem (block norms, leaf factors, one launch per level
 // for the non-leaf steps), then expansion and projection per problem.
@@ -1385,30 +1391,29 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
   // device input): the leaf phase split into its two kernels
   cudaEvent_t kev[4 * kLeafClasses] = {};
   bool kev_ok = false;
-  auto leaf_factor = [&](const uint32_t* codes, int n, int c, bool timed) {
+  auto leaf_factor = [&](const uint32_t* codes, int n, int c, bool timed, bool jacobi) {
     if (n <= 0) return;
     const int P = even_up(std::max(2, cls_maxm[c]));
-    if constexpr (sizeof(T) == 4) {
-      if (mixed) {
+    if constexpr (f32) {
+      if (mixed || cls_maxm[c] <= kGramRows) {
         if (timed) cudaEventRecord(kev[4 * c], st);
-        ok_launch &= launch_gram(d_ga, codes, n, cls_maxm[c], st);  // row scales, then the Gram matrices
-        counted(DH2_KC_GRAM_SCALES, true);
+        if (mixed) {
+          ok_launch &= launch_gram(d_ga, codes, n, cls_maxm[c], st);  // row scales, then the Gram matrices
+          counted(DH2_KC_GRAM_SCALES, true);
+        } else {
+          ok_launch &= launch_gram_i64(d_pa, codes, nullptr, n, P, st);
+        }
         counted(DH2_KC_LEAF_GRAM + c, true);
         if (timed) cudaEventRecord(kev[4 * c + 1], st);
         // pivoted Cholesky, then Jacobi, rank and Q
         if (timed) cudaEventRecord(kev[4 * c + 2], st);
-        ok_launch &= launch_pair_kernel_gram(d_pa, codes, n, P, false, st);
+        ok_launch &= launch_gram_cholesky(d_pa, codes, n, P, false, st);
         counted(DH2_KC_LEAF_FACTOR + c, true);
-        counted(DH2_KC_LEAF_JACOBI + c, true);
+        if (jacobi) {
+          ok_launch &= launch_gram_jacobi(d_pa, codes, n, P, false, st);
+          counted(DH2_KC_LEAF_JACOBI + c, true);
+        }
         if (timed) cudaEventRecord(kev[4 * c + 3], st);
-        return;
-      }
-      if (cls_maxm[c] <= kGramRows) {
-        ok_launch &= launch_gram_i64(d_pa, codes, nullptr, n, P, st);
-        counted(DH2_KC_LEAF_GRAM + c, true);
-        ok_launch &= launch_pair_kernel_gram(d_pa, codes, n, P, false, st);
-        counted(DH2_KC_LEAF_FACTOR + c, true);
-        counted(DH2_KC_LEAF_JACOBI + c, true);
         return;
       }
     }
@@ -1416,7 +1421,7 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
     counted(DH2_KC_LEAF_FACTOR + c, true);
   };
   auto leaf_lists = [&](const HList* L) {
-    for (int c = 0; c < kLeafClasses; ++c) leaf_factor(L[c].d_codes, (int)L[c].codes->size(), c, false);
+    for (int c = 0; c < kLeafClasses; ++c) leaf_factor(L[c].d_codes, (int)L[c].codes->size(), c, false, true);
   };
   auto leaf_rq = [&](const HList* L) {
     for (int c = 0; c < kLeafClasses; ++c)
@@ -1509,9 +1514,22 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
         kev_ok = cudaEventCreate(&kev[i]) == cudaSuccess;
       if (!kev_ok) cudaGetLastError();  // no split timing; the compression itself goes on
     }
+    // few pairs: one Jacobi launch for all size classes (their CTAs sized by the
+    // largest), so that the classes' longest pairs run side by side
+    int one_cls = -1;
+    for (int c = 0; c < kLeafClasses; ++c)
+      if (f32 && cls_begin[c + 1] > cls_begin[c] && (mixed || cls_maxm[c] <= kGramRows)) one_cls = c;
+    const bool one_jacobi = one_cls > 0 && cls_begin[one_cls + 1] <= kOneJacobi;
     for (int c = 0; c < kLeafClasses; ++c)
       leaf_factor(d_leaf + cls_begin[c], (int)(cls_begin[c + 1] - cls_begin[c]), c,
-                  kev_ok && cls_begin[c + 1] > cls_begin[c]);
+                  kev_ok && cls_begin[c + 1] > cls_begin[c], !(one_jacobi && c <= one_cls));
+    if constexpr (f32)
+      if (one_jacobi) {
+        ok_launch &= launch_gram_jacobi(d_pa, d_leaf, (int)cls_begin[one_cls + 1],
+                                        even_up(std::max(2, cls_maxm[one_cls])), false, st);
+        counted(DH2_KC_LEAF_JACOBI + one_cls, true);
+        if (kev_ok) cudaEventRecord(kev[4 * one_cls + 3], st);
+      }
     rec(2);
     // R of the leaf pairs: in the mixed mode one tensor-core launch over every
     // class's tiles; otherwise one launch per size class (shared memory sized by
@@ -1585,7 +1603,9 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
         cudaGetLastError();
         ok_launch = false;
       }
-      launch_classify<T>(d_pa, d_nl[l], n, d_cls, d_cnt, st);
+      // few pairs: their row classes' longest run side by side in one launch
+      const bool merge = f32 && n <= kOneLevel;
+      launch_classify<T>(d_pa, d_nl[l], n, d_cls, d_cnt, merge, st);
       counted(DH2_KC_CLASSIFY, true);
       const int Pc[4] = {32, 48, 64, P_level[l]};
       // FP32: pairs of at most kGramRows rows from the Gram matrices of their
@@ -1594,12 +1614,15 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
       if constexpr (f32) {
         ok_launch &= launch_gram_i64(d_pa, nullptr, d_gseg[l], (int)n_gseg[l], P_level[l], st);
         counted(DH2_KC_LEVEL_FACTOR, true);
-        for (int c = 0; c < 3; ++c) {
-          if (c > 0 && Pc[c - 1] >= P_level[l]) break;  // no pair of this level has more rows
-          ok_launch &= launch_pair_kernel_gram(d_pa, d_cls + (int64_t)c * n, n, std::min(Pc[c], std::max(P_level[l], 2)),
-                                               true, st, d_cnt + c);
+        for (int c = merge ? 2 : 0; c < 3; ++c) {
+          if (!merge && c > 0 && Pc[c - 1] >= P_level[l]) break;  // no pair of this level has more rows
+          const int P = std::min(Pc[c], std::max(P_level[l], 2));
+          ok_launch &= launch_gram_cholesky(d_pa, d_cls + (int64_t)c * n, n, P, true, st, d_cnt + c);
+          ok_launch &= launch_gram_jacobi(d_pa, d_cls + (int64_t)c * n, n, P, true, st, d_cnt + c);
           counted(DH2_KC_LEVEL_FACTOR + c, true);
           counted(DH2_KC_LEVEL_FACTOR + c, true);
+          for (int m = 0; merge && m < 2; ++m)  // a launch over several classes counts in each of them
+            if (m == 0 || Pc[m - 1] < P_level[l]) ++kcl[DH2_KC_LEVEL_FACTOR + m];
         }
       }
       // wide pairs: their column segments' factors first, by row class

@@ -233,8 +233,10 @@ bool launch_pair_kernel(const PairArgs<T>* args_dev, const uint32_t* codes, int 
 // and Q.  Non-leaf pairs (from_r): H summed over the pair's column segments;
 // count as for launch_pair_kernel.
 constexpr int kGramRows = 64;
-bool launch_pair_kernel_gram(const PairArgs<float>* args_dev, const uint32_t* codes, int nblocks, int P, bool from_r,
-                             cudaStream_t st, const int* count = nullptr);
+bool launch_gram_cholesky(const PairArgs<float>* args_dev, const uint32_t* codes, int nblocks, int P, bool from_r,
+                          cudaStream_t st, const int* count = nullptr);
+bool launch_gram_jacobi(const PairArgs<float>* args_dev, const uint32_t* codes, int nblocks, int P, bool from_r,
+                        cudaStream_t st, const int* count = nullptr);
 
 // H = A A^* from products of fixed-point integers on the integer pipe, FP32
 // mode's leaf pairs (codes) or a level's pairs by segments of kGramSegCols
@@ -253,9 +255,10 @@ bool launch_rq_kernel(const PairArgs<T>* args_dev, const uint64_t* tiles, int nt
                       cudaStream_t st);
 
 // Non-leaf codes of one level split by the row count of their Ghat (from the
-// sons' ranks): out = 4 segments of n codes, counts[4] zeroed by the caller.
+// sons' ranks): out = 4 segments of n codes, counts[4] zeroed by the caller;
+// merge: the pairs of at most kGramRows rows all in segment 2.
 template <typename T>
-void launch_classify(const PairArgs<T>* args_dev, const uint32_t* codes, int n, uint32_t* out, int* counts,
+void launch_classify(const PairArgs<T>* args_dev, const uint32_t* codes, int n, uint32_t* out, int* counts, bool merge,
                      cudaStream_t st);
 // the same for segment entries (code << 32 | segment)
 template <typename T>

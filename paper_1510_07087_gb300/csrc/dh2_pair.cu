@@ -2345,10 +2345,11 @@ bool prof_read_pair(unsigned long long* out17) {
 
 // Non-leaf pairs of one level by row count p = k_t1c' + k_t2c' (known only
 // once the sons' ranks are): class 0..3 for p <= 32, <= 48, <= 64, more.
-// out holds 4 segments of n codes; counts[c] the class sizes.
+// out holds 4 segments of n codes; counts[c] the class sizes.  merge: classes 0 to
+// 2 as one, in class 2's place.
 template <typename T>
 __global__ void classify_kernel(const PairArgs<T>* __restrict__ args, const uint32_t* __restrict__ codes, int n,
-                                uint32_t* __restrict__ out, int* __restrict__ counts) {
+                                uint32_t* __restrict__ out, int* __restrict__ counts, bool merge) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const uint32_t code = codes[i];
@@ -2356,7 +2357,7 @@ __global__ void classify_kernel(const PairArgs<T>* __restrict__ args, const uint
   const int side = (int)((code >> kCodeSideShift) & 1u);
   const int pid = (int)(code & kCodePairMask);
   const int p = a.rank[side][a.son[side][2 * pid]] + a.rank[side][a.son[side][2 * pid + 1]];
-  const int cls = p <= 32 ? 0 : p <= 48 ? 1 : p <= 64 ? 2 : 3;
+  const int cls = p > kGramRows ? 3 : merge ? 2 : p <= 32 ? 0 : p <= 48 ? 1 : 2;
   out[(int64_t)cls * n + atomicAdd(&counts[cls], 1)] = code;
 }
 
@@ -2411,9 +2412,9 @@ bool launch_rq_kernel(const PairArgs<T>* args, const uint64_t* tiles, int ntiles
   return launch_rq_leaf<T>(args, tiles, ntiles, P, st);
 }
 template <typename T>
-void launch_classify(const PairArgs<T>* args, const uint32_t* codes, int n, uint32_t* out, int* counts,
+void launch_classify(const PairArgs<T>* args, const uint32_t* codes, int n, uint32_t* out, int* counts, bool merge,
                      cudaStream_t st) {
-  if (n > 0) classify_kernel<T><<<(n + 255) / 256, 256, 0, st>>>(args, codes, n, out, counts);
+  if (n > 0) classify_kernel<T><<<(n + 255) / 256, 256, 0, st>>>(args, codes, n, out, counts, merge);
 }
 template <typename T>
 void launch_classify_seg(const PairArgs<T>* args, const uint64_t* segs, int n, uint64_t* out, int* counts,
@@ -2423,8 +2424,8 @@ void launch_classify_seg(const PairArgs<T>* args, const uint64_t* segs, int n, u
 template void launch_classify_seg<float>(const PairArgs<float>*, const uint64_t*, int, uint64_t*, int*, cudaStream_t);
 template void launch_classify_seg<double>(const PairArgs<double>*, const uint64_t*, int, uint64_t*, int*,
                                           cudaStream_t);
-template void launch_classify<float>(const PairArgs<float>*, const uint32_t*, int, uint32_t*, int*, cudaStream_t);
-template void launch_classify<double>(const PairArgs<double>*, const uint32_t*, int, uint32_t*, int*, cudaStream_t);
+template void launch_classify<float>(const PairArgs<float>*, const uint32_t*, int, uint32_t*, int*, bool, cudaStream_t);
+template void launch_classify<double>(const PairArgs<double>*, const uint32_t*, int, uint32_t*, int*, bool, cudaStream_t);
 
 template bool launch_rq_kernel<float>(const PairArgs<float>*, const uint64_t*, int, int, bool, bool, cudaStream_t);
 template bool launch_rq_kernel<double>(const PairArgs<double>*, const uint64_t*, int, int, bool, bool, cudaStream_t);
@@ -2474,11 +2475,10 @@ bool launch_gram_i64(const PairArgs<float>* args, const uint32_t* codes, const u
 // CTAs, so more pairs at once; at most 32 CTAs per SM).  A level's pairs are few:
 // 4 x rows.
 template <int P_T, int NT, int NTN, int NTM, bool FROM_R>
-bool launch_gram_factor(const PairArgs<float>* args, const uint32_t* codes, int nblocks, int P, cudaStream_t st,
-                        const int* count) {
+bool launch_jacobi(const PairArgs<float>* args, const uint32_t* codes, int nblocks, int P, cudaStream_t st,
+                   const int* count) {
   static_assert(NT % 32 == 0 && NTN % 32 == 0 && NTM % 32 == 0 && NTM >= P_T,
                 "whole warps (the Jacobi reductions run converged), one thread per column of the rank step");
-  if (!launch_one<float, P_T, FROM_R, NT, true>(args, codes, nblocks, P, st, count)) return false;
   const size_t smem = (((size_t)P * (P + 1) * sizeof(C2<float>) + 15) & ~(size_t)15) + (size_t)P * sizeof(double) +
                       (size_t)P * sizeof(int);
   constexpr int MINB = 2048 / NT - 4;
@@ -2504,20 +2504,32 @@ bool launch_gram_factor(const PairArgs<float>* args, const uint32_t* codes, int 
   return true;
 }
 
-bool launch_pair_kernel_gram(const PairArgs<float>* args, const uint32_t* codes, int nblocks, int P, bool from_r,
-                             cudaStream_t st, const int* count) {
+bool launch_gram_cholesky(const PairArgs<float>* args, const uint32_t* codes, int nblocks, int P, bool from_r,
+                          cudaStream_t st, const int* count) {
   if (nblocks <= 0) return true;
   if (from_r) {
-    if (P <= 32) return launch_gram_factor<32, 128, 64, 32, true>(args, codes, nblocks, P, st, count);
-    if (P <= 48) return launch_gram_factor<48, 192, 96, 64, true>(args, codes, nblocks, P, st, count);
-    if (P <= 64) return launch_gram_factor<64, 256, 128, 64, true>(args, codes, nblocks, P, st, count);
-    return false;
+    if (P <= 32) return launch_one<float, 32, true, 128, true>(args, codes, nblocks, P, st, count);
+    if (P <= 48) return launch_one<float, 48, true, 192, true>(args, codes, nblocks, P, st, count);
+    return P <= 64 && launch_one<float, 64, true, 256, true>(args, codes, nblocks, P, st, count);
   }
-  if (P <= 32) return launch_gram_factor<32, 128, 64, 32, false>(args, codes, nblocks, P, st, count);
-  if (P <= 40) return launch_gram_factor<40, 160, 96, 64, false>(args, codes, nblocks, P, st, count);
-  if (P <= 48) return launch_gram_factor<48, 192, 96, 64, false>(args, codes, nblocks, P, st, count);
-  if (P <= 64) return launch_gram_factor<64, 256, 128, 64, false>(args, codes, nblocks, P, st, count);
-  return false;
+  if (P <= 32) return launch_one<float, 32, false, 128, true>(args, codes, nblocks, P, st, count);
+  if (P <= 40) return launch_one<float, 40, false, 160, true>(args, codes, nblocks, P, st, count);
+  if (P <= 48) return launch_one<float, 48, false, 192, true>(args, codes, nblocks, P, st, count);
+  return P <= 64 && launch_one<float, 64, false, 256, true>(args, codes, nblocks, P, st, count);
+}
+
+bool launch_gram_jacobi(const PairArgs<float>* args, const uint32_t* codes, int nblocks, int P, bool from_r,
+                        cudaStream_t st, const int* count) {
+  if (nblocks <= 0) return true;
+  if (from_r) {
+    if (P <= 32) return launch_jacobi<32, 128, 64, 32, true>(args, codes, nblocks, P, st, count);
+    if (P <= 48) return launch_jacobi<48, 192, 96, 64, true>(args, codes, nblocks, P, st, count);
+    return P <= 64 && launch_jacobi<64, 256, 128, 64, true>(args, codes, nblocks, P, st, count);
+  }
+  if (P <= 32) return launch_jacobi<32, 128, 64, 32, false>(args, codes, nblocks, P, st, count);
+  if (P <= 40) return launch_jacobi<40, 160, 96, 64, false>(args, codes, nblocks, P, st, count);
+  if (P <= 48) return launch_jacobi<48, 192, 96, 64, false>(args, codes, nblocks, P, st, count);
+  return P <= 64 && launch_jacobi<64, 256, 128, 64, false>(args, codes, nblocks, P, st, count);
 }
 
 template bool launch_pair_kernel<float>(const PairArgs<float>*, const uint32_t*, int, int, bool, cudaStream_t,
