@@ -34,6 +34,14 @@ namespace dh2 {
 constexpr int kLeafClasses = 5;
 inline bool mode_f32(int mode) { return mode != DH2_MODE_FP64; }  // complex64 data, FP32 kernels
 inline bool mode_mixed(int mode) { return mode == DH2_MODE_MIXED_BF16X3; }
+// sort key of a leaf pair: its class, then costliest first (29 bits of the cost's
+// float), then the launch code
+inline uint64_t leaf_key(int cls, double cost, uint32_t code) {
+  const float c = (float)cost;
+  uint32_t bits;
+  std::memcpy(&bits, &c, 4);  // non-negative: ordered as an integer
+  return ((uint64_t)cls << 61) | ((uint64_t)((0x7fffffffu - bits) >> 2) << 32) | code;
+}
 inline int leaf_class(int m) { return m <= 32 ? 0 : m <= 40 ? 1 : m <= 48 ? 2 : m <= 64 ? 3 : 4; }
 
 // The process's tuning table (dh2_tuning_set, dh2_autotune): read once by each
@@ -123,6 +131,10 @@ struct Tree::Dev {
   int64_t S_elems = 0, near_elems = 0, bmax_elems = 0;
   int64_t nadm = 0, ninadm = 0;
   int64_t nleaf_codes = 0;
+  // host copies for the merged lists of a batch
+  std::vector<int32_t> adm_h, inadm_h;
+  std::vector<int64_t> pieces_h, pbegin_h;
+  std::vector<uint64_t> leaf_keys_h;  // leaf_key of every leaf pair
   // leaf codes grouped by size class (rows <= 32, <= 40, <= 48, <= 64, more), each
   // group costliest first; the pair kernel's CTA is sized to the class
   int64_t leaf_class_begin[kLeafClasses + 1] = {};
@@ -457,8 +469,10 @@ dh2_status upload_tree(Tree& tr) {
     }
     pbeg.push_back((int64_t)pcs.size());
     D->nnorm_pieces = (int64_t)pcs.size();
-    add64(std::move(pcs), &D->norm_pieces);
-    add64(std::move(pbeg), &D->norm_pbegin);
+    D->pieces_h = std::move(pcs);
+    D->pbegin_h = std::move(pbeg);
+    bufs.push_back({D->pieces_h.data(), bytes_of(D->pieces_h), (void**)&D->norm_pieces});
+    bufs.push_back({D->pbegin_h.data(), bytes_of(D->pbegin_h), (void**)&D->norm_pbegin});
   }
   std::vector<int32_t> item_begin[2], unit_begin[2];
   for (int sd = 0; sd < 2; ++sd) {
@@ -474,7 +488,7 @@ dh2_status upload_tree(Tree& tr) {
     }
     D->nnear_units[sd] = unit_begin[sd].back();
     D->nleaf_units[sd] = (int32_t)leaf_units[sd].size();
-    bufs.push_back({nullptr, sizeof(NearItem) * inadm.size(), (void**)&D->near_items[sd]});
+    bufs.push_back({nullptr, sizeof(NearItem) * (size_t)D->ninadm, (void**)&D->near_items[sd]});
     bufs.push_back({nullptr, sizeof(NearUnit) * (size_t)D->nnear_units[sd], (void**)&D->near_units[sd]});
     bufs.push_back({nullptr, 4 * (size_t)nc, (void**)&near_cursor[sd]});
     add32(std::move(item_begin[sd]), &near_ibegin[sd]);
@@ -482,8 +496,10 @@ dh2_status upload_tree(Tree& tr) {
     bufs.push_back({leaf_units[sd].data(), bytes_of(leaf_units[sd]), (void**)&D->leaf_units[sd]});
   }
   add64(std::move(noff), &D->near_off);
-  add32(std::move(adm), &D->adm_list);
-  add32(std::move(inadm), &D->inadm_list);
+  D->adm_h = std::move(adm);
+  D->inadm_h = std::move(inadm);
+  bufs.push_back({D->adm_h.data(), bytes_of(D->adm_h), (void**)&D->adm_list});
+  bufs.push_back({D->inadm_h.data(), bytes_of(D->inadm_h), (void**)&D->inadm_list});
   // matvec lists: own blocks and father pairs per pair, row side (the
   // product) and column side (the adjoint product)
   for (int sd = 0; sd < 2; ++sd) {
@@ -524,6 +540,7 @@ dh2_status upload_tree(Tree& tr) {
         const int m = tr.size[tr.side[sd].pairs[p].cluster];
         lc.push_back({leaf_class(m), (double)m * m * (double)tr.side[sd].pairs[p].ncols,
                       (int32_t)((sd << kCodeSideShift) | (int32_t)p), m});
+        D->leaf_keys_h.push_back(leaf_key(lc.back().cls, lc.back().cost, (uint32_t)lc.back().code));
       }
     std::stable_sort(lc.begin(), lc.end(), [](const LC& a, const LC& b) {
       return a.cls != b.cls ? a.cls < b.cls : a.cost > b.cost;
@@ -957,7 +974,9 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
   int cls_maxm[kLeafClasses] = {};
   int64_t tile_cls_begin[kLeafClasses + 1] = {};
   std::vector<std::vector<uint64_t>> nl_tiles(maxdepth + 1);
-  size_t args_bytes = align256(sizeof(PairArgs<T>) * nprob) + align256(sizeof(NormsArgs<T>) * nprob);
+  const bool mixed = mode_mixed(cp.mode);
+  size_t args_bytes = align256(sizeof(PairArgs<T>) * nprob) + align256(sizeof(NormsArgs<T>) * nprob) +
+                      align256(mixed ? sizeof(GramArgs) * nprob : 0);
   size_t codes_bytes = 0;
   // FP32 and mixed modes: the column segments of a level's pairs (Gram matrices)
   constexpr bool f32 = sizeof(T) == 4;
@@ -965,57 +984,48 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
   std::vector<const uint64_t*> d_gseg(maxdepth + 1, nullptr);
   std::vector<int64_t> n_gseg(maxdepth + 1, 0);
   if (nprob > 1) {
-    struct LC {
-      int cls;
-      double cost;
-      uint32_t code;
-      int m;
-    };
-    std::vector<LC> lc;
+    // merged from the trees' own lists, the problem in the code's upper bits
+    std::vector<uint64_t> keys;
+    size_t nk = 0, nb = 0, npc = 0, nadm = 0;
+    for (const dh2_matrix* M : Ms) {
+      const Tree::Dev* D = M->tree->tr.dev;
+      nk += D->leaf_keys_h.size();
+      nb += D->adm_h.size() + D->inadm_h.size();
+      npc += D->pieces_h.size();
+      nadm += D->adm_h.size();
+    }
+    keys.reserve(nk);
+    norm_codes.reserve(nb);
+    pieces.reserve(npc);
+    pbegin.reserve(nadm + 1);
     for (int i = 0; i < nprob; ++i) {
       const Tree& tr = Ms[i]->tree->tr;
-      for (int sd = 0; sd < 2; ++sd)
-        for (int64_t p : tr.side[sd].leaf_pairs) {
-          const int m = tr.size[tr.side[sd].pairs[p].cluster];
-          lc.push_back({leaf_class(m), (double)m * m * (double)tr.side[sd].pairs[p].ncols,
-                        ((uint32_t)i << kCodeProbShift) | ((uint32_t)sd << kCodeSideShift) | (uint32_t)p, m});
-        }
+      const Tree::Dev* D = tr.dev;
+      const uint32_t prob = (uint32_t)i << kCodeProbShift;
+      for (uint64_t k : D->leaf_keys_h) keys.push_back(k | prob);
+      for (int c = 0; c < kLeafClasses; ++c) cls_maxm[c] = std::max(cls_maxm[c], (int)D->leaf_class_maxm[c]);
       for (int l = tr.depth; l >= 0; --l)
         for (int sd = 0; sd < 2; ++sd)
           for (int64_t p : tr.side[sd].nonleaf_by_level[l])
-            nl_codes[l].push_back(((uint32_t)i << kCodeProbShift) | ((uint32_t)sd << kCodeSideShift) | (uint32_t)p);
-      if (f32) {
-        const Tree::Dev* D = tr.dev;
+            nl_codes[l].push_back(prob | ((uint32_t)sd << kCodeSideShift) | (uint32_t)p);
+      if (f32)
         for (int l = 0; l <= tr.depth; ++l)
           for (int64_t q = D->gseg_begin[l]; q < D->gseg_begin[l] + D->gseg_count[l]; ++q)
-            gsegs[l].push_back(D->gseg_h[q] | ((uint64_t)i << (32 + kCodeProbShift)));
-      }
-      for (size_t b = 0; b < tr.blocks.size(); ++b)
-        if (tr.blocks[b].adm) norm_codes.push_back(((uint32_t)i << 26) | (uint32_t)b);
-    }
-    n_norm_adm = (int64_t)norm_codes.size();  // admissible blocks first, then the nearfield blocks
-    for (int i = 0; i < nprob; ++i) {
-      const Tree& tr = Ms[i]->tree->tr;
-      for (size_t b = 0; b < tr.blocks.size(); ++b)
-        if (!tr.blocks[b].adm) norm_codes.push_back(((uint32_t)i << 26) | (uint32_t)b);
-    }
-    for (int64_t q = 0; q < n_norm_adm; ++q) {
-      pbegin.push_back((int64_t)pieces.size());
-      const uint32_t code = norm_codes[q];
-      const Tree& tr = Ms[code >> 26]->tree->tr;
-      const Block& B = tr.blocks[code & ((1u << 26) - 1u)];
-      const uint64_t nsl = ((uint64_t)tr.size[B.t] + 31) / 32, ngr = ((uint64_t)tr.size[B.s] + kNormCols - 1) / kNormCols;
-      for (uint64_t sl = 0; sl < nsl; ++sl)
-        for (uint64_t g = 0; g < ngr; ++g) pieces.push_back(((uint64_t)code << 32) | (sl << 16) | g);
+            gsegs[l].push_back(D->gseg_h[q] | ((uint64_t)prob << 32));
+      for (int32_t b : D->adm_h) norm_codes.push_back(prob | (uint32_t)b);
+      const int64_t p0 = (int64_t)pieces.size();
+      for (size_t q = 0; q + 1 < D->pbegin_h.size(); ++q) pbegin.push_back(p0 + D->pbegin_h[q]);
+      for (int64_t pc : D->pieces_h) pieces.push_back((uint64_t)pc | ((uint64_t)prob << 32));
     }
     pbegin.push_back((int64_t)pieces.size());
-    std::stable_sort(lc.begin(), lc.end(), [](const LC& a, const LC& b) {
-      return a.cls != b.cls ? a.cls < b.cls : a.cost > b.cost;
-    });
-    for (size_t i = 0; i < lc.size(); ++i) {
-      leaf_codes.push_back(lc[i].code);
-      cls_maxm[lc[i].cls] = std::max(cls_maxm[lc[i].cls], lc[i].m);
-      cls_begin[lc[i].cls + 1] = (int64_t)i + 1;
+    n_norm_adm = (int64_t)norm_codes.size();  // admissible blocks first, then the nearfield blocks
+    for (int i = 0; i < nprob; ++i)
+      for (int32_t b : Ms[i]->tree->tr.dev->inadm_h) norm_codes.push_back(((uint32_t)i << 26) | (uint32_t)b);
+    std::sort(keys.begin(), keys.end());
+    leaf_codes.reserve(nk);
+    for (size_t i = 0; i < keys.size(); ++i) {
+      leaf_codes.push_back((uint32_t)keys[i]);
+      cls_begin[(keys[i] >> 61) + 1] = (int64_t)i + 1;
     }
     for (int c = 1; c <= kLeafClasses; ++c) cls_begin[c] = std::max(cls_begin[c], cls_begin[c - 1]);
     auto tiles_of = [&](const std::vector<uint32_t>& codes, std::vector<uint64_t>& out) {
@@ -1078,11 +1088,9 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
   // FP32 and mixed modes: the leaf Gram matrices (double-float, mp x mp per leaf
   // pair) and those of the largest level, per problem; mixed modes: the block
   // maxima the leaf slices are scaled by
-  const bool mixed = mode_mixed(cp.mode);
   std::vector<size_t> gram_h_off(nprob, 0), gram_l_off(nprob, 0), gram_m_off(nprob, 0), gram_lvl_off(nprob, 0);
   size_t gram_bytes = 0;
   if (f32) {
-    if (mixed) gram_bytes = align256(sizeof(GramArgs) * nprob);
     for (int i = 0; i < nprob; ++i) {
       const Tree::Dev* D = Ms[i]->tree->tr.dev;
       gram_h_off[i] = gram_bytes;
@@ -1137,9 +1145,9 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
     for (const auto& v : seg_lists) seg_bytes += 5 * align256(8 * v.size()) + align256(16);  // list, 4 classes, counts
   }
   void* scratch = nullptr;
-  if (dev_malloc_async(&scratch, args_bytes + codes_bytes + cls_bytes + host_bytes + gram_bytes + ovr_bytes +
-                                     part_bytes + seg_bytes + 256,
-                       st) != cudaSuccess) {
+  const size_t scratch_bytes = args_bytes + codes_bytes + cls_bytes + host_bytes + gram_bytes + ovr_bytes + part_bytes +
+                               seg_bytes + 256;  // the last 256 bytes: a batch's combined status
+  if (dev_malloc_async(&scratch, scratch_bytes, st) != cudaSuccess) {
     cudaGetLastError();
     return DH2_ENOMEM;
   }
@@ -1189,7 +1197,6 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
       sp2 += align256(16);
     }
   }
-  GramArgs* d_ga = (GramArgs*)gram_base;
   std::vector<GramArgs> gas;
   for (int i = 0; i < nprob && f32; ++i) {
     pas[i].H = Ms[i]->gram ? (float4*)Ms[i]->gram : (float4*)(gram_base + gram_h_off[i]);
@@ -1228,24 +1235,22 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
       g.spin_limit = (uint32_t)std::min<int64_t>(std::max<int64_t>(cp.spin_limit, 0), (int64_t)UINT32_MAX);
     }
   }
+  // the argument blocks and, for a batch, the merged lists go up in one copy
+  std::vector<char> stage(args_bytes + codes_bytes);
   char* sp = (char*)scratch;
-  PairArgs<T>* d_pa = (PairArgs<T>*)sp;
-  sp += align256(sizeof(PairArgs<T>) * nprob);
-  NormsArgs<T>* d_na = (NormsArgs<T>*)sp;
-  sp += align256(sizeof(NormsArgs<T>) * nprob);
-  cudaError_t ce = cudaMemcpyAsync(d_pa, pas.data(), sizeof(PairArgs<T>) * nprob, cudaMemcpyHostToDevice, st);
-  if (ce == cudaSuccess && mixed)
-    ce = cudaMemcpyAsync(d_ga, gas.data(), sizeof(GramArgs) * nprob, cudaMemcpyHostToDevice, st);
-  if (ce == cudaSuccess) ce = ce_ovr;
-  if (ce == cudaSuccess)
-    ce = cudaMemcpyAsync(d_na, nas.data(), sizeof(NormsArgs<T>) * nprob, cudaMemcpyHostToDevice, st);
+  auto put = [&](const void* v, size_t bytes) -> void* {
+    void* d = sp;
+    if (bytes) std::memcpy(stage.data() + (sp - (char*)scratch), v, bytes);
+    sp += align256(bytes);
+    return d;
+  };
+  PairArgs<T>* d_pa = (PairArgs<T>*)put(pas.data(), sizeof(PairArgs<T>) * nprob);
+  NormsArgs<T>* d_na = (NormsArgs<T>*)put(nas.data(), sizeof(NormsArgs<T>) * nprob);
+  GramArgs* d_ga = (GramArgs*)put(gas.data(), sizeof(GramArgs) * gas.size());
+  cudaError_t ce = ce_ovr;
   if (nprob > 1) {
-    auto up = [&](const std::vector<uint32_t>& v) -> const uint32_t* {
-      uint32_t* d = (uint32_t*)sp;
-      if (!v.empty() && ce == cudaSuccess) ce = cudaMemcpyAsync(d, v.data(), 4 * v.size(), cudaMemcpyHostToDevice, st);
-      sp += align256(4 * v.size());
-      return d;
-    };
+    auto up = [&](const std::vector<uint32_t>& v) { return (const uint32_t*)put(v.data(), 4 * v.size()); };
+    auto up64 = [&](const std::vector<uint64_t>& v) { return (const uint64_t*)put(v.data(), 8 * v.size()); };
     d_leaf = up(leaf_codes);
     n_leaf = (int64_t)leaf_codes.size();
     d_norm = up(norm_codes);
@@ -1256,23 +1261,11 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
       d_nl[l] = up(nl_codes[l]);
       n_nl[l] = (int64_t)nl_codes[l].size();
     }
-    auto up64 = [&](const std::vector<uint64_t>& v) -> const uint64_t* {
-      uint64_t* d = (uint64_t*)sp;
-      if (!v.empty() && ce == cudaSuccess) ce = cudaMemcpyAsync(d, v.data(), 8 * v.size(), cudaMemcpyHostToDevice, st);
-      sp += align256(8 * v.size());
-      return d;
-    };
     d_ltiles = up64(leaf_tiles);
     n_ltiles = (int64_t)leaf_tiles.size();
     d_pieces = up64(pieces);
     n_pieces = (int64_t)pieces.size();
-    {
-      int64_t* d = (int64_t*)sp;
-      if (!pbegin.empty() && ce == cudaSuccess)
-        ce = cudaMemcpyAsync(d, pbegin.data(), 8 * pbegin.size(), cudaMemcpyHostToDevice, st);
-      sp += align256(8 * pbegin.size());
-      d_pbegin = d;
-    }
+    d_pbegin = (const int64_t*)put(pbegin.data(), 8 * pbegin.size());
     for (int l = 0; l <= maxdepth; ++l) {
       d_nltiles[l] = up64(nl_tiles[l]);
       n_nltiles[l] = (int64_t)nl_tiles[l].size();
@@ -1308,6 +1301,8 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
       n_gseg[l] = D->gseg_count[l];
     }
   }
+  if (ce == cudaSuccess)
+    ce = cudaMemcpyAsync(scratch, stage.data(), (size_t)(sp - (char*)scratch), cudaMemcpyHostToDevice, st);
   if (hs) {
     char* hp = (char*)scratch + args_bytes + codes_bytes + cls_bytes;
     for (HList& L : hl) {
@@ -1724,11 +1719,17 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
     }
     return DH2_OK;
   }
+  // the status words of a batch are combined on the device: one read
+  uint32_t all = 0;
+  const uint32_t* d_status = Ms[0]->status;
+  if (nprob > 1) {
+    uint32_t* o = (uint32_t*)((char*)scratch + scratch_bytes - 256);
+    launch_status_or<T>(d_pa, nprob, o, st);
+    ++nlaunch;
+    d_status = o;
+  }
+  const cudaError_t e1 = cudaMemcpyAsync(&all, d_status, sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
   cudaFreeAsync(scratch, st);
-  std::vector<uint32_t> status(nprob, 0);
-  cudaError_t e1 = cudaSuccess;
-  for (int i = 0; i < nprob && e1 == cudaSuccess; ++i)
-    e1 = cudaMemcpyAsync(&status[i], Ms[i]->status, sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
   cudaError_t e2 = cudaStreamSynchronize(st);
   cudaError_t e3 = cudaGetLastError();
   float ph[6] = {0, 0, 0, 0, 0, 0};
@@ -1764,8 +1765,7 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
     }
   }
 #endif
-  uint32_t all = ok_launch ? 0u : kStatusTooLarge;
-  for (uint32_t v : status) all |= v;
+  if (!ok_launch) all |= kStatusTooLarge;
   // a timed-out wait leaves later results undefined: it is reported first
   if (all & kStatusTimeout) return DH2_ETIMEOUT;
   if (all & kStatusTooLarge) return DH2_EUNSUPPORTED;
@@ -2030,12 +2030,12 @@ dh2_status prepare_matrix(const dh2_tree* Tc, const void* G, dh2_dtype dtype, in
   sz[ns++] = align256(M->nearfield_copy ? es * D->near_elems : 0);
   sz[ns++] = align256(8 * kSigStride * D->npairs[0]);
   sz[ns++] = align256(8 * kSigStride * D->npairs[1]);
+  sz[ns++] = align256(8 * tr.blocks.size());
+  sz[ns++] = align256(8 * nl);  // eps2, zpow: one copy
+  sz[ns++] = align256(8 * nl);
+  sz[ns++] = align256(16);  // status and both sides' ranks: one memset
   sz[ns++] = align256(4 * D->npairs[0]);
   sz[ns++] = align256(4 * D->npairs[1]);
-  sz[ns++] = align256(8 * tr.blocks.size());
-  sz[ns++] = align256(8 * nl);
-  sz[ns++] = align256(8 * nl);
-  sz[ns++] = align256(16);
   sz[ns++] = align256(16);
   sz[ns++] = align256(gen ? (nrm_host ? 48 : 24) * (size_t)tr.n : 0);  // points (and normals)
   sz[ns++] = align256(es / 2 * (size_t)tr.side[0].nleafcols);
@@ -2060,9 +2060,8 @@ dh2_status prepare_matrix(const dh2_tree* Tc, const void* G, dh2_dtype dtype, in
   }
   char* p = (char*)M->arena;
   void** dst[22] = {&M->R[0], &M->R[1], &M->Q[0], &M->Q[1], &M->X[0], &M->X[1], &M->S, &M->near,
-                    (void**)&M->sig[0], (void**)&M->sig[1], (void**)&M->rank[0], (void**)&M->rank[1],
-                    (void**)&M->invw, (void**)&M->eps2, (void**)&M->zpow, (void**)&M->status, (void**)&M->acc,
-                    (void**)&M->pts, &M->colw[0], &M->colw[1], (void**)&M->bnorm2,
+                    (void**)&M->sig[0], (void**)&M->sig[1], (void**)&M->invw, (void**)&M->eps2, (void**)&M->zpow,
+                    (void**)&M->status, (void**)&M->rank[0], (void**)&M->rank[1], (void**)&M->acc, (void**)&M->pts, &M->colw[0], &M->colw[1], (void**)&M->bnorm2,
                     (void**)&M->pts32};
   for (int i = 0; i < ns; ++i) {
     *dst[i] = p;
@@ -2081,12 +2080,12 @@ dh2_status prepare_matrix(const dh2_tree* Tc, const void* G, dh2_dtype dtype, in
     M->eps2_h[l] = e * e;
     M->zpow_h[l] = std::pow(cp.zeta, -(double)l);
   }
-  cudaError_t ce = cudaMemcpyAsync(M->eps2, M->eps2_h.data(), 8 * nl, cudaMemcpyHostToDevice, M->stream);
+  std::vector<double> tol((size_t)(M->zpow - M->eps2) + nl);
+  std::memcpy(tol.data(), M->eps2_h.data(), 8 * nl);
+  std::memcpy(tol.data() + (M->zpow - M->eps2), M->zpow_h.data(), 8 * nl);
+  cudaError_t ce = cudaMemcpyAsync(M->eps2, tol.data(), 8 * tol.size(), cudaMemcpyHostToDevice, M->stream);
   if (ce == cudaSuccess)
-    ce = cudaMemcpyAsync(M->zpow, M->zpow_h.data(), 8 * nl, cudaMemcpyHostToDevice, M->stream);
-  if (ce == cudaSuccess) ce = cudaMemsetAsync(M->status, 0, 16, M->stream);
-  if (ce == cudaSuccess) ce = cudaMemsetAsync(M->rank[0], 0, 4 * D->npairs[0], M->stream);
-  if (ce == cudaSuccess) ce = cudaMemsetAsync(M->rank[1], 0, 4 * D->npairs[1], M->stream);
+    ce = cudaMemsetAsync(M->status, 0, (size_t)((char*)M->rank[1] - (char*)M->status) + 4 * D->npairs[1], M->stream);
   if (ce == cudaSuccess && gen) {
     // points (then normals) in the tree's permuted order
     const size_t n3 = 3 * (size_t)tr.n;

@@ -265,6 +265,10 @@ template <typename T>
 void launch_classify_seg(const PairArgs<T>* args_dev, const uint64_t* segs, int n, uint64_t* out, int* counts,
                          cudaStream_t st);
 
+// *out = the problems' status words combined (n <= kMaxBatch)
+template <typename T>
+void launch_status_or(const PairArgs<T>* args_dev, int n, uint32_t* out, cudaStream_t st);
+
 // Arguments of the leaf Gram kernel of the mixed modes (one per problem).
 // Index [side] selects the row (0) or column (1) basis.
 struct GramArgs {

@@ -2412,6 +2412,19 @@ bool launch_rq_kernel(const PairArgs<T>* args, const uint64_t* tiles, int ntiles
   return launch_rq_leaf<T>(args, tiles, ntiles, P, st);
 }
 template <typename T>
+__global__ void status_or_kernel(const PairArgs<T>* __restrict__ args, int n, uint32_t* __restrict__ out) {
+  uint32_t v = 0;
+  for (int i = threadIdx.x; i < n; i += 32) v |= *args[i].status;
+  v = __reduce_or_sync(0xffffffffu, v);
+  if (threadIdx.x == 0) *out = v;
+}
+template <typename T>
+void launch_status_or(const PairArgs<T>* args, int n, uint32_t* out, cudaStream_t st) {
+  status_or_kernel<T><<<1, 32, 0, st>>>(args, n, out);
+}
+template void launch_status_or<float>(const PairArgs<float>*, int, uint32_t*, cudaStream_t);
+template void launch_status_or<double>(const PairArgs<double>*, int, uint32_t*, cudaStream_t);
+template <typename T>
 void launch_classify(const PairArgs<T>* args, const uint32_t* codes, int n, uint32_t* out, int* counts, bool merge,
                      cudaStream_t st) {
   if (n > 0) classify_kernel<T><<<(n + 255) / 256, 256, 0, st>>>(args, codes, n, out, counts, merge);
