@@ -2554,7 +2554,6 @@ dh2_status matvec_launches(const dh2_matrix* M, int adj, const void* xv, void* y
   C2<T>* yh = (C2<T>*)((char*)buf + hx);
   const C2<T>* x = (const C2<T>*)xv;
   C2<T>* y = (C2<T>*)yv;
-  DH2_CUDA_TRY(cudaMemsetAsync(y, 0, sizeof(C2<T>) * n * nrhs, st));
   const SideView<T> Vin = side_view<T>(tr, M, si);
   MvArgs<T> a;
   a.V = side_view<T>(tr, M, so);
@@ -2586,16 +2585,21 @@ dh2_status matvec_launches(const dh2_matrix* M, int adj, const void* xv, void* y
   SideLease lease(may_overlap ? M->device : -1);
   const SideStream& side = lease.get();
   bool forked = false;
+  // without the fork the forward step zeroes y, and the leaves' last step and the
+  // nearfield share a launch: n = 1024 30.7 -> 22.5 us
+  const bool zero_first = side.st || D->nleaf[si] == 0;
+  if (zero_first) DH2_CUDA_TRY(cudaMemsetAsync(y, 0, sizeof(C2<T>) * n * nrhs, st));
   if (side.st) {
     forked = cudaEventRecord(side.fork, st) == cudaSuccess && cudaStreamWaitEvent(side.st, side.fork, 0) == cudaSuccess;
     if (forked) {
-      launch_mv_near<T>(a, adj != 0, nrhs, x, y, n, side.st);
+      launch_mv_near<T>(a, adj != 0, nrhs, x, y, n, nullptr, nullptr, 0, side.st);
       DH2_CUDA_TRY(cudaEventRecord(side.join, side.st));
     } else {
       cudaGetLastError();
     }
   }
-  launch_mv_forward_leaf<T>(Vin, D->leaf_list[si], (int)D->nleaf[si], x, nrhs, n, xh, D->hoff[si], st);
+  launch_mv_forward_leaf<T>(Vin, D->leaf_list[si], (int)D->nleaf[si], x, nrhs, n, xh, D->hoff[si],
+                            zero_first ? nullptr : y, st);
   for (int l = tr.depth; l >= 0; --l) {
     const int64_t b = D->lvl_nl_begin[si][l], e = D->lvl_end[si][l];
     if (e > b) launch_mv_forward_up<T>(Vin, D->iota[si] + b, (int)(e - b), nrhs, xh, D->hoff[si], st);
@@ -2607,9 +2611,12 @@ dh2_status matvec_launches(const dh2_matrix* M, int adj, const void* xv, void* y
     const int64_t b = D->lvl_son_begin[so][l], e = D->lvl_son_end[so][l];
     if (e > b) launch_mv_backward_down<T>(a, D->son_list[so] + b, (int)(e - b), nrhs, st);
   }
-  launch_mv_backward_leaf<T>(a, D->leaf_list[so], D->leaf_units[so], D->nleaf_units[so], nrhs, y, n, st);
-  if (forked) DH2_CUDA_TRY(cudaStreamWaitEvent(st, side.join, 0));
-  else launch_mv_near<T>(a, adj != 0, nrhs, x, y, n, st);
+  if (forked) {
+    launch_mv_backward_leaf<T>(a, D->leaf_list[so], D->leaf_units[so], D->nleaf_units[so], nrhs, y, n, st);
+    DH2_CUDA_TRY(cudaStreamWaitEvent(st, side.join, 0));
+  } else {
+    launch_mv_near<T>(a, adj != 0, nrhs, x, y, n, D->leaf_list[so], D->leaf_units[so], D->nleaf_units[so], st);
+  }
   DH2_CUDA_TRY(cudaGetLastError());
   return DH2_OK;
 }

@@ -116,15 +116,23 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
+template <typename T, int NR>
+__device__ __forceinline__ void leaf_unit(const MvArgs<T>& a, const int32_t* __restrict__ pairs, const NearUnit& u,
+                                          int rh0, int nr, int nrhs, C2<T>* __restrict__ y, int64_t n, C2<T>* red);
 template <typename T, int NR, bool ADJ>
 __global__ void __launch_bounds__(128) mv_near(MvArgs<T> a, int rh0, int nr, const C2<T>* __restrict__ x,
-                                               C2<T>* __restrict__ y, int64_t n) {
+                                               C2<T>* __restrict__ y, int64_t n, const int32_t* __restrict__ pairs,
+                                               const NearUnit* __restrict__ leafs, int nrhs) {
   // stages (static shared memory, below 48 KB); FP64 takes half a piece at a time
   constexpr int S = NR <= 4 ? 3 : 2;
   constexpr int SG = kNearElems * 4 / (int)sizeof(T), SX = kNearPiece * NR * 4 / (int)sizeof(T);
   __shared__ __align__(16) C2<T> sm[S * (SG + SX)];
   __shared__ int sw[S];  // width of the piece in each stage, 0 past the last
   static_assert(128 * NR <= S * (SG + SX), "the reduction reuses the stages");
+  if ((int)blockIdx.x >= a.nunits) {  // a small product's leaf step in the same launch
+    leaf_unit<T, NR>(a, pairs, leafs[blockIdx.x - a.nunits], rh0, nr, nrhs, y, n, sm);
+    return;
+  }
   const NearUnit u = a.units[blockIdx.x];
   const int tid = threadIdx.x;
   const int mr = u.cw, r = tid % mr, c = tid / mr, cg = 128 / mr;
@@ -258,12 +266,17 @@ __device__ __forceinline__ void cols_dot(const C2<T>* M, int ld, int p, int k, i
   for (int h = 0; h < NR; ++h) out[h] = C2<T>{sum8(vr[h], lane), sum8(vi[h], lane)};
 }
 
-// forward transformation, leaves: xh_sc = W_sc^* x|_s (Eq. mvm1), one warp per pair
+// forward transformation, leaves: xh_sc = W_sc^* x|_s (Eq. mvm1), one warp per
+// pair; y0 (nzero entries, or NULL): a small product's result, zeroed on the way
 template <typename T, int NR>
 __global__ void __launch_bounds__(128) mv_forward_leaf(SideView<T> W, const int32_t* __restrict__ pairs, int np,
                                                        int rh0, int nr, const C2<T>* __restrict__ x, int nrhs,
                                                        int64_t n, C2<T>* __restrict__ xh,
-                                                       const int64_t* __restrict__ hoff) {
+                                                       const int64_t* __restrict__ hoff, C2<T>* __restrict__ y0,
+                                                       int64_t nzero) {
+  if (y0)
+    for (int64_t i = blockIdx.x * (int64_t)128 + threadIdx.x; i < nzero; i += (int64_t)gridDim.x * 128)
+      y0[i] = czero<T>();
   const int w = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (w >= np) return;
   const int pid = pairs[w];
@@ -511,11 +524,8 @@ __global__ void __launch_bounds__(128) mv_backward_down(MvArgs<T> a, const int32
 // cluster (unit: pairs first .. first + count - 1 of the list, rows as in
 // mv_near), one atomic addition per row and run
 template <typename T, int NR>
-__global__ void __launch_bounds__(128) mv_backward_leaf(MvArgs<T> a, const int32_t* __restrict__ pairs,
-                                                        const NearUnit* __restrict__ units, int rh0, int nr, int nrhs,
-                                                        C2<T>* __restrict__ y, int64_t n) {
-  __shared__ C2<T> red[128 * NR];
-  const NearUnit u = units[blockIdx.x];
+__device__ __forceinline__ void leaf_unit(const MvArgs<T>& a, const int32_t* __restrict__ pairs, const NearUnit& u,
+                                          int rh0, int nr, int nrhs, C2<T>* __restrict__ y, int64_t n, C2<T>* red) {
   const int tid = threadIdx.x;
   const int m = u.cw, r = tid % m, c = tid / m, cg = 128 / m;
   C2<T> acc[NR];
@@ -547,6 +557,13 @@ __global__ void __launch_bounds__(128) mv_backward_leaf(MvArgs<T> a, const int32
     }
     red_add(y + u.out + i + (int64_t)(rh0 + h) * n, s);
   }
+}
+template <typename T, int NR>
+__global__ void __launch_bounds__(128) mv_backward_leaf(MvArgs<T> a, const int32_t* __restrict__ pairs,
+                                                        const NearUnit* __restrict__ units, int rh0, int nr, int nrhs,
+                                                        C2<T>* __restrict__ y, int64_t n) {
+  __shared__ C2<T> red[128 * NR];
+  leaf_unit<T, NR>(a, pairs, units[blockIdx.x], rh0, nr, nrhs, y, n, red);
 }
 
 // The right-hand sides in chunks of a compiled width: f(width constant, first,
@@ -633,10 +650,11 @@ void launch_mv_lists(const NearFill& f, const int32_t* own_blk, int64_t nown, co
 
 template <typename T>
 void launch_mv_forward_leaf(const SideView<T>& W, const int32_t* pairs, int np, const C2<T>* x, int nrhs, int64_t n,
-                            C2<T>* xh, const int64_t* hoff, cudaStream_t st) {
+                            C2<T>* xh, const int64_t* hoff, C2<T>* y0, cudaStream_t st) {
   if (np <= 0) return;
   rhs_chunks<T, sizeof(T) == 4 ? 4 : 2>(nrhs, [&](auto w, int rh, int nr) {
-    mv_forward_leaf<T, decltype(w)::value><<<(np + 3) / 4, 128, 0, st>>>(W, pairs, np, rh, nr, x, nrhs, n, xh, hoff);
+    mv_forward_leaf<T, decltype(w)::value>
+        <<<(np + 3) / 4, 128, 0, st>>>(W, pairs, np, rh, nr, x, nrhs, n, xh, hoff, rh == 0 ? y0 : nullptr, n * nrhs);
   });
 }
 template <typename T>
@@ -677,17 +695,20 @@ void launch_mv_backward_leaf(const MvArgs<T>& a, const int32_t* pairs, const Nea
   });
 }
 template <typename T>
-void launch_mv_near(const MvArgs<T>& a, bool adj, int nrhs, const C2<T>* x, C2<T>* y, int64_t n, cudaStream_t st) {
-  if (a.nunits <= 0) return;
+void launch_mv_near(const MvArgs<T>& a, bool adj, int nrhs, const C2<T>* x, C2<T>* y, int64_t n,
+                    const int32_t* pairs, const NearUnit* leafs, int nleafs, cudaStream_t st) {
+  const int grid = a.nunits + nleafs;
+  if (grid <= 0) return;
   rhs_chunks<T, 8>(nrhs, [&](auto w, int rh, int nr) {
-    if (adj) mv_near<T, decltype(w)::value, true><<<a.nunits, 128, 0, st>>>(a, rh, nr, x, y, n);
-    else mv_near<T, decltype(w)::value, false><<<a.nunits, 128, 0, st>>>(a, rh, nr, x, y, n);
+    constexpr int NR = decltype(w)::value;
+    if (adj) mv_near<T, NR, true><<<grid, 128, 0, st>>>(a, rh, nr, x, y, n, pairs, leafs, nrhs);
+    else mv_near<T, NR, false><<<grid, 128, 0, st>>>(a, rh, nr, x, y, n, pairs, leafs, nrhs);
   });
 }
 
 #define DH2_MV_INST(T)                                                                                      \
   template void launch_mv_forward_leaf<T>(const SideView<T>&, const int32_t*, int, const C2<T>*, int,      \
-                                          int64_t, C2<T>*, const int64_t*, cudaStream_t);                  \
+                                          int64_t, C2<T>*, const int64_t*, C2<T>*, cudaStream_t);          \
   template void launch_mv_forward_up<T>(const SideView<T>&, const int32_t*, int, int, C2<T>*,              \
                                         const int64_t*, cudaStream_t);                                     \
   template void launch_mv_coupling<T>(const MvArgs<T>&, int, int, cudaStream_t);                           \
@@ -695,7 +716,8 @@ void launch_mv_near(const MvArgs<T>& a, bool adj, int nrhs, const C2<T>* x, C2<T
   template void launch_mv_backward_down<T>(const MvArgs<T>&, const int32_t*, int, int, cudaStream_t);      \
   template void launch_mv_backward_leaf<T>(const MvArgs<T>&, const int32_t*, const NearUnit*, int, int,    \
                                            C2<T>*, int64_t, cudaStream_t);                                 \
-  template void launch_mv_near<T>(const MvArgs<T>&, bool, int, const C2<T>*, C2<T>*, int64_t, cudaStream_t);
+  template void launch_mv_near<T>(const MvArgs<T>&, bool, int, const C2<T>*, C2<T>*, int64_t, const int32_t*, \
+                                  const NearUnit*, int, cudaStream_t);
 DH2_MV_INST(float)
 DH2_MV_INST(double)
 

@@ -186,7 +186,7 @@ template <typename T> void launch_expand(const SideView<T>& S, const int32_t* pa
 template <typename T> void launch_project(const ProjArgs<T>& a, int nadm, cudaStream_t st);
 template <typename T>
 void launch_mv_forward_leaf(const SideView<T>& W, const int32_t* pairs, int np, const C2<T>* x, int nrhs,
-                            int64_t n, C2<T>* xh, const int64_t* hoff, cudaStream_t st);
+                            int64_t n, C2<T>* xh, const int64_t* hoff, C2<T>* y0, cudaStream_t st);
 template <typename T>
 void launch_mv_forward_up(const SideView<T>& W, const int32_t* pairs, int np, int nrhs, C2<T>* xh,
                           const int64_t* hoff, cudaStream_t st);
@@ -197,7 +197,8 @@ template <typename T>
 void launch_mv_backward_leaf(const MvArgs<T>& a, const int32_t* pairs, const NearUnit* units, int nunits, int nrhs,
                              C2<T>* y, int64_t n, cudaStream_t st);
 template <typename T>
-void launch_mv_near(const MvArgs<T>& a, bool adj, int nrhs, const C2<T>* x, C2<T>* y, int64_t n, cudaStream_t st);
+void launch_mv_near(const MvArgs<T>& a, bool adj, int nrhs, const C2<T>* x, C2<T>* y, int64_t n,
+                    const int32_t* pairs, const NearUnit* leafs, int nleafs, cudaStream_t st);
 template <typename T, typename RT>
 void launch_error(const ErrArgs<T>& a, const C2<RT>* Gref, int64_t ldr, int nblocks, double* acc,
                   cudaStream_t st);
