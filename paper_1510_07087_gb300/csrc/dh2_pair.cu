@@ -59,15 +59,8 @@ __device__ __forceinline__ C2<T> czero() { return C2<T>{T(0), T(0)}; }
 template <typename T>
 __device__ __forceinline__ C2<T> cadd(C2<T> a, C2<T> b) { return C2<T>{a.re + b.re, a.im + b.im}; }
 template <typename T>
-__device__ __forceinline__ C2<T> csub(C2<T> a, C2<T> b) { return C2<T>{a.re - b.re, a.im - b.im}; }
-template <typename T>
 __device__ __forceinline__ C2<T> cmul(C2<T> a, C2<T> b) {
   return C2<T>{a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re};
-}
-// a * conj(b)
-template <typename T>
-__device__ __forceinline__ C2<T> cmulc(C2<T> a, C2<T> b) {
-  return C2<T>{a.re * b.re + a.im * b.im, a.im * b.re - a.re * b.im};
 }
 template <typename T>
 __device__ __forceinline__ T cnorm2(C2<T> a) { return a.re * a.re + a.im * a.im; }
@@ -911,7 +904,7 @@ __device__ __forceinline__ void jacobi_precondition(C2<double>* Lm, int LDL, int
 // the rank from the tail sums, Q), shared by pair_kernel and
 // gram_jacobi_kernel.  work: free shared memory of work_n entries (FP64's
 // preconditioner; none in FP32).
-template <typename T, int P_T, int NT>
+template <typename T, int P_T, int NT, bool FROM_R>
 __device__ __forceinline__ void jacobi_rank_q(const PairArgs<T>& a, int side, int pid, int p, int LDL, int K,
                                               double E_K, int kcap, int lvl, C2<T>* Lm, double* sig2, int* ord,
                                               int32_t* rank_out, double* sig_out, long long t_b, C2<T>* work,
@@ -922,7 +915,10 @@ __device__ __forceinline__ void jacobi_rank_q(const PairArgs<T>& a, int side, in
   (void)work;
   (void)work_n;
   const int pe = K + (K & 1);
-  const int tpp = a.jacobi_tpp[factor_class(P_T)];
+  // FP64 leaf pairs, many at once: few threads per column pair, so that a warp's
+  // rotation scalars serve eight pairs (n = 8192, leaf factors: 4 threads 24.8 ms,
+  // 8 and more 25.8; a level's few pairs run faster with more)
+  const int tpp = min(a.jacobi_tpp[factor_class(P_T)], sizeof(T) == 8 && !FROM_R ? 4 : 32);
   if constexpr (sizeof(T) == 8 && P_T <= 64)
     if (pe >= 4 && pe * LDL + (pe * pe + 1) / 2 <= work_n)
       jacobi_precondition<P_T, NT>(Lm, LDL, p, pe, work, tpp);
@@ -1036,7 +1032,9 @@ constexpr int gram_min_blocks() {
 
 // FP64: 4 CTAs at 128 threads (128 registers, a few spills) and 2 at 160 and 192
 // keep the FP64 pipe fed between the barriers of a round or step (leaf factors at
-// n = 8192, 128 threads: 2 CTAs 30.9 ms, 3 26.9, 4 25.8)
+// n = 8192, 128 threads: 2 CTAs 30.9 ms, 3 26.9, 4 25.8; now 22.7, and 41.9 before
+// the preconditioned Jacobi.  The pipe, 16 cycles per warp instruction, is ~80%
+// busy: half of it with the LQ's reflections)
 template <int NT, typename T>
 constexpr int pair_min_blocks() {
   return sizeof(T) == 4 ? DH2_PAIR_MINB
@@ -1274,20 +1272,26 @@ __global__ void __launch_bounds__(NT, (GRAM ? gram_min_blocks<NT>() : pair_min_b
     C2<T> x[E];
 #pragma unroll
     for (int u = 0; u < E; u += 2) load_c2x2(xs + ccol(u), x[u], x[u + 1]);
-    C2<T> wa[4] = {czero<T>(), czero<T>(), czero<T>(), czero<T>()};
+    C2<T> w;
+    if constexpr (sizeof(T) == 8) {
+      // one chain, begun with the entry of column j in the group's first lane: 10
+      // additions fewer per row on the FP64 pipe, whose other warps hide the chain
+      w = lq == 0 ? cmul(lrj, v0) : czero<T>();
 #pragma unroll
-    for (int u = 0; u < E; u += 2)
-      if (used(u)) {
-        wa[u & 3] = cmacc(wa[u & 3], c[u], x[u]);
-        wa[(u + 1) & 3] = cmacc(wa[(u + 1) & 3], c[u + 1], x[u + 1]);
-      }
-    C2<T> w = cadd(cadd(wa[0], wa[1]), cadd(wa[2], wa[3]));
+      for (int u = 0; u < E; u += 2)
+        if (used(u)) w = cmacc(cmacc(w, c[u], x[u]), c[u + 1], x[u + 1]);
+    } else {
+      C2<T> wa[4] = {czero<T>(), czero<T>(), czero<T>(), czero<T>()};
+#pragma unroll
+      for (int u = 0; u < E; ++u) wa[u & 3] = cmacc(wa[u & 3], c[u], x[u]);
+      w = cadd(cadd(wa[0], wa[1]), cadd(wa[2], wa[3]));
+    }
 #pragma unroll
     for (int o = 1; o < LQT; o <<= 1) {
       w.re += __shfl_xor_sync(qmask, w.re, o);
       w.im += __shfl_xor_sync(qmask, w.im, o);
     }
-    w = cadd(w, cmul(lrj, v0));
+    if constexpr (sizeof(T) == 4) w = cadd(w, cmul(lrj, v0));
     const C2<T> tw = C2<T>{tau * w.re, tau * w.im};
 #pragma unroll
     for (int u = 0; u < E; u += 2)
@@ -1295,7 +1299,7 @@ __global__ void __launch_bounds__(NT, (GRAM ? gram_min_blocks<NT>() : pair_min_b
         c[u] = cnmac(c[u], tw, x[u]);
         c[u + 1] = cnmac(c[u + 1], tw, x[u + 1]);
       }
-    if (lq == 0) Lm[j * LDL + r] = csub(lrj, cmulc(tw, v0));
+    if (lq == 0) Lm[j * LDL + r] = cnmac(lrj, tw, C2<T>{v0.re, -v0.im});
   };
 
   auto stage = [&](int j0, int cwid, int ncols, C2<T>* dst) {
@@ -1510,29 +1514,62 @@ __global__ void __launch_bounds__(NT, (GRAM ? gram_min_blocks<NT>() : pair_min_b
     // residual energy of the unchosen rows and the pivot (lowest row on ties);
     // the butterfly leaves the same values in every lane of every warp
     T e = T(0);
-    T best = T(-1);
     int pv = p;
-    for (int r = lane; r < p; r += 32) {
-      if (pcol[r] < 0) {
-        const T v = nu[r];
-        e += v;
-        if (v > best) {
-          best = v;
-          pv = r;
+    if constexpr (sizeof(T) == 8) {
+      // the pivot by the norms' high words (positive doubles order as integers;
+      // 20 bits of the fraction), and only warp 0 sums the energy: every warp's
+      // comparisons and sums had taken a fifth of the step's FP64 operations
+      int best = -1;
+      for (int r = lane; r < p; r += 32)
+        if (pcol[r] < 0) {
+          const int v = __double2hiint(nu[r]);
+          if (warp == 0) e += nu[r];
+          if (v > best) {
+            best = v;
+            pv = r;
+          }
+        }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        if (warp == 0) e += __shfl_xor_sync(0xffffffffu, e, o);
+        const int ob = __shfl_xor_sync(0xffffffffu, best, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, pv, o);
+        if (ob > best || (ob == best && oi < pv)) {
+          best = ob;
+          pv = oi;
+        }
+      }
+      if (tid == 0) {
+        sh_v0[1].re = e;
+        sh_skip[1] = e <= tau_drop_t;
+      }
+      __syncthreads();
+      e = sh_v0[1].re;
+      if (sh_skip[1]) pv = p;
+    } else {
+      T best = T(-1);
+      for (int r = lane; r < p; r += 32) {
+        if (pcol[r] < 0) {
+          const T v = nu[r];
+          e += v;
+          if (v > best) {
+            best = v;
+            pv = r;
+          }
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        e += __shfl_xor_sync(0xffffffffu, e, o);
+        const T ob = __shfl_xor_sync(0xffffffffu, best, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, pv, o);
+        if (ob > best || (ob == best && oi < pv)) {
+          best = ob;
+          pv = oi;
         }
       }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      e += __shfl_xor_sync(0xffffffffu, e, o);
-      const T ob = __shfl_xor_sync(0xffffffffu, best, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, pv, o);
-      if (ob > best || (ob == best && oi < pv)) {
-        best = ob;
-        pv = oi;
-      }
-    }
-    if (e <= tau_drop_t || pv >= p) {
+    if ((sizeof(T) == 4 && e <= tau_drop_t) || pv >= p) {
       K = i;
       E_K = (double)e;
       break;
@@ -1592,7 +1629,7 @@ __global__ void __launch_bounds__(NT, (GRAM ? gram_min_blocks<NT>() : pair_min_b
             Lm[c * LDL + row] = x;
             s = nmac(s, x);
           }
-          if (q == 0) Lm[i * LDL + row] = csub(Lm[i * LDL + row], cmulc(tw, v0));
+          if (q == 0) Lm[i * LDL + row] = cnmac(Lm[i * LDL + row], tw, C2<T>{v0.re, -v0.im});
         } else {
           for (int c = i + 1 + q; c < p; c += LPR) s = nmac(s, Lm[c * LDL + row]);
         }
@@ -1632,7 +1669,7 @@ __global__ void __launch_bounds__(NT, (GRAM ? gram_min_blocks<NT>() : pair_min_b
     }
   }
   __syncthreads();
-  jacobi_rank_q<T, P_T, NT>(a, side, pid, p, LDL, K, E_K, kcap, lvl, Lm, sig2, ord, rank_out, sig_out, t_b,
+  jacobi_rank_q<T, P_T, NT, FROM_R>(a, side, pid, p, LDL, K, E_K, kcap, lvl, Lm, sig2, ord, rank_out, sig_out, t_b,
                             Lm + (int64_t)P * LDL, XTRA * LDL);
 }
 
@@ -1675,7 +1712,7 @@ __global__ void __launch_bounds__(NT, MINB)
 #if DH2_PROF_ON
   t_b = clock64();
 #endif
-  jacobi_rank_q<float, P_T, NT>(a, side, pid, p, LDL, K, E_K, a.kcap[side][pid], a.level[side][pid], Lm, sig2, ord,
+  jacobi_rank_q<float, P_T, NT, FROM_R>(a, side, pid, p, LDL, K, E_K, a.kcap[side][pid], a.level[side][pid], Lm, sig2, ord,
                                 rank_out, sig_out, t_b, nullptr, 0);
 }
 
