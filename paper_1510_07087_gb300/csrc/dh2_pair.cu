@@ -423,12 +423,11 @@ __device__ void gram_cholesky(const PairArgs<T>& a, int side, int pid, int p, in
     // warp 0: Schur trace of the unchosen rows (double-float), the pivot
     // (largest diagonal, lowest row on ties) and its scalars; -1 = stop
     if ((tid >> 5) == 0) {
-      Df e{0.f, 0.f};
-      float best = -1.f;
+      float best = -1.f, ef = 0.f;
       int pv = p;
       for (int r = lane; r < p; r += 32)
         if (pcol[r] < 0) {
-          e = df_add(e, Df{dhi[r], dlo[r]});
+          ef += dhi[r];
           if (dhi[r] > best) {
             best = dhi[r];
             pv = r;
@@ -436,7 +435,7 @@ __device__ void gram_cholesky(const PairArgs<T>& a, int side, int pid, int p, in
         }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
-        e = df_add(e, df_shfl_xor(e, o));
+        ef += __shfl_xor_sync(0xffffffffu, ef, o);
         const float ob = __shfl_xor_sync(0xffffffffu, best, o);
         const int oi = __shfl_xor_sync(0xffffffffu, pv, o);
         if (ob > best || (ob == best && oi < pv)) {
@@ -444,7 +443,17 @@ __device__ void gram_cholesky(const PairArgs<T>& a, int side, int pid, int p, in
           pv = oi;
         }
       }
-      const Df gap = df_add(e, df_neg(tau_s));  // e - tau
+      // the FP32 trace decides while it is clear of the threshold (a trace falls by
+      // orders of magnitude from step to step); near it, or if it is not finite, the
+      // double-float one does (n = 8192 mixed: launches 249 -> 239 us, 32768: 889 -> 845)
+      Df e{0.f, 0.f}, gap{1.f, 0.f};
+      if (!(ef > 1.001f * tau_s.hi && ef <= 3.4028235e38f)) {
+        for (int r = lane; r < p; r += 32)
+          if (pcol[r] < 0) e = df_add(e, Df{dhi[r], dlo[r]});
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) e = df_add(e, df_shfl_xor(e, o));
+        gap = df_add(e, df_neg(tau_s));  // e - tau
+      }
       const bool stop = !(gap.hi > 0.f) || pv >= p || !(best > 0.f);
       if (lane == 0) {
         sh_pv = stop ? -1 : pv;
