@@ -639,7 +639,9 @@ def run_gpu(args):
                                   "ms": fac_ms}}
     else:
         kern_ms = leaf_ms
-        roof = {"bound": "hbm", "kernel": "pair_kernel (leaf launches: LQ, pivoted truncation, Jacobi, Q)",
+        roof = {"bound": "hbm", "kernel": "leaf launches: " + ("pair_kernel (LQ, pivoted truncation, Jacobi, Q)"
+                                                           if args.mode == "fp64" else
+                                                           "gram_i64_kernel, pair_kernel<...,GRAM>, gram_jacobi_kernel"),
                 "achieved": leaf_bytes / (kern_ms * 1e-3) / 1e9, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": leaf_bytes / (kern_ms * 1e-3) / 1e9 / peaks["hbm_gbs"], "peak_source": src,
                 "traffic": _traffic("pair", src_sha, args), "alg_bytes_per_launch": leaf_bytes,

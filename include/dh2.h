@@ -56,8 +56,9 @@ typedef enum { DH2_C64 = 0, DH2_C128 = 1 } dh2_dtype;
 
 /* Arithmetic of the compression.
  *  FP64: complex128 input and FP64 everywhere (the plain form).
- *  FP32: complex64 input, FP32 factorisations on the non-squared factors
- *        (streamed Householder LQ), FP64 tail sums for the rank decisions.
+ *  FP32: complex64 input, FP32 Jacobi on factors of Gram matrices summed
+ *        exactly in 64-bit integers (pairs of up to 64 rows; wider ones by a
+ *        streamed Householder LQ), FP64 tail sums for the rank decisions.
  *  MIXED_BF16X3: complex64 input; the leaf step of Section 6 reduces each
  *        leaf matrix G^omega_tc to its Gram matrix on the tensor cores
  *        (tcgen05, bf16 operands, FP32 accumulation in tensor memory) from
@@ -290,7 +291,8 @@ void dh2_plan_free(dh2_plan* P);
  *                    (default, measured faster).  The two agree to FP32
  *                    rounding.
  *  level_seg_cols  : non-leaf pairs with more than 2 x level_seg_cols
- *                    columns are factored in column segments of that width
+ *                    columns (FP64, and FP32 pairs of more than 64 rows)
+ *                    are factored in column segments of that width
  *                    (each segment's LQ factor L_i by its own CTA, then the
  *                    pair's factor from [L_1 ... L_S], which has the same
  *                    singular values and left singular vectors); 0 = never

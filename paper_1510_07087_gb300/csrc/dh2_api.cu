@@ -2125,8 +2125,8 @@ dh2_status prepare_matrix(const dh2_tree* Tc, const void* G, dh2_dtype dtype, in
 // backward error (2^-23 of a row's largest entry) and the double-float Gram
 // matrix resolve sigma^2 to about 2^-46 of the leaf matrix's squared norm,
 // which reaches the tail sums of the rank rule once eps falls below ~1e-5.
-// There (unless the Gram matrices are asked for) the leaves take the FP32
-// streamed LQ, which works on the leaf matrix itself.
+// There (unless the Gram matrices are asked for) the leaves take the FP32 mode's
+// Gram matrices, 27 bits per entry and exact (gram_i64_kernel).
 constexpr double kMixedMinEps = 1e-5;
 dh2_compress_params leaf_path(const dh2_compress_params& p) {
   dh2_compress_params q = p;

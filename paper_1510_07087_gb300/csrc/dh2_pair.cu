@@ -10,7 +10,10 @@
 //      lower-triangular factor L with A = L Omega, Omega with orthonormal
 //      rows: an LQ factorisation by Householder reflections applied chunk by
 //      chunk, so the Gram matrix A A^* is never formed and singular values
-//      are not squared;
+//      are not squared (FP64, and FP32 pairs of more than kGramRows rows; the
+//      other FP32 pairs and the mixed mode's leaves take a pivoted Cholesky
+//      factor of a Gram matrix formed exactly instead: gram_i64_kernel here, or
+//      the tensor cores);
 //   2. runs one-sided (Hestenes) Jacobi on the columns of L held in shared
 //      memory, one column pair per group of 8 threads and all pairs of a
 //      round at once: L J = U Sigma, so the normalised columns are the left
@@ -1741,7 +1744,7 @@ __global__ void __launch_bounds__(NT, MINB)
 // Threads: 4 x 4 tiles of the lower triangle, the columns of a chunk dealt to
 // G = NT / tiles threads per tile, summed at the end.
 // n = 8192, eps 1e-6, FP32 (leaf factors): streamed LQ with its Jacobi 2.32 ms;
-// this 0.58 ms, Cholesky 0.32, Jacobi 0.60 (with divisions in the staging and no
+// this 0.58 ms, Cholesky 0.31, Jacobi 0.60 (with divisions in the staging and no
 // prefetch 1.12 ms).  Bound by issue: staging, scan and conversion, ~250 per 32
 // entries; the integer products are a fifth of it.  Singular values lie half as
 // far from FP64's as the LQ's (mean 2.3e-7 against 4.1e-7 of the largest).
