@@ -225,7 +225,8 @@ dh2_status dh2_compress_batched(int32_t nprob, const dh2_tree* const* trees, con
  * points, so no dense G is needed.  pts_xyz: host, n x 3 row-major doubles in
  * the caller's order (the array given to dh2_tree_build), copied during the
  * call.  params->mode selects FP32 (complex64 entries: distances and phase
- * reduction in FP64, sin/cos of the reduced phase in FP32) or FP64.  The
+ * reduction in double-float, or in FP64 for points close beside the extent,
+ * sin/cos of the reduced phase in FP32) or FP64.  The
  * nearfield is always copied (params->nearfield must be 0).  dh2_error on the
  * result accepts G_ref = NULL: the reference is then generated in FP64. */
 dh2_status dh2_compress_kernel(const dh2_tree* tree, const double* pts_xyz, double kappa, double diag,

@@ -740,8 +740,12 @@ void fill_args(dh2_matrix* M, const dh2_compress_params& cp, PairArgs<T>& pa, No
       return Df{h, (float)(v - (double)h)};
     };
     const double f = M->pts_factor, kap = M->kappa / f;  // f: a power of two
-    pa.entry = {M->pts32, M->nrm != nullptr, split(kap * 0.31830988618379067), split(kap), (float)M->diag,
-                (float)(M->nrm ? f * f : f)};
+    const double scale = M->nrm ? f * f : f;
+    // double-float while the scale is a normal float and the phases keep 2^-26 beside their double-float error
+    const bool in_range = scale >= 0x1p-126 && scale <= 0x1p126 && std::fabs(kap) <= 0x1p18;
+    pa.entry = {M->pts32,       M->nrm != nullptr, split(kap * 0.31830988618379067), split(kap), (float)M->diag,
+                (float)scale,   in_range ? 0x1p-42f : INFINITY,
+                {M->pts, M->nrm, M->kappa, M->diag}};
   }
   na.entry = pa.entry;
   na.gen = M->gen;

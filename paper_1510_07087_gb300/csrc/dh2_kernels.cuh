@@ -121,11 +121,19 @@ __device__ __forceinline__ Df df_split(double v) {
 // of two above its extent, (and normals) split into two floats each, per point
 // two (with normals four) float4: hi parts, lo parts.  Differences, r, the phase
 // and its reduction are formed in double-float, sin and cos of the reduced
-// phase in FP32: an entry's error is that of its FP32 roundings, as with FP64
-// differences and phase, which GB300's narrow FP64 pipe (about 2 lanes per SM
-// against 128) had made most of the matrix-free mode's time.  n = 16384 cube,
-// before -> after: norms and nearfield 14.9 -> 1.7 ms, leaf R 4.7 -> 0.9 ms, leaf
-// factors 11.5 -> 7.8 ms.  Bound by instruction issue (~120 per entry).
+// phase in FP32, while that leaves an entry's error to its FP32 roundings.  It
+// does not where a difference cancels: a coordinate difference is off by up to
+// 2^-49 (of the scaled extent), <x_i - x_j, n_j> by 2^-48 + 2^-45.5 r.  Entries
+// with r or |<x_i - x_j, n_j>| below 2^22 times that, and all of them where the
+// scaled quantities leave the range (near2 infinite), are formed from the FP64
+// points as in the FP64 form (gen_entry_f64): rare on a surface mesh (spacing
+// above 2^-21 of its extent), but one in six entries on a flat face of a double
+// layer, most of those exactly zero.  GB300's narrow FP64 pipe (about 2 lanes per SM
+// against 128) had made FP64 differences and phases for every entry most of the
+// matrix-free mode's time.  n = 16384 cube, before -> after: norms and nearfield
+// 14.9 -> 1.7 ms, leaf R 4.7 -> 0.9 ms, leaf factors 11.5 -> 7.8 ms (the whole
+// compression 32.3 -> 7.7 ms, 8.0 with the tests for cancellation; double layer
+// 42.9 -> 10.7 ms).
 template <>
 struct Gen<float> {
   const float4* pts;
@@ -133,7 +141,34 @@ struct Gen<float> {
   Df ppi, kap;   // kappa / pi, kappa, for the scaled points
   float diag;
   float scale;   // of the entries: the points' factor (double layer: its square)
+  float near2;   // entries with r^2 below this go by the FP64 points
+  Gen<double> g64;
 };
+// An entry from the FP64 points: differences, distance, phase and its reduction
+// in FP64, sin and cos of the reduced phase in FP32.  (Arguments by value: by
+// reference the callers' copies went through local memory.)
+static __device__ __noinline__ C2<float> gen_entry_f64(const Gen<double> g, int i, int j) {
+  const double *x = g.pts + 3 * (int64_t)i, *y = g.pts + 3 * (int64_t)j;
+  const double dx = x[0] - y[0], dy = x[1] - y[1], dz = x[2] - y[2];
+  double dn = 0.0;
+  if (g.nrm) {
+    const double* v = g.nrm + 3 * (int64_t)j;
+    const double nx = v[0], ny = v[1], nz = v[2];
+    // an axis-parallel flat face: every product is an exact zero (two points at one place: below)
+    if ((dx == 0.0 || nx == 0.0) && (dy == 0.0 || ny == 0.0) && (dz == 0.0 || nz == 0.0) &&
+        (dx != 0.0 || dy != 0.0 || dz != 0.0))
+      return C2<float>{0.f, 0.f};
+    dn = dx * nx + dy * ny + dz * nz;
+  }
+  const double r = sqrt(dx * dx + dy * dy + dz * dz), kr = g.kappa * r;
+  const float sc = (float)(g.nrm ? dn / (12.566370614359172 * r * r * r) : 1.0 / (12.566370614359172 * r));
+  double th = kr * 0.31830988618379067;  // phase / pi
+  th -= 2.0 * rint(0.5 * th);            // reduced to [-1, 1]
+  float sn, cs;
+  sincospif((float)th, &sn, &cs);
+  const float k = g.nrm ? (float)kr : 0.f;
+  return C2<float>{fmaf(k, sn, cs) * sc, fmaf(-k, cs, sn) * sc};
+}
 __device__ __forceinline__ C2<float> gen_entry(const Gen<float>& g, int64_t i, int64_t j) {
   if (i == j) return C2<float>{g.diag, 0.f};
   const int st = g.dlp ? 4 : 2;
@@ -146,6 +181,7 @@ __device__ __forceinline__ C2<float> gen_entry(const Gen<float>& g, int64_t i, i
   const Df2 sx = df_sq(dx), sy = df_sq(dy), sz = df_sq(dz);
   const Df2 s1 = two_sum(sx.p, sy.p), s2 = two_sum(s1.p, sz.p);
   const Df d2 = df_fast_sum(s2.p, ((sx.e + sy.e) + sz.e) + (s1.e + s2.e));
+  if (!(d2.hi >= g.near2)) return gen_entry_f64(g.g64, (int)i, (int)j);
   // r = sqrt(d2): one Newton step from the FP32 square root
   const float ir = rsqrtf(d2.hi), r0 = __fmul_rn(d2.hi, ir);
   const float rest = fmaf(-r0, r0, d2.hi) + d2.lo;
@@ -163,6 +199,7 @@ __device__ __forceinline__ C2<float> gen_entry(const Gen<float>& g, int64_t i, i
   }
   const float4 nh = __ldg(pj + 2), nl = __ldg(pj + 3);
   const Df dn = df_add(df_add(df_mul(dx, Df{nh.x, nl.x}), df_mul(dy, Df{nh.y, nl.y})), df_mul(dz, Df{nh.z, nl.z}));
+  if (fabsf(dn.hi) < fmaf(0x1p-19f, r.hi, 0x1p-21f)) return gen_entry_f64(g.g64, (int)i, (int)j);
   const Df q = df_mul(df_fast_sum(q4.p, q4.e), d2);
   const float iq = __frcp_rn(q.hi), s0 = dn.hi * iq;
   const float sc = fmaf((fmaf(-s0, q.hi, dn.hi) + dn.lo) - s0 * q.lo, iq, s0) * g.scale;
