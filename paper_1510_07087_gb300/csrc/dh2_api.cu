@@ -2130,7 +2130,7 @@ dh2_status prepare_matrix(const dh2_tree* Tc, const void* G, dh2_dtype dtype, in
 // matrix resolve sigma^2 to about 2^-46 of the leaf matrix's squared norm,
 // which reaches the tail sums of the rank rule once eps falls below ~1e-5.
 // There (unless the Gram matrices are asked for) the leaves take the FP32 mode's
-// Gram matrices, 27 bits per entry and exact (gram_i64_kernel).
+// Gram matrices, 26 or 27 bits per entry and exact (gram_i64_kernel).
 constexpr double kMixedMinEps = 1e-5;
 dh2_compress_params leaf_path(const dh2_compress_params& p) {
   dh2_compress_params q = p;

@@ -1736,11 +1736,15 @@ __global__ void __launch_bounds__(NT, MINB)
 // point, q = rint(a 2^(b - e)) with every |re|, |im| of the row below 2^e, and
 // the products are summed exactly in 64-bit integers (IMAD.WIDE, 32 lanes per
 // clock and SM: four per complex product, against 36 FP32 operations in
-// double-float and sixteen for the reflections of an LQ).  b: the sum of N
-// columns stays below 2^62; 27 bits up to 128 columns, 26 to 512, 25 to 2048: a
-// backward error of 2^-(b+1) of each row's largest entry, below FP32's own
-// rounding of the LQ.  A chunk of 64 columns that raises a row's e shifts the sums
-// it enters (their dropped bits lie below the new resolution).
+// double-float and sixteen for the reflections of an LQ).  b: the sum of the
+// columns stays below 2^62: 27 bits up to 128 columns, 26 to 512.  Wider pairs
+// keep 26: where a diagonal sum (by Cauchy and Schwarz the largest are among
+// them) has passed 2^61 the sums go to H in double-float and start anew.  (In one
+// 64-bit sum a pair of 16k columns had 23 bits, and its noise, sqrt(N) 2^-(b+1) of
+// a row's largest entry, raised ranks beyond the compiled limits.)  The backward
+// error is 2^-(b+1) of each row's largest entry per entry.
+// A chunk of 64 columns that raises a row's e shifts the sums it enters (their
+// dropped bits lie below the new resolution).
 // Threads: 4 x 4 tiles of the lower triangle, the columns of a chunk dealt to
 // G = NT / tiles threads per tile, summed at the end.
 // n = 8192, eps 1e-6, FP32 (leaf factors): streamed LQ with its Jacobi 2.32 ms;
@@ -1752,6 +1756,8 @@ __host__ __device__ constexpr int gram_i64_ld(int p) {  // rows in fours, an odd
   return ((p + 3) / 4 | 1) * 4;
 }
 constexpr int kGramI64Chunk = 64;
+constexpr int kGramI64Flush = 512;
+static_assert(kGramSegCols <= kGramI64Flush && kGramI64Flush % kGramI64Chunk == 0, "a level pair's segment is one sum");
 template <bool FROM_R, int NT>
 __global__ void __launch_bounds__(NT, NT <= 128 ? 4 : 3)
     gram_i64_kernel(const PairArgs<float>* __restrict__ args, const uint32_t* __restrict__ codes,
@@ -1761,6 +1767,7 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 4 : 3)
   // two chunks, column jj from jj * LD: A's stored entries as float2, then q in place
   int2* const buf = reinterpret_cast<int2*>(smem);
   __shared__ int rexp[kGramRows], rdel[kGramRows], rmax[kGramRows];
+  __shared__ unsigned char tile_i[kGramRows / 4 * (kGramRows / 4 + 1) / 2], tile_j[kGramRows / 4 * (kGramRows / 4 + 1) / 2];
   __shared__ int cgc[2][CW];
   __shared__ float cwt[2][CW];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1812,8 +1819,12 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 4 : 3)
     while (ti * (ti + 1) / 2 > t) --ti;
     while ((ti + 1) * (ti + 2) / 2 <= t) ++ti;
     tj = t - ti * (ti + 1) / 2;
+    if (grp == 0) {
+      tile_i[t] = (unsigned char)ti;
+      tile_j[t] = (unsigned char)tj;
+    }
   }
-  const int lg = 32 - __clz(N - 1 | 1);  // N <= 2^lg
+  const int lg = 32 - __clz((min(N, kGramI64Flush) - 1) | 1);  // columns of one sum <= 2^lg
   const int b = min(27, (61 - lg) >> 1);  // (27: 2^(b - e) stays finite)
   long long ar[4][4], ai[4][4];
 #pragma unroll
@@ -1821,7 +1832,10 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 4 : 3)
 #pragma unroll
     for (int j = 0; j < 4; ++j) ar[i][j] = ai[i][j] = 0;
   if (tid < kGramRows) rexp[tid] = -1000;
-  for (int i = tid; i < 2 * CW * (LD - p); i += NT) buf[(i / (LD - p)) * LD + p + i % (LD - p)] = make_int2(0, 0);
+  auto zero_pad = [&]() {  // the staging buffers' rows past p
+    for (int i = tid; i < 2 * CW * (LD - p); i += NT) buf[(i / (LD - p)) * LD + p + i % (LD - p)] = make_int2(0, 0);
+  };
+  zero_pad();
   bool bad = false;
   const int RG = (p + 31) >> 5;            // 32-row groups
   const int r = (warp % RG) * 32 + lane;   // the row this thread scans and converts
@@ -1850,6 +1864,53 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 4 : 3)
     }
     cp_async_commit();
   };
+  // the groups' sums (16 entries per tile) added up in the staging buffers, where
+  // no copy may be in flight, and from there into H, added to those of the
+  // columns before; last: both triangles
+  bool flushed = false;
+  auto store = [&](bool last) {
+    longlong2* red = reinterpret_cast<longlong2*>(smem);
+    for (int g = 0; g < G; ++g) {
+      __syncthreads();
+      if (grp == g)
+#pragma unroll
+        for (int u = 0; u < 16; ++u) {
+          longlong2 v = make_longlong2(ar[u >> 2][u & 3], ai[u >> 2][u & 3]);
+          if (g > 0) {
+            const longlong2 w = red[u * ntile + tid % ntile];
+            v.x += w.x;
+            v.y += w.y;
+          }
+          red[u * ntile + tid % ntile] = v;
+        }
+    }
+    __syncthreads();
+    auto to_df = [](long long v, int ex) {
+      const float hi = __ll2float_rn(v);
+      const float lo = __ll2float_rn(v - __float2ll_rn(hi));
+      // 2^ex in two factors (either may lie outside the normal range alone)
+      const int h = ex >> 1;
+      const float s0 = __int_as_float((h + 127) << 23), s1 = __int_as_float((ex - h + 127) << 23);
+      return Df{hi * s0 * s1, lo * s0 * s1};
+    };
+#pragma unroll 1
+    for (int e = tid; e < 16 * ntile; e += NT) {
+      const int u = e / ntile, t = e - u * ntile;
+      const int rr = 4 * tile_i[t] + (u >> 2), cc = 4 * tile_j[t] + (u & 3);
+      if (rr >= p || cc > rr) continue;
+      const longlong2 v = red[e];
+      const int ex = rexp[rr] + rexp[cc] - 2 * b;
+      Df re = to_df(v.x, ex), im = to_df(v.y, ex);
+      float4* h = Hout + rr + (int64_t)cc * mp;
+      if (flushed) {
+        const float4 o = *h;
+        re = df_add(Df{o.x, o.y}, re);
+        im = df_add(Df{o.z, o.w}, im);
+      }
+      *h = make_float4(re.hi, re.lo, im.hi, im.lo);
+      if (last && cc != rr) Hout[cc + (int64_t)rr * mp] = make_float4(re.hi, re.lo, -im.hi, -im.lo);
+    }
+  };
   table(0, 0);
   __syncthreads();
   entries(0, 0);
@@ -1860,8 +1921,17 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 4 : 3)
     if (tid < kGramRows) rmax[tid] = 0;
     if (more) table(j0 + CW, s ^ 1);
     cp_async_wait_all();
-    __syncthreads();  // this chunk has landed; the other buffer's products are done
-    if (more && !gen) entries(j0 + CW, s ^ 1);
+    // flush after this chunk?  Looked at every kGramI64Flush columns, which add at
+    // most 2^62 to a sum: those of 2^61 at one look stay below 2^63 beyond the next
+    bool big = false;
+    if (!FROM_R && more && (j0 + CW) % kGramI64Flush == 0 && grp < G && ti == tj)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) big = big || ar[i][i] > (1ll << 61) / G;
+    // this chunk has landed; the other buffer's products are done
+    bool full = false;
+    if constexpr (FROM_R) __syncthreads();
+    else full = __syncthreads_or(big);
+    if (more && !gen && !full) entries(j0 + CW, s ^ 1);
     if (scan) {
       int m = 0;  // largest |re|, |im| as bits (NaN and infinity above every finite value)
       for (int j = c0; j < cw; j += cs) {
@@ -1924,50 +1994,22 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 4 : 3)
           }
         }
       }
-    if (more && gen) entries(j0 + CW, s ^ 1);
-  }
-  // the groups' sums, through the staging buffer (16 entries per tile)
-  longlong2* red = reinterpret_cast<longlong2*>(smem);
-  for (int g = 1; g < G; ++g) {
-    __syncthreads();
-    if (grp == g)
+    if (full || !more) {
+      store(!more);
+      if (!more) break;
+      flushed = true;
 #pragma unroll
-      for (int u = 0; u < 16; ++u) red[u * ntile + tid % ntile] = make_longlong2(ar[u >> 2][u & 3], ai[u >> 2][u & 3]);
-    __syncthreads();
-    if (grp == 0)
+      for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int u = 0; u < 16; ++u) {
-        const longlong2 v = red[u * ntile + tid];
-        ar[u >> 2][u & 3] += v.x;
-        ai[u >> 2][u & 3] += v.y;
-      }
+        for (int j = 0; j < 4; ++j) ar[i][j] = ai[i][j] = 0;
+      __syncthreads();  // the staging buffers are free again
+      zero_pad();
+    }
+    if (gen || full) entries(j0 + CW, s ^ 1);
   }
   if (__syncthreads_or(bad)) {  // non-finite entries: reported, H zero
     if (tid == 0) atomicOr(a.status, kStatusNaN);
     for (int i = tid; i < mp * mp; i += NT) Hout[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    return;
-  }
-  if (grp == 0) {
-    auto to_df = [](long long v, int ex) {
-      const float hi = __ll2float_rn(v);
-      const float lo = __ll2float_rn(v - __float2ll_rn(hi));
-      // 2^ex in two factors (either may lie outside the normal range alone)
-      const int h = ex >> 1;
-      const float s0 = __int_as_float((h + 127) << 23), s1 = __int_as_float((ex - h + 127) << 23);
-      return make_float2(hi * s0 * s1, lo * s0 * s1);
-    };
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int rr = 4 * ti + i, cc = 4 * tj + j;
-        if (rr < p && cc <= rr) {
-          const int ex = rexp[rr] + rexp[cc] - 2 * b;
-          const float2 re = to_df(ar[i][j], ex), im = to_df(ai[i][j], ex);
-          Hout[rr + (int64_t)cc * mp] = make_float4(re.x, re.y, im.x, im.y);
-          if (cc != rr) Hout[cc + (int64_t)rr * mp] = make_float4(re.x, re.y, -im.x, -im.y);
-        }
-      }
   }
 }
 
