@@ -2489,53 +2489,87 @@ void dh2_matrix_free(dh2_matrix* M) { matrix_release(M); }
 namespace {
 
 // A second stream for the nearfield product beside the transformations, with
-// its fork and join events: taken from a small pool for the time of one call's
-// launches (two threads never enqueue on one at a time), at most kSideStreams
-// per device, kept until the process ends.  Work of an earlier call still
-// running on it only delays this call's.
+// its fork and join events: taken for the time of one call's launches (two
+// threads never enqueue on one at a time) from at most kSideStreams per device,
+// kept until the process ends.  Taken is one that served this caller's stream last
+// (which waits for that product anyway) or whose last product is done: behind
+// another stream's unfinished one this call would wait for whatever that stream
+// waits for.  With none of these the call runs on the caller's stream alone.
 constexpr int kSideStreams = 8;
 struct SideStream {
   cudaStream_t st = nullptr;
   cudaEvent_t fork = nullptr, join = nullptr;
+  unsigned long long served = 0;  // id of the last caller's stream (ids are never used twice)
+  bool leased = false;
 };
 std::mutex g_side_mu;
-std::vector<SideStream> g_side_idle[64];
+SideStream g_side[64][kSideStreams];
 int g_side_made[64] = {};
 class SideLease {
  public:
-  explicit SideLease(int dev) : dev_(dev) {
-    if (dev < 0 || dev >= 64) return;
+  SideLease(int dev, cudaStream_t st) : caller_(st) {
+    unsigned long long id = 0;
+    if (dev < 0 || dev >= 64 || cudaStreamGetId(st, &id) != cudaSuccess) {
+      cudaGetLastError();
+      return;
+    }
     std::lock_guard<std::mutex> lk(g_side_mu);
-    if (!g_side_idle[dev].empty()) {
-      s_ = g_side_idle[dev].back();
-      g_side_idle[dev].pop_back();
-    } else if (g_side_made[dev] < kSideStreams) {
+    SideStream* const all = g_side[dev];
+    for (int i = 0; i < g_side_made[dev] && !s_; ++i)
+      if (!all[i].leased && all[i].served == id) s_ = &all[i];
+    for (int i = 0; i < g_side_made[dev] && !s_; ++i)
+      if (!all[i].leased && cudaEventQuery(all[i].join) == cudaSuccess) s_ = &all[i];
+    if (!s_ && g_side_made[dev] < kSideStreams) {
       SideStream s;
       if (cudaStreamCreateWithFlags(&s.st, cudaStreamNonBlocking) == cudaSuccess &&
           cudaEventCreateWithFlags(&s.fork, cudaEventDisableTiming) == cudaSuccess &&
           cudaEventCreateWithFlags(&s.join, cudaEventDisableTiming) == cudaSuccess) {
-        g_side_idle[dev].reserve(kSideStreams);  // giving it back cannot throw
-        ++g_side_made[dev];
-        s_ = s;
+        s_ = &all[g_side_made[dev]++];
+        *s_ = s;
       } else {
-        cudaGetLastError();
         if (s.fork) cudaEventDestroy(s.fork);
         if (s.st) cudaStreamDestroy(s.st);
       }
     }
+    cudaGetLastError();  // (not ready, or no stream: not this call's errors)
+    if (s_) {
+      s_->served = id;
+      s_->leased = true;
+    }
   }
   ~SideLease() {
-    if (!s_.st) return;
+    if (!s_) return;
+    if (forked_ && !joined_) join();  // an error on the way: the caller's stream still waits
     std::lock_guard<std::mutex> lk(g_side_mu);
-    g_side_idle[dev_].push_back(s_);
+    s_->leased = false;
   }
   SideLease(const SideLease&) = delete;
   SideLease& operator=(const SideLease&) = delete;
-  const SideStream& get() const { return s_; }
+  cudaStream_t stream() const { return s_ ? s_->st : nullptr; }
+  // the side stream behind the caller's
+  bool fork() {
+    forked_ = cudaEventRecord(s_->fork, caller_) == cudaSuccess && cudaStreamWaitEvent(s_->st, s_->fork, 0) == cudaSuccess;
+    if (!forked_) cudaGetLastError();
+    return forked_;
+  }
+  // everything launched on the side stream so far
+  cudaError_t mark() {
+    const cudaError_t e = cudaEventRecord(s_->join, s_->st);
+    marked_ = e == cudaSuccess;
+    return e;
+  }
+  // the caller's stream behind the mark (the host itself, should that fail)
+  cudaError_t join() {
+    joined_ = true;
+    const cudaError_t e = marked_ || mark() == cudaSuccess ? cudaStreamWaitEvent(caller_, s_->join, 0) : cudaErrorUnknown;
+    if (e != cudaSuccess) cudaStreamSynchronize(s_->st);
+    return e;
+  }
 
  private:
-  int dev_;
-  SideStream s_;
+  SideStream* s_ = nullptr;
+  cudaStream_t caller_;
+  bool forked_ = false, marked_ = false, joined_ = false;
 };
 // nearfield entries from which the fork and join (about 6 us) pay: the product's
 // other kernels, ~20 us and more there, are bound by latency and leave HBM idle,
@@ -2581,25 +2615,24 @@ dh2_status matvec_launches(const dh2_matrix* M, int adj, const void* xv, void* y
   // the nearfield on a second stream, beside the transformations (not in a
   // caller's capture: the pool's streams would join it)
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (may_overlap && (D->near_elems < kOverlapElems || D->nadm == 0 ||
-                      cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)) {
+  int dev = -1;
+  if (may_overlap && (D->near_elems < kOverlapElems || D->nadm == 0 || cudaGetDevice(&dev) != cudaSuccess ||
+                      dev != M->device || cudaStreamIsCapturing(st, &cap) != cudaSuccess ||
+                      cap != cudaStreamCaptureStatusNone)) {
     cudaGetLastError();
     may_overlap = false;
   }
-  SideLease lease(may_overlap ? M->device : -1);
-  const SideStream& side = lease.get();
+  SideLease side(may_overlap ? M->device : -1, st);
   bool forked = false;
   // without the fork the forward step zeroes y, and the leaves' last step and the
   // nearfield share a launch: n = 1024 30.7 -> 22.5 us
-  const bool zero_first = side.st || D->nleaf[si] == 0;
+  const bool zero_first = side.stream() || D->nleaf[si] == 0;
   if (zero_first) DH2_CUDA_TRY(cudaMemsetAsync(y, 0, sizeof(C2<T>) * n * nrhs, st));
-  if (side.st) {
-    forked = cudaEventRecord(side.fork, st) == cudaSuccess && cudaStreamWaitEvent(side.st, side.fork, 0) == cudaSuccess;
+  if (side.stream()) {
+    forked = side.fork();
     if (forked) {
-      launch_mv_near<T>(a, adj != 0, nrhs, x, y, n, nullptr, nullptr, 0, side.st);
-      DH2_CUDA_TRY(cudaEventRecord(side.join, side.st));
-    } else {
-      cudaGetLastError();
+      launch_mv_near<T>(a, adj != 0, nrhs, x, y, n, nullptr, nullptr, 0, side.stream());
+      DH2_CUDA_TRY(side.mark());
     }
   }
   launch_mv_forward_leaf<T>(Vin, D->leaf_list[si], (int)D->nleaf[si], x, nrhs, n, xh, D->hoff[si],
@@ -2617,7 +2650,7 @@ dh2_status matvec_launches(const dh2_matrix* M, int adj, const void* xv, void* y
   }
   if (forked) {
     launch_mv_backward_leaf<T>(a, D->leaf_list[so], D->leaf_units[so], D->nleaf_units[so], nrhs, y, n, st);
-    DH2_CUDA_TRY(cudaStreamWaitEvent(st, side.join, 0));
+    DH2_CUDA_TRY(side.join());
   } else {
     launch_mv_near<T>(a, adj != 0, nrhs, x, y, n, D->leaf_list[so], D->leaf_units[so], D->nleaf_units[so], st);
   }
