@@ -30,6 +30,7 @@
 #include <type_traits>
 
 #include "dh2_check.cuh"
+#include "dh2_scalar.cuh"
 #include "dh2_internal.h"
 #include "dh2_kernels.cuh"
 
@@ -116,30 +117,6 @@ struct Eps<double> {
   static constexpr double u = 1.1102230246251565e-16;
   static constexpr double tiny = 1e-280;
 };
-
-// Reciprocal square root and reciprocal for the rotation and reflector scalars:
-// hardware approximations in FP32 (a few ulp; the rotations and reflections
-// stay unitary to that level).  In FP64 the hardware's approximation (better
-// than 2^-18) and one third-order (Halley) step from h = 1 - x y0^2 or 1 - x y0:
-// within 2 ulp in 5 and 3 operations of the narrow FP64 pipe; arguments are
-// normal and finite (squared norms above Eps::tiny), or give NaN.
-__device__ __forceinline__ float frsqrt(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double rsqrt_from(double x, double y0) {
-  const double h = fma(-x * y0, y0, 1.0);
-  return fma(y0 * h, fma(0.375, h, 0.5), y0);
-}
-__device__ __forceinline__ double frsqrt(double x) {
-  double y0;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
-  return rsqrt_from(x, y0);
-}
-__device__ __forceinline__ float frcp(float x) { return __fdividef(1.f, x); }
-__device__ __forceinline__ double frcp(double x) {
-  double y0;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
-  const double h = fma(-x, y0, 1.0);
-  return fma(y0, fma(h, h, h), y0);
-}
 
 // Asynchronous global -> shared copies (cp.async): not held up by CTA
 // barriers; completed by cp_async_wait_all in the issuing thread.
