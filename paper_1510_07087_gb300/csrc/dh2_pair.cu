@@ -749,11 +749,14 @@ __device__ __forceinline__ bool jacobi_sweeps(C2<T>* Lm, int LDL, int p, C2<T>* 
 
 // FP64: L turned by the right singular vectors that an FP32 Jacobi finds, so
 // that the FP64 sweeps start from columns orthogonal to ~1e-6 and two of them
-// are left (of 5.6).  V (FP32, accumulated rotations) is unitary to ~1e-6; L is
-// multiplied by its polar factor V (I + E)^{-1/2} = V (I - F), E = V^* V - I, F =
-// E/2 - 3/8 E^2 (E^3 is below 1e-18; E^2 in FP32 to 1e-19), unitary to FP64
-// rounding: L' = Y - Y F, Y = L V.  About 12 p K^2 FP64 operations, less than a
-// sweep.  work: at least pe LDL + pe^2/2 entries.
+// are left (of 5.6).  V (FP32, accumulated rotations) is unitary to ~5e-6 (|E| below, by
+// row sums: 4.6e-6 in the middle, 1.0e-5 at most over the leaf pairs of n = 2048 and
+// 4096 at eps 1e-4 to 1e-8); L is multiplied by its polar factor V (I + E)^{-1/2} =
+// V (I - F), E = V^* V - I, F = E/2 - 3/8 E^2 + 5/16 E^3, E^2 and E^3 in FP32.  With
+// |E| <= kMaxE what is left out, 35/128 |E|^4, is below 3e-19 and E^2's rounding
+// below 2^-53: unitary to FP64 rounding.  L' = Y - Y F, Y = L V.  About 12 p K^2
+// FP64 operations, less than a sweep.  work: at least pe LDL + pe^2/2 entries.
+constexpr float kMaxE = 3e-5f;
 template <int P_T, int NT>
 __device__ __forceinline__ void jacobi_precondition(C2<double>* Lm, int LDL, int p, int pe, C2<double>* work,
                                                     int tpp_max) {
@@ -775,7 +778,7 @@ __device__ __forceinline__ void jacobi_precondition(C2<double>* Lm, int LDL, int
   ex = sh_ex;
   if (ex <= 1 || ex >= 2045) return;  // zero or not finite
   __syncthreads();
-  if (tid == 0) sh_ex = 0;  // then the largest |E| (its bits)
+  if (tid == 0) sh_ex = 0;  // then whether E is too large
   const double sc = __hiloint2double((2046 - ex) << 20, 0);
   for (int i = tid; i < pe * p; i += NT) {
     const C2<double> v = Lm[(i / p) * LDL + i % p];
@@ -827,38 +830,44 @@ __device__ __forceinline__ void jacobi_precondition(C2<double>* Lm, int LDL, int
   }
   __syncthreads();
   C2<float>* E32 = V;  // V has been read
-  float emax = 0.f;
+  auto tiles = [&](auto f) {  // f(entry, its row, its column) over this thread's entries
 #pragma unroll
-  for (int h = 0; h < ET; ++h) {
-    const int i = tid + h * NT, j = 2 * (i % ht), k = 2 * (i / ht);
-    if (i < ht * ht)
+    for (int h = 0; h < ET; ++h) {
+      const int i = tid + h * NT, j = 2 * (i % ht), k = 2 * (i / ht);
+      if (i < ht * ht)
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int jj = j + (u & 1), kk = k + (u >> 1);
-        if (jj == kk) E[h][u].re -= 1.0;
-        const C2<float> e{(float)E[h][u].re, (float)E[h][u].im};
-        E32[kk * pe + jj] = e;
-        emax = fmaxf(emax, fmaxf(fabsf(e.re), fabsf(e.im)));
-      }
-  }
-  atomicMax(&sh_ex, __float_as_int(emax));
+        for (int u = 0; u < 4; ++u) f(E[h][u], j + (u & 1), k + (u >> 1));
+    }
+  };
+  tiles([&](C2<double>& e, int jj, int kk) {
+    if (jj == kk) e.re -= 1.0;
+    E32[kk * pe + jj] = C2<float>{(float)e.re, (float)e.im};
+  });
   __syncthreads();
-  // not unitary enough for the expansion (not seen; NaN and infinity order
-  // above): L stays as it is, and the FP64 sweeps do all the work
-  if (__int_as_float(sh_ex) > 2e-5f || sh_ex < 0 || sh_ex >= 0x7f800000) return;
-#pragma unroll
-  for (int h = 0; h < ET; ++h) {
-    const int i = tid + h * NT, j = 2 * (i % ht), k = 2 * (i / ht);
-    if (i < ht * ht)
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int jj = j + (u & 1), kk = k + (u >> 1);
-        C2<float> s = czero<float>();
-        for (int l = 0; l < pe; ++l) s = cmacc(s, E32[kk * pe + l], E32[jj * pe + l]);  // E is Hermitian
-        Lm[kk * LDL + jj] =
-            C2<double>{fma(-0.375, (double)s.re, 0.5 * E[h][u].re), fma(-0.375, (double)s.im, 0.5 * E[h][u].im)};
-      }
+  if (tid < pe) {
+    float rs = 0.f;  // |E| <= the largest of its row sums
+    for (int l = 0; l < pe; ++l) rs += fabsf(E32[l * pe + tid].re) + fabsf(E32[l * pe + tid].im);
+    if (!(rs <= kMaxE)) sh_ex = 1;
   }
+  __syncthreads();
+  // not unitary enough for the expansion, or not finite (not seen): L stays as it
+  // is, and the FP64 sweeps do all the work
+  if (sh_ex) return;
+  C2<float>* S32 = reinterpret_cast<C2<float>*>(Lm);  // E^2, where L was (ld pe)
+  tiles([&](C2<double>& e, int jj, int kk) {
+    C2<float> s = czero<float>();
+    for (int l = 0; l < pe; ++l) s = cmacc(s, E32[kk * pe + l], E32[jj * pe + l]);  // E is Hermitian
+    S32[kk * pe + jj] = s;
+    e = C2<double>{fma(-0.375, (double)s.re, 0.5 * e.re), fma(-0.375, (double)s.im, 0.5 * e.im)};
+  });
+  __syncthreads();
+  tiles([&](C2<double>& e, int jj, int kk) {
+    C2<float> s = czero<float>();
+    for (int l = 0; l < pe; ++l) s = cmacc(s, S32[kk * pe + l], E32[jj * pe + l]);
+    e = C2<double>{fma(0.3125, (double)s.re, e.re), fma(0.3125, (double)s.im, e.im)};
+  });
+  __syncthreads();
+  tiles([&](C2<double>& e, int jj, int kk) { Lm[kk * LDL + jj] = e; });  // F
   __syncthreads();
   // L' = Y - Y F, held until every thread has read F
   constexpr int YT = (P_T / 4 * P_T + NT - 1) / NT;
