@@ -646,18 +646,10 @@ __global__ void __launch_bounds__(256) norms_adm_kernel(const NormsArgs<T>* __re
 }
 
 // The admissible blocks' pass of the matrix-free mode, by the same pieces: the
-// entries are generated and their squares added, in FP64 (double) or
-// double-float (float: the FP64 pipe would take longer than the entries do).
+// entries are generated and their squares added in FP64 (two operations of the
+// narrow FP64 pipe per entry, under the ~120 instructions that generate it).
 // One warp per block had left the few coarse blocks of millions of entries to
 // one warp each.
-__device__ __forceinline__ void sq_acc(double& s, C2<double> g) { s += g.re * g.re + g.im * g.im; }
-__device__ __forceinline__ void sq_acc(Df& s, C2<float> g) {  // lo: the errors so far
-  const Df2 a = df_sq(Df{g.re, 0.f}), b = df_sq(Df{g.im, 0.f});
-  const Df2 t = two_sum(s.hi, a.p), u = two_sum(t.p, b.p);
-  s = Df{u.p, s.lo + ((a.e + b.e) + (t.e + u.e))};
-}
-__device__ __forceinline__ double sq_value(double s) { return s; }
-__device__ __forceinline__ double sq_value(Df s) { return (double)s.hi + (double)s.lo; }
 template <typename T>
 __global__ void __launch_bounds__(256) norms_gen_kernel(const NormsArgs<T>* __restrict__ args,
                                                         const uint64_t* __restrict__ pieces, int64_t n,
@@ -674,10 +666,13 @@ __global__ void __launch_bounds__(256) norms_gen_kernel(const NormsArgs<T>* __re
   const int64_t t0 = a.cstart[t], s0 = a.cstart[s];
   const int r = slab * 32 + lane;
   const int c0 = grp * kNormCols, c1 = min(a.csize[s], c0 + kNormCols);
-  typename std::conditional<sizeof(T) == 8, double, Df>::type acc{};
+  double acc = 0.0;
   if (r < a.csize[t])
-    for (int j = c0; j < c1; ++j) sq_acc(acc, gen_entry(a.entry, t0 + r, s0 + j));
-  const double tot = warp_sum(sq_value(acc));
+    for (int j = c0; j < c1; ++j) {
+      const C2<T> g = gen_entry(a.entry, t0 + r, s0 + j);
+      acc = fma((double)g.re, (double)g.re, fma((double)g.im, (double)g.im, acc));
+    }
+  const double tot = warp_sum(acc);
   if (lane == 0) partial[w] = tot;
 }
 
