@@ -278,12 +278,16 @@ void dh2_plan_free(dh2_plan* P);
  * plan keeps the choices it was captured with).
  *  jacobi_tpp[c]   : most threads per column pair of a Jacobi round, factor
  *                    class c (rows <= 32, <= 40, <= 48, <= 64, more): 4, 8,
- *                    16 or 32 (default 32).  Changes the summation order of
- *                    the rotation sums, so results move by rounding only.
- *  jacobi_narrow[c]: mixed mode, leaf classes 0..3: threads per CTA of the
- *                    Jacobi launch, 0 = 4 x rows, 1 = about 2 x rows
+ *                    16 or 32 (default 32, for which FP64 leaf pairs take 4).
+ *                    Changes the summation order of the rotation sums, so
+ *                    results move by rounding only.
+ *  jacobi_narrow[c]: FP32 and mixed modes, leaf classes 0..3: threads per CTA
+ *                    of the Jacobi launch, 0 = 4 x rows, 1 = about 2 x rows
  *                    (default), 2 = about 1 x rows (a multiple of 32), at the
  *                    same threads per SM.  Changes the rounding as above.
+ *                    FP32 and mixed modes, up to 2432 leaf pairs: one launch
+ *                    of the largest class takes all of them, with that class's
+ *                    jacobi_narrow and jacobi_tpp.
  *  rq_ctas_per_sm  : resident CTAs per SM of the persistent leaf R kernel
  *                    of the FP32 pipes, 1..4 within its occupancy limit, 0 =
  *                    that limit (default).  Changes no result.
@@ -323,9 +327,10 @@ typedef struct {
 /* Autotune the table on one problem: compresses (tree, G) with `params`
  * under each candidate of each knob in turn (coordinate descent: in the
  * mixed mode the R kernel, then the R grid, the level steps' segment width
- * (if a non-leaf pair has more than 1024 columns), then per factor class the
- * Jacobi launch width and the threads per column pair; a
- * class with no pairs in the problem is skipped), `reps` calls per candidate
+ * (if a non-leaf pair of more than 1024 columns is factored by column
+ * segments), then per factor class the Jacobi launch width (FP32 and mixed
+ * modes) and the threads per column pair; a class with no leaf pairs in the
+ * problem, or whose entry none of its launches reads, is skipped), `reps` calls per candidate
  * (1..15), keeps the fastest value of each knob, installs the result and
  * returns it in `out`.  records: NULL, or room for `cap` records, of which
  * *nrec are written (every candidate timed, in order; NULL nrec allowed when

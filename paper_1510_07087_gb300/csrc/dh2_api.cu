@@ -923,6 +923,15 @@ struct PlanState {
 // one Cholesky and one Jacobi launch take all row classes (4 per SM).
 constexpr int64_t kOneJacobi = 152 * 16;
 constexpr int kOneLevel = 152 * 4;
+// The class whose Jacobi launch takes the leaf pairs of every class up to it
+// (CTAs sized by the largest, so that the classes' longest pairs run side by
+// side), or -1: each class launches its own.
+int merged_jacobi(bool f32, bool mixed, const int64_t* cls_begin, const int* cls_maxm) {
+  int one = -1;
+  for (int c = 0; c < kLeafClasses; ++c)
+    if (f32 && cls_begin[c + 1] > cls_begin[c] && (mixed || cls_maxm[c] <= kGramRows)) one = c;
+  return one > 0 && cls_begin[one + 1] <= kOneJacobi ? one : -1;
+}
 
 // The compression of one or several independent problems: each phase is one
 // launch over every problem (block norms, leaf factors, one launch per level
@@ -1513,17 +1522,12 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
         kev_ok = cudaEventCreate(&kev[i]) == cudaSuccess;
       if (!kev_ok) cudaGetLastError();  // no split timing; the compression itself goes on
     }
-    // few pairs: one Jacobi launch for all size classes (their CTAs sized by the
-    // largest), so that the classes' longest pairs run side by side
-    int one_cls = -1;
-    for (int c = 0; c < kLeafClasses; ++c)
-      if (f32 && cls_begin[c + 1] > cls_begin[c] && (mixed || cls_maxm[c] <= kGramRows)) one_cls = c;
-    const bool one_jacobi = one_cls > 0 && cls_begin[one_cls + 1] <= kOneJacobi;
+    const int one_cls = merged_jacobi(f32, mixed, cls_begin, cls_maxm);
     for (int c = 0; c < kLeafClasses; ++c)
       leaf_factor(d_leaf + cls_begin[c], (int)(cls_begin[c + 1] - cls_begin[c]), c,
-                  kev_ok && cls_begin[c + 1] > cls_begin[c], !(one_jacobi && c <= one_cls));
+                  kev_ok && cls_begin[c + 1] > cls_begin[c], c > one_cls);
     if constexpr (f32)
-      if (one_jacobi) {
+      if (one_cls >= 0) {
         ok_launch &= launch_gram_jacobi(d_pa, d_leaf, (int)cls_begin[one_cls + 1],
                                         even_up(std::max(2, cls_maxm[one_cls])), false, st);
         counted(DH2_KC_LEAF_JACOBI + one_cls, true);
@@ -2400,7 +2404,7 @@ dh2_status dh2_autotune(const dh2_tree* T, const void* G, dh2_dtype dtype, int64
   if (nrec) *nrec = 0;
   if (!T || !G || !params || !out || reps < 1 || reps > 15 || (records && (cap < 0 || !nrec))) return DH2_EINVAL;
   const TuneTable saved = tune_current();
-  const bool mixed = mode_mixed(leaf_path(*params).mode);
+  const bool mixed = mode_mixed(leaf_path(*params).mode), f32 = mode_f32(params->mode);
   // factor classes with leaf pairs in this problem
   bool has[5] = {false, false, false, false, false};
   for (int sd = 0; sd < 2; ++sd)
@@ -2453,24 +2457,46 @@ dh2_status dh2_autotune(const dh2_tree* T, const void* G, dh2_dtype dtype, int64
     return DH2_OK;
   };
   dh2_status s = DH2_OK;
+  // non-leaf pairs wide enough to split into column segments, and factored by the
+  // LQ (FP32: above kGramRows rows)
+  bool wide = false;
   {
     dh2_matrix* M = nullptr;  // untimed first call: uploads and first-use allocations
     s = dh2_compress(T, G, dtype, ld, params, stream, &M);
-    if (s == DH2_OK) dh2_matrix_free(M);
+    for (int sd = 0; sd < 2 && s == DH2_OK; ++sd) {
+      const std::vector<Pair>& pairs = T->tr.side[sd].pairs;
+      if (pairs.empty()) continue;
+      std::vector<int32_t> k(pairs.size());
+      s = dh2_matrix_ranks(M, sd, k.data());
+      for (const Pair& P : pairs)
+        if (!P.leaf && P.ncols > 2 * 512)
+          wide = wide || !f32 || k[P.son_pair[0]] + k[P.son_pair[1]] > kGramRows;
+    }
+    dh2_matrix_free(M);
   }
   static const int kRq[3] = {0, 1, 2}, kNarrow[3] = {0, 1, 2}, kTpp[3] = {32, 16, 8}, kTensor[2] = {0, 1};
   if (s == DH2_OK && mixed) s = descend(3, 0, kTensor, 2, &best.rq_tensor);
   if (s == DH2_OK) s = descend(0, 0, kRq, 3, &best.rq_ctas_per_sm);
-  // the level steps' column segments, if the problem has non-leaf pairs wide enough to split
-  bool wide = false;
-  for (int sd = 0; sd < 2; ++sd)
-    for (const Pair& P : T->tr.side[sd].pairs) wide = wide || (!P.leaf && P.ncols > 2 * 512);
   static const int kSeg[4] = {1024, 0, 512, 2048};
   if (s == DH2_OK && wide) s = descend(4, 0, kSeg, 4, &best.level_seg_cols);
+  // classes whose entries act on this problem's launches: of the leaf pairs those
+  // with a Jacobi launch of their own, of the level steps those launched
+  const Tree::Dev* D = T->tr.dev;
+  bool lvl[5] = {false, false, false, false, false};
+  for (int l = 0; l <= T->tr.depth && s == DH2_OK; ++l) {
+    const int64_t n = D->nl_code_count[l];
+    if (n == 0) continue;
+    const int P = even_up(std::max(2, (int)D->nl_rowcap_max[l])), Pc[3] = {32, 48, 64};
+    if (f32 && n <= kOneLevel) lvl[std::min(P, 64) <= 32 ? 0 : std::min(P, 64) <= 48 ? 2 : 3] = true;
+    else
+      for (int c = 0; c < 3 && (c == 0 || Pc[c - 1] < P); ++c) lvl[c == 0 ? 0 : c + 1] = true;
+    lvl[4] = lvl[4] || P > 64;
+  }
+  const int one = s == DH2_OK ? merged_jacobi(f32, mixed, D->leaf_class_begin, D->leaf_class_maxm) : -1;
   for (int c = 0; c < 5 && s == DH2_OK; ++c) {
     if (!has[c]) continue;
-    if (mixed && c < 4) s = descend(1, c, kNarrow, 3, &best.jacobi_narrow[c]);
-    if (s == DH2_OK) s = descend(2, c, kTpp, 3, &best.jacobi_tpp[c]);
+    if (f32 && c < 4 && c >= one) s = descend(1, c, kNarrow, 3, &best.jacobi_narrow[c]);
+    if (s == DH2_OK && (c >= one || lvl[c])) s = descend(2, c, kTpp, 3, &best.jacobi_tpp[c]);
   }
   if (nrec) *nrec = nr;
   if (s != DH2_OK) {

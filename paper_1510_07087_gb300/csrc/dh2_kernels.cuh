@@ -18,7 +18,7 @@ struct __align__(2 * sizeof(T)) C2 {
 // table per process, read when a compression prepares its launches.
 struct TuneTable {
   int32_t jacobi_tpp[5];     // factor classes (<= 32, 40, 48, 64 rows, more): most threads per Jacobi column pair
-  int32_t jacobi_narrow[4];  // mixed mode leaf classes: Jacobi CTAs of ~4 (0), ~2 (1) or ~1 (2) x rows threads
+  int32_t jacobi_narrow[4];  // FP32 and mixed leaf classes: Jacobi CTAs of ~4 (0), ~2 (1) or ~1 (2) x rows threads
   int32_t rq_ctas_per_sm;    // leaf R kernel: resident CTAs per SM (0: its occupancy limit)
   int32_t rq_tensor;         // mixed mode: leaf R on the tensor cores (1) or the FP32 pipes (0)
   int32_t level_seg_cols;    // non-leaf pairs wider than twice this: factored by column segments (0: never)

@@ -915,8 +915,10 @@ __device__ __forceinline__ void jacobi_rank_q(const PairArgs<T>& a, int side, in
   const int pe = K + (K & 1);
   // FP64 leaf pairs, many at once: few threads per column pair, so that a warp's
   // rotation scalars serve eight pairs (n = 8192, leaf factors: 4 threads 24.8 ms,
-  // 8 and more 25.8; a level's few pairs run faster with more)
-  const int tpp = min(a.jacobi_tpp[factor_class(P_T)], sizeof(T) == 8 && !FROM_R ? 4 : 32);
+  // 8 and more 25.8; a level's few pairs run faster with more), unless the table
+  // asks for another number than its default
+  const int most = a.jacobi_tpp[factor_class(P_T)];
+  const int tpp = sizeof(T) == 8 && !FROM_R && most == 32 ? 4 : most;
   if constexpr (sizeof(T) == 8 && P_T <= 64)
     if (pe >= 4 && pe * LDL + (pe * pe + 1) / 2 <= work_n)
       jacobi_precondition<P_T, NT>(Lm, LDL, p, pe, work, tpp);
