@@ -128,6 +128,8 @@ struct Tree::Dev {
   std::vector<uint64_t> gseg_h;  // per level: non-leaf pairs' column segments, code << 32 | segment
   std::vector<int64_t> gseg_begin, gseg_count;
   uint64_t* gseg = nullptr;
+  std::vector<int32_t> gseg_cols_h;  // per level: columns of a segment
+  int32_t* gseg_cols = nullptr;
   int64_t S_elems = 0, near_elems = 0, bmax_elems = 0;
   int64_t nadm = 0, ninadm = 0;
   int64_t nleaf_codes = 0;
@@ -304,6 +306,16 @@ dh2_status upload_tree(Tree& tr) {
   D->max_leaf = tr.max_leaf;
 
   std::vector<int64_t> lvl_gram(tr.depth + 1, 0);  // both sides of a level share its Gram buffer
+  auto gram_segs = [&](const Pair& P) { return (P.ncols + D->gseg_cols_h[P.level] - 1) / D->gseg_cols_h[P.level]; };
+  D->gseg_cols_h.assign(tr.depth + 1, kGramSegCols);
+  for (int l = 0; l <= tr.depth; ++l)
+    for (;; D->gseg_cols_h[l] *= 2) {
+      int64_t extra = 0;
+      for (const Side& S : tr.side)
+        for (int64_t p : S.nonleaf_by_level[l]) extra += gram_segs(S.pairs[p]) - 1;
+      if (extra <= kGramSegMax) break;
+    }
+  add32(std::vector<int32_t>(D->gseg_cols_h), &D->gseg_cols);
   for (int sd = 0; sd < 2; ++sd) {
     Side& S = tr.side[sd];
     const int64_t np = (int64_t)S.pairs.size();
@@ -325,7 +337,7 @@ dh2_status upload_tree(Tree& tr) {
       if (P.leaf) {
         rc[p] = tr.size[P.cluster];
         kc[p] = (int32_t)std::min<int64_t>(rc[p], P.ncols);
-        const int64_t mpd = (rc[p] + 7) & ~7;  // Gram matrix: mp x mp
+        const int64_t mpd = rc[p] <= kGramRows ? (rc[p] + 7) & ~7 : 0;  // Gram matrix: mp x mp
         go[p] = D->gram_elems;
         D->gram_elems += mpd * mpd;
       } else {
@@ -339,7 +351,7 @@ dh2_status upload_tree(Tree& tr) {
         X_e += (int64_t)tr.size[P.cluster] * kc[p];
         const int64_t mpd = (std::min(rc[p], kGramRows) + 7) & ~7;
         go[p] = lvl_gram[P.level];
-        lvl_gram[P.level] += mpd * mpd * ((P.ncols + kGramSegCols - 1) / kGramSegCols);
+        lvl_gram[P.level] += mpd * mpd * gram_segs(P);
       }
       ro[p] = R_e;
       R_e += (int64_t)kc[p] * P.ncols;
@@ -566,7 +578,7 @@ dh2_status upload_tree(Tree& tr) {
       for (int sd = 0; sd < 2; ++sd)
         for (int64_t p : tr.side[sd].nonleaf_by_level[l]) {
           codes.push_back((int32_t)((sd << kCodeSideShift) | (int32_t)p));
-          const int64_t nseg = (tr.side[sd].pairs[p].ncols + kGramSegCols - 1) / kGramSegCols;
+          const int64_t nseg = gram_segs(tr.side[sd].pairs[p]);
           for (int64_t g = 0; g < nseg; ++g) D->gseg_h.push_back(((uint64_t)(uint32_t)codes.back() << 32) | (uint64_t)g);
           D->nl_rowcap_max[l] = std::max(D->nl_rowcap_max[l], D->rowcap_h[sd][p]);
         }
@@ -777,6 +789,7 @@ void fill_args(dh2_matrix* M, const dh2_compress_params& cp, PairArgs<T>& pa, No
   pa.invw = M->invw;
   pa.eps2 = M->eps2;
   pa.H = pa.L4 = pa.Hl = nullptr;  // set by run_compress in the FP32 and mixed modes
+  pa.gseg_cols = D->gseg_cols;
   for (int sd = 0; sd < 2; ++sd) {
     pa.hoff[sd] = D->gram_off[sd];
     pa.rank_ovr[sd] = nullptr;  // set by run_compress when ranks are given
@@ -1103,19 +1116,21 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
   // maxima the leaf slices are scaled by
   std::vector<size_t> gram_h_off(nprob, 0), gram_l_off(nprob, 0), gram_m_off(nprob, 0), gram_lvl_off(nprob, 0);
   size_t gram_bytes = 0;
-  if (f32) {
-    for (int i = 0; i < nprob; ++i) {
+  bool gram = f32;  // the FP32 leaf and the level factors from Gram matrices (false: by the LQ)
+  auto gram_layout = [&]() {
+    gram_bytes = 0;
+    for (int i = 0; i < nprob && (gram || mixed); ++i) {
       const Tree::Dev* D = Ms[i]->tree->tr.dev;
       gram_h_off[i] = gram_bytes;
       if (!Ms[i]->gram) gram_bytes += align256(sizeof(float4) * (size_t)D->gram_elems);  // else kept by the matrix
       gram_l_off[i] = gram_bytes;  // Cholesky factors: over H, or beside the kept Gram matrices
       if (Ms[i]->gram) gram_bytes += align256(sizeof(float4) * (size_t)D->gram_elems);
       gram_lvl_off[i] = gram_bytes;
-      gram_bytes += align256(sizeof(float4) * (size_t)D->lvl_gram_elems);
+      if (gram) gram_bytes += align256(sizeof(float4) * (size_t)D->lvl_gram_elems);
       gram_m_off[i] = gram_bytes;
       if (mixed) gram_bytes += align256(sizeof(float) * (size_t)D->bmax_elems);
     }
-  }
+  };
   // ranks given instead of the truncation rule (one problem only)
   size_t ovr_bytes = 0;
   if (nprob == 1)
@@ -1127,13 +1142,18 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
   // non-leaf pairs wider than twice the tuning table's segment width are
   // factored by column segments: per level the segment entries (code << 32 |
   // segment), per problem and side each pair's slot in the segment buffer
-  // (p x p per segment, p at most the pair's row capacity)
+  // (p x p per segment, p at most the pair's row capacity), which the levels
+  // use one after another; pairs that only Gram matrices factor have none
   const int seg_cols = tune_current().level_seg_cols;
-  std::vector<std::vector<uint64_t>> seg_lists(maxdepth + 1);
-  std::vector<std::vector<int64_t>> seg_off_h((size_t)nprob * 2);
+  std::vector<std::vector<uint64_t>> seg_lists;
+  std::vector<std::vector<int64_t>> seg_off_h;
   int64_t seg_elems = 0;
-  if (seg_cols > 0)
-    for (int i = 0; i < nprob; ++i) {
+  size_t seg_bytes = 0;
+  auto seg_layout = [&]() {
+    std::vector<int64_t> lvl_elems(maxdepth + 1, 0);
+    seg_lists.assign(maxdepth + 1, {});
+    seg_off_h.assign((size_t)nprob * 2, {});
+    for (int i = 0; i < nprob && seg_cols > 0; ++i) {
       const Tree& tr = Ms[i]->tree->tr;
       const Tree::Dev* D = tr.dev;
       for (int sd = 0; sd < 2; ++sd) {
@@ -1142,27 +1162,32 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
         for (int l = tr.depth; l >= 0; --l)
           for (int64_t p : tr.side[sd].nonleaf_by_level[l]) {
             const int64_t nc = tr.side[sd].pairs[p].ncols;
-            if (nc <= 2 * (int64_t)seg_cols) continue;
-            const int64_t nseg = (nc + seg_cols - 1) / seg_cols, rc = D->rowcap_h[sd][p];
-            so[p] = seg_elems;
-            seg_elems += nseg * rc * rc;
+            const int64_t nseg = seg_cols > 0 ? (nc + seg_cols - 1) / seg_cols : 0, rc = D->rowcap_h[sd][p];
+            if (nc <= 2 * (int64_t)seg_cols || (gram && rc <= kGramRows)) continue;
+            so[p] = lvl_elems[l];
+            lvl_elems[l] += nseg * rc * rc;
             const uint32_t code = ((uint32_t)i << kCodeProbShift) | ((uint32_t)sd << kCodeSideShift) | (uint32_t)p;
             for (int64_t s = 0; s < nseg; ++s) seg_lists[l].push_back(((uint64_t)code << 32) | (uint64_t)s);
           }
       }
     }
-  size_t seg_bytes = 0;
-  if (seg_elems > 0) {
+    seg_elems = *std::max_element(lvl_elems.begin(), lvl_elems.end());
+    seg_bytes = 0;
+    if (seg_elems == 0) return;
     seg_bytes += align256(sizeof(C2<T>) * (size_t)seg_elems);
     for (const auto& v : seg_off_h) seg_bytes += align256(8 * std::max<size_t>(v.size(), 1));
     for (const auto& v : seg_lists) seg_bytes += 5 * align256(8 * v.size()) + align256(16);  // list, 4 classes, counts
-  }
+  };
   void* scratch = nullptr;
-  const size_t scratch_bytes = args_bytes + codes_bytes + cls_bytes + host_bytes + gram_bytes + ovr_bytes + part_bytes +
-                               seg_bytes + 256;  // the last 256 bytes: a batch's combined status
-  if (dev_malloc_async(&scratch, scratch_bytes, st) != cudaSuccess) {
+  size_t scratch_bytes = 0;
+  for (;; gram = false) {  // without room for the Gram matrices: the LQ, which needs none
+    gram_layout();
+    seg_layout();
+    scratch_bytes = args_bytes + codes_bytes + cls_bytes + host_bytes + gram_bytes + ovr_bytes + part_bytes + seg_bytes +
+                    256;  // the last 256 bytes: a batch's combined status
+    if (dev_malloc_async(&scratch, scratch_bytes, st) == cudaSuccess) break;
     cudaGetLastError();
-    return DH2_ENOMEM;
+    if (!gram) return DH2_ENOMEM;
   }
   char* const gram_base = (char*)scratch + args_bytes + codes_bytes + cls_bytes + host_bytes;
   char* const ovr_base = gram_base + gram_bytes;
@@ -1211,7 +1236,7 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
     }
   }
   std::vector<GramArgs> gas;
-  for (int i = 0; i < nprob && f32; ++i) {
+  for (int i = 0; i < nprob && (gram || mixed); ++i) {
     pas[i].H = Ms[i]->gram ? (float4*)Ms[i]->gram : (float4*)(gram_base + gram_h_off[i]);
     pas[i].L4 = Ms[i]->gram ? (float4*)(gram_base + gram_l_off[i]) : pas[i].H;
     pas[i].Hl = (float4*)(gram_base + gram_lvl_off[i]);
@@ -1403,13 +1428,13 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
     if (n <= 0) return;
     const int P = even_up(std::max(2, cls_maxm[c]));
     if constexpr (f32) {
-      if (mixed || cls_maxm[c] <= kGramRows) {
+      if (mixed || (gram && cls_maxm[c] <= kGramRows)) {
         if (timed) cudaEventRecord(kev[4 * c], st);
         if (mixed) {
           ok_launch &= launch_gram(d_ga, codes, n, cls_maxm[c], st);  // row scales, then the Gram matrices
           counted(DH2_KC_GRAM_SCALES, true);
         } else {
-          ok_launch &= launch_gram_i64(d_pa, codes, nullptr, n, P, st);
+          ok_launch &= launch_gram_i64(d_pa, codes, nullptr, n, P, 0, st);
         }
         counted(DH2_KC_LEAF_GRAM + c, true);
         if (timed) cudaEventRecord(kev[4 * c + 1], st);
@@ -1522,7 +1547,7 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
         kev_ok = cudaEventCreate(&kev[i]) == cudaSuccess;
       if (!kev_ok) cudaGetLastError();  // no split timing; the compression itself goes on
     }
-    const int one_cls = merged_jacobi(f32, mixed, cls_begin, cls_maxm);
+    const int one_cls = merged_jacobi(gram || mixed, mixed, cls_begin, cls_maxm);
     for (int c = 0; c < kLeafClasses; ++c)
       leaf_factor(d_leaf + cls_begin[c], (int)(cls_begin[c + 1] - cls_begin[c]), c,
                   kev_ok && cls_begin[c + 1] > cls_begin[c], c > one_cls);
@@ -1607,15 +1632,18 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
         ok_launch = false;
       }
       // few pairs: their row classes' longest run side by side in one launch
-      const bool merge = f32 && n <= kOneLevel;
+      const bool merge = gram && n <= kOneLevel;
       launch_classify<T>(d_pa, d_nl[l], n, d_cls, d_cnt, merge, st);
       counted(DH2_KC_CLASSIFY, true);
       const int Pc[4] = {32, 48, 64, P_level[l]};
       // FP32: pairs of at most kGramRows rows from the Gram matrices of their
       // column segments; the LQ launches take the others
-      const int c_lq = f32 ? 3 : 0;
-      if constexpr (f32) {
-        ok_launch &= launch_gram_i64(d_pa, nullptr, d_gseg[l], (int)n_gseg[l], P_level[l], st);
+      const int c_lq = gram ? 3 : 0;
+      if constexpr (f32) if (gram) {
+        int w = 0;
+        for (const dh2_matrix* M : Ms)
+          if (l <= M->tree->tr.depth) w = std::max(w, M->tree->tr.dev->gseg_cols_h[l]);
+        ok_launch &= launch_gram_i64(d_pa, nullptr, d_gseg[l], (int)n_gseg[l], P_level[l], w, st);
         counted(DH2_KC_LEVEL_FACTOR, true);
         for (int c = merge ? 2 : 0; c < 3; ++c) {
           if (!merge && c > 0 && Pc[c - 1] >= P_level[l]) break;  // no pair of this level has more rows
@@ -1629,7 +1657,7 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
         }
       }
       // wide pairs: their column segments' factors first, by row class
-      const int nsg = P_level[l] > (f32 ? kGramRows : 0) ? (int)seg_lists[l].size() : 0;
+      const int nsg = P_level[l] > (gram ? kGramRows : 0) ? (int)seg_lists[l].size() : 0;
       if (nsg > 0) {
         if (cudaMemsetAsync(d_seg_cnt[l], 0, 4 * sizeof(int), st) != cudaSuccess) {
           cudaGetLastError();

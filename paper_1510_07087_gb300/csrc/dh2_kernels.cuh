@@ -237,6 +237,7 @@ struct PairArgs {
   // pair's (one per column segment, mp x mp each) in Hl, from its level's start
   const int64_t* hoff[2];
   float4* Hl;
+  const int32_t* gseg_cols;           // per level: columns of a non-leaf pair's Gram segment
   const int32_t* rank_ovr[2];         // per pair a rank replacing the truncation rule (< 0: the rule), or NULL
   int32_t max_sweeps;
   int32_t jacobi_tpp[5];              // per factor class: most threads per Jacobi column pair (TuneTable)
@@ -276,12 +277,17 @@ bool launch_gram_jacobi(const PairArgs<float>* args_dev, const uint32_t* codes, 
                         cudaStream_t st, const int* count = nullptr);
 
 // H = A A^* from products of fixed-point integers on the integer pipe, FP32
-// mode's leaf pairs (codes) or a level's pairs by segments of kGramSegCols
-// columns (segs: code << 32 | segment; pairs above kGramRows rows are left to
-// the LQ launches).  P: most rows of the list.
-constexpr int kGramSegCols = 256;
+// mode's leaf pairs (codes) or a level's pairs by segments of their level's
+// gseg_cols columns (segs: code << 32 | segment; pairs above kGramRows rows are
+// left to the LQ launches).  P: most rows of the list.  A level's segments are
+// kGramSegCols columns wide, or the first doubling of that with at most
+// kGramSegMax segments beside one per pair: a matrix of up to 64 KB each, so
+// that the scratch stays a few hundred MB (n = 32768, paper's parameters, 256
+// columns throughout: 3.3 GB) with some ten waves of CTAs.
+constexpr int kGramSegCols = 256, kGramSegMax = 4096;
+// seg_cols: of the segments, at most.
 bool launch_gram_i64(const PairArgs<float>* args_dev, const uint32_t* codes, const uint64_t* segs, int n, int P,
-                     cudaStream_t st);
+                     int seg_cols, cudaStream_t st);
 
 // R = Q^* A for the pairs of a pair-kernel launch, after it, by tiles of 32
 // columns, tiles[i] = launch code << 32 | first column (P as for the pair

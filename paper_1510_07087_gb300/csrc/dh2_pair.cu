@@ -1184,7 +1184,7 @@ __global__ void __launch_bounds__(NT, (GRAM ? gram_min_blocks<NT>() : pair_min_b
     // (a non-leaf pair's L goes over its first segment's H, read by then)
     const float4* Hin = (FROM_R ? a.Hl : a.H) + a.hoff[side][pid];
     gram_cholesky<T, NT, LPR>(a, side, pid, p, P, row, q, live, drop * a.eps2[lvl], Hin,
-                              FROM_R ? (N + kGramSegCols - 1) / kGramSegCols : 1,
+                              FROM_R ? (N + a.gseg_cols[lvl] - 1) / a.gseg_cols[lvl] : 1,
                               reinterpret_cast<C2<T>*>((FROM_R ? a.Hl : a.L4) + a.hoff[side][pid]), Hs, nu, dlo, piv,
                               pcol, K, E_K);
 #if DH2_PROF_ON
@@ -1745,8 +1745,10 @@ __host__ __device__ constexpr int gram_i64_ld(int p) {  // rows in fours, an odd
 }
 constexpr int kGramI64Chunk = 64;
 constexpr int kGramI64Flush = 512;
-static_assert(kGramSegCols <= kGramI64Flush && kGramI64Flush % kGramI64Chunk == 0, "a level pair's segment is one sum");
-template <bool FROM_R, int NT>
+static_assert(kGramSegCols % kGramI64Chunk == 0 && kGramI64Flush % kGramI64Chunk == 0, "whole chunks");
+// WIDE: more than kGramI64Flush columns are possible (without the flush no
+// registers are spilled: plan of n = 8191, paper's parameters, 6.88 -> 6.56 ms)
+template <bool FROM_R, int NT, bool WIDE>
 __global__ void __launch_bounds__(NT, NT <= 128 ? 4 : 3)
     gram_i64_kernel(const PairArgs<float>* __restrict__ args, const uint32_t* __restrict__ codes,
                     const uint64_t* __restrict__ segs, const int P) {
@@ -1775,15 +1777,16 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 4 : 3)
     if (!DH2_IN(s0, c_lim.npairs[side], 12, pid) || !DH2_IN(s1, c_lim.npairs[side], 13, pid)) return;
     src.k1 = a.rank[side][s0];
     p = src.k1 + a.rank[side][s1];
-    src.off0 = a.sonoff[side][2 * pid] + seg * kGramSegCols;
-    src.off1 = a.sonoff[side][2 * pid + 1] + seg * kGramSegCols;
+    const int W = a.gseg_cols[a.level[side][pid]];
+    src.off0 = a.sonoff[side][2 * pid] + seg * W;
+    src.off1 = a.sonoff[side][2 * pid + 1] + seg * W;
     src.ld0 = a.kcap[side][s0];
     src.ld1 = a.kcap[side][s1];
     src.roff0 = a.Roff[side][s0];
     src.roff1 = a.Roff[side][s1];
     src.R0 = a.R[side] + src.roff0;
     src.R1 = a.R[side] + src.roff1;
-    N = min(kGramSegCols, N - seg * kGramSegCols);
+    N = min(W, N - seg * W);
   } else {
     p = a.m[side][pid];
     src.r0 = a.start[side][pid];
@@ -1912,13 +1915,13 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 4 : 3)
     // flush after this chunk?  Looked at every kGramI64Flush columns, which add at
     // most 2^62 to a sum: those of 2^61 at one look stay below 2^63 beyond the next
     bool big = false;
-    if (!FROM_R && more && (j0 + CW) % kGramI64Flush == 0 && grp < G && ti == tj)
+    if (WIDE && more && (j0 + CW) % kGramI64Flush == 0 && grp < G && ti == tj)
 #pragma unroll
       for (int i = 0; i < 4; ++i) big = big || ar[i][i] > (1ll << 61) / G;
     // this chunk has landed; the other buffer's products are done
     bool full = false;
-    if constexpr (FROM_R) __syncthreads();
-    else full = __syncthreads_or(big);
+    if constexpr (WIDE) full = __syncthreads_or(big);
+    else __syncthreads();
     if (more && !gen && !full) entries(j0 + CW, s ^ 1);
     if (scan) {
       int m = 0;  // largest |re|, |im| as bits (NaN and infinity above every finite value)
@@ -2543,22 +2546,23 @@ bool launch_pair_kernel(const PairArgs<T>* args, const uint32_t* codes, int nblo
   return launch_one<T, 128, true, 256>(args, codes, nblocks, P, st, count, segs);
 }
 
-template <bool FROM_R, int NT>
+template <bool FROM_R, int NT, bool WIDE>
 bool launch_i64(const PairArgs<float>* args, const uint32_t* codes, const uint64_t* segs, int n, int P,
                 cudaStream_t st) {
-  auto kern = gram_i64_kernel<FROM_R, NT>;
+  auto kern = gram_i64_kernel<FROM_R, NT, WIDE>;
   const size_t smem = 2 * (size_t)kGramI64Chunk * gram_i64_ld(P) * sizeof(int2);
   if (!set_smem(kern, smem)) return false;
   kern<<<n, NT, smem, st>>>(args, codes, segs, P);
   return true;
 }
 bool launch_gram_i64(const PairArgs<float>* args, const uint32_t* codes, const uint64_t* segs, int n, int P,
-                     cudaStream_t st) {
+                     int seg_cols, cudaStream_t st) {
   if (n <= 0) return true;
   P = std::min(P, kGramRows);
   // 55 tiles at 40 rows fill 110 of 128 threads; 78 at 48 rows 156 of 160, 136 at 64
-  if (P <= 40) return segs ? launch_i64<true, 128>(args, codes, segs, n, P, st) : launch_i64<false, 128>(args, codes, segs, n, P, st);
-  return segs ? launch_i64<true, 160>(args, codes, segs, n, P, st) : launch_i64<false, 160>(args, codes, segs, n, P, st);
+  if (!segs) return P <= 40 ? launch_i64<false, 128, true>(args, codes, segs, n, P, st) : launch_i64<false, 160, true>(args, codes, segs, n, P, st);
+  if (seg_cols > kGramI64Flush) return P <= 40 ? launch_i64<true, 128, true>(args, codes, segs, n, P, st) : launch_i64<true, 160, true>(args, codes, segs, n, P, st);
+  return P <= 40 ? launch_i64<true, 128, false>(args, codes, segs, n, P, st) : launch_i64<true, 160, false>(args, codes, segs, n, P, st);
 }
 
 // The Jacobi launch of a class: NT = 4 x rows threads per CTA, or (the
