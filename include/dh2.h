@@ -463,7 +463,9 @@ dh2_status dh2_matrix_launch_count(const dh2_matrix* M, int32_t* launches);
 /* Kernel classes of dh2_matrix_class_launches (instrumentation only; the paper
  * has no counterpart).  A factor kernel's class is its row class: leaf pairs by
  * cluster size (0: <= 32, 1: <= 40, 2: <= 48, 3: <= 64, 4: more rows),
- * non-leaf pairs by k_t1c' + k_t2c' (0: <= 32, 1: <= 48, 2: <= 64, 3: more). */
+ * non-leaf pairs by k_t1c' + k_t2c' (0: <= 32, 1: <= 48, 2: <= 64, 3: more).
+ * A launch that takes the pairs of several classes (few pairs) counts in each of
+ * them. */
 enum {
   DH2_KC_LEAF_FACTOR = 0,   /* + leaf row class 0..4: leaf factorisation (Section 6, leaf step)  */
   DH2_KC_LEAF_R = 5,        /* + leaf row class 0..4: R_tc = Q_tc^* G^omega_tc                   */
@@ -478,6 +480,7 @@ enum {
   DH2_KC_GRAM_SCALES = 24,  /* row scales of the leaf Gram matrices (MIXED_BF16X3)               */
   DH2_KC_LEAF_JACOBI = 25,  /* + leaf row class 0..3: Jacobi, rank and Q after the Cholesky (MIXED, FP32) */
   DH2_KC_LEAF_R_TC = 29,    /* leaf R_tc = Q_tc^* G^omega_tc on the tensor cores, all classes (MIXED) */
+  DH2_KC_LEVEL_GRAM = 30,   /* Gram matrices of a level's pairs, all classes (MIXED, FP32)       */
   DH2_KC_COUNT = 32
 };
 /* Launches of the last compression that produced M, by kernel class

@@ -37,6 +37,7 @@ KC_LEAF_GRAM = 20
 KC_GRAM_SCALES = 24
 KC_LEAF_JACOBI = 25
 KC_LEAF_R_TC = 29
+KC_LEVEL_GRAM = 30
 KC_GRAM_SCALES = 24
 KC_COUNT = 32
 

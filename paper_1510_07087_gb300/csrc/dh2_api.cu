@@ -1556,6 +1556,7 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
         ok_launch &= launch_gram_jacobi(d_pa, d_leaf, (int)cls_begin[one_cls + 1],
                                         even_up(std::max(2, cls_maxm[one_cls])), false, st);
         counted(DH2_KC_LEAF_JACOBI + one_cls, true);
+        for (int c = 0; c < one_cls; ++c) kcl[DH2_KC_LEAF_JACOBI + c] += cls_begin[c + 1] > cls_begin[c];
         if (kev_ok) cudaEventRecord(kev[4 * one_cls + 3], st);
       }
     rec(2);
@@ -1644,7 +1645,7 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
         for (const dh2_matrix* M : Ms)
           if (l <= M->tree->tr.depth) w = std::max(w, M->tree->tr.dev->gseg_cols_h[l]);
         ok_launch &= launch_gram_i64(d_pa, nullptr, d_gseg[l], (int)n_gseg[l], P_level[l], w, st);
-        counted(DH2_KC_LEVEL_FACTOR, true);
+        counted(DH2_KC_LEVEL_GRAM, true);
         for (int c = merge ? 2 : 0; c < 3; ++c) {
           if (!merge && c > 0 && Pc[c - 1] >= P_level[l]) break;  // no pair of this level has more rows
           const int P = std::min(Pc[c], std::max(P_level[l], 2));
@@ -1653,7 +1654,7 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
           counted(DH2_KC_LEVEL_FACTOR + c, true);
           counted(DH2_KC_LEVEL_FACTOR + c, true);
           for (int m = 0; merge && m < 2; ++m)  // a launch over several classes counts in each of them
-            if (m == 0 || Pc[m - 1] < P_level[l]) ++kcl[DH2_KC_LEVEL_FACTOR + m];
+            if (m == 0 || Pc[m - 1] < P_level[l]) kcl[DH2_KC_LEVEL_FACTOR + m] += 2;
         }
       }
       // wide pairs: their column segments' factors first, by row class
