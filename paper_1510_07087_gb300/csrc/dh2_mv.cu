@@ -8,6 +8,8 @@
 //
 // Right-hand sides are taken NR at a time from one read of the matrix; a
 // chunk's unused slots (nr < NR) repeat slot 0 and are not written.
+#include <algorithm>
+
 #include "dh2_check.cuh"
 #include "dh2_internal.h"
 #include "dh2_ops.cuh"
@@ -84,6 +86,13 @@ struct Rhs {
   }
 };
 
+// A launch takes right-hand sides [first, first + count), NR per blockIdx.y: the
+// first of this CTA's, and how many it has.
+template <int NR>
+__device__ __forceinline__ int chunk_begin(int rh0) { return rh0 + blockIdx.y * NR; }
+template <int NR>
+__device__ __forceinline__ int chunk_width(int count) { return min(NR, count - (int)blockIdx.y * NR); }
+
 // ---------------------------------------------------------------- nearfield
 // y|_t += G_b x|_s over the inadmissible blocks (ADJ: y|_s += G_b^* x|_t), a
 // unit (a slab of one row cluster's rows, or of one column cluster's columns,
@@ -120,9 +129,10 @@ template <typename T, int NR>
 __device__ __forceinline__ void leaf_unit(const MvArgs<T>& a, const int32_t* __restrict__ pairs, const NearUnit& u,
                                           int rh0, int nr, int nrhs, C2<T>* __restrict__ y, int64_t n, C2<T>* red);
 template <typename T, int NR, bool ADJ>
-__global__ void __launch_bounds__(128) mv_near(MvArgs<T> a, int rh0, int nr, const C2<T>* __restrict__ x,
+__global__ void __launch_bounds__(128) mv_near(MvArgs<T> a, int first, int count, const C2<T>* __restrict__ x,
                                                C2<T>* __restrict__ y, int64_t n, const int32_t* __restrict__ pairs,
                                                const NearUnit* __restrict__ leafs, int nrhs) {
+  const int rh0 = chunk_begin<NR>(first), nr = chunk_width<NR>(count);
   // stages (static shared memory, below 48 KB); FP64 takes half a piece at a time
   constexpr int S = NR <= 4 ? 3 : 2;
   constexpr int SG = kNearElems * 4 / (int)sizeof(T), SX = kNearPiece * NR * 4 / (int)sizeof(T);
@@ -192,12 +202,13 @@ __global__ void __launch_bounds__(128) mv_near(MvArgs<T> a, int rh0, int nr, con
       if (qi + 1 < u.count) nx = items[qi + 1];
     }
   };
-  // sums in two steps: of a piece (FP64, where the additions cost pipe time: of
-  // eight half pieces), and of those.  One chain over the unit's ~1600 columns had
+  // sums in two steps: of a piece (where the additions cost pipe time, of several:
+  // 5 to 8 vectors in FP32 four, 12% slower by single ones; FP64 eight half
+  // pieces), and of those.  One chain over the unit's ~1600 columns had
   // 1.2 to 1.7 times the rounding error of block after block (n = 8192, leaf 64,
   // against FP64: 4.7e-7, by block 2.7e-7, now 1.5e-7), for 1% of the time in
   // FP32 (n = 32768, one vector: 1162 -> 1171 us)
-  constexpr int FOLD = sizeof(T) == 4 ? 1 : 8;
+  constexpr int FOLD = sizeof(T) == 8 ? 8 : NR < 8 ? 1 : 4;
   C2<T> acc[NR], sum[NR];
 #pragma unroll
   for (int k = 0; k < NR; ++k) acc[k] = sum[k] = czero<T>();
@@ -286,11 +297,12 @@ __device__ __forceinline__ void cols_dot(const C2<T>* M, int ld, int p, int k, i
 // pair; y0 (nzero entries, or NULL): a small product's result, zeroed on the way
 template <typename T, int NR>
 __global__ void __launch_bounds__(128) mv_forward_leaf(SideView<T> W, const int32_t* __restrict__ pairs, int np,
-                                                       int rh0, int nr, const C2<T>* __restrict__ x, int nrhs,
+                                                       int first, int count, const C2<T>* __restrict__ x, int nrhs,
                                                        int64_t n, C2<T>* __restrict__ xh,
                                                        const int64_t* __restrict__ hoff, C2<T>* __restrict__ y0,
                                                        int64_t nzero) {
-  if (y0)
+  const int rh0 = chunk_begin<NR>(first), nr = chunk_width<NR>(count);
+  if (y0 && blockIdx.y == 0)
     for (int64_t i = blockIdx.x * (int64_t)128 + threadIdx.x; i < nzero; i += (int64_t)gridDim.x * 128)
       y0[i] = czero<T>();
   const int w = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -316,8 +328,9 @@ __global__ void __launch_bounds__(128) mv_forward_leaf(SideView<T> W, const int3
 // forward transformation, non-leaves: xh_sc = [E_s1c; E_s2c]^* [xh_s1c'; xh_s2c'],
 // one CTA per pair, its warps take 8 columns each
 template <typename T, int NR>
-__global__ void __launch_bounds__(128) mv_forward_up(SideView<T> W, const int32_t* __restrict__ pairs, int rh0, int nr,
+__global__ void __launch_bounds__(128) mv_forward_up(SideView<T> W, const int32_t* __restrict__ pairs, int first, int count,
                                                      int nrhs, C2<T>* xh, const int64_t* __restrict__ hoff) {
+  const int rh0 = chunk_begin<NR>(first), nr = chunk_width<NR>(count);
   const int pid = pairs[blockIdx.x];
   const int lane = threadIdx.x & 31;
   const int k = W.rank[pid];
@@ -391,7 +404,8 @@ struct OwnWalk {
 // Bound by the latency of a block's few loads (a pair has 8 blocks on average;
 // one warp per pair took 185 us at n = 32768, four 138).
 template <typename T, int NR>
-__global__ void __launch_bounds__(128) mv_coupling(MvArgs<T> a, int rh0, int nr, int nrhs) {
+__global__ void __launch_bounds__(128) mv_coupling(MvArgs<T> a, int first, int count, int nrhs) {
+  const int rh0 = chunk_begin<NR>(first), nr = chunk_width<NR>(count);
   __shared__ C2<T> red[4][32 * NR];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int pid = blockIdx.x;
@@ -436,7 +450,8 @@ __global__ void __launch_bounds__(128) mv_coupling(MvArgs<T> a, int rh0, int nr,
 // adjoint coupling: yh_sc = sum over the column pair's blocks b of S_b^* xh_tc;
 // in a warp two lanes per column of S_b and 16 columns per pass
 template <typename T, int NR>
-__global__ void __launch_bounds__(128) mv_coupling_adj(MvArgs<T> a, int rh0, int nr, int nrhs) {
+__global__ void __launch_bounds__(128) mv_coupling_adj(MvArgs<T> a, int first, int count, int nrhs) {
+  const int rh0 = chunk_begin<NR>(first), nr = chunk_width<NR>(count);
   __shared__ C2<T> red[4][16 * NR];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int pid = blockIdx.x;
@@ -489,7 +504,8 @@ __global__ void __launch_bounds__(128) mv_coupling_adj(MvArgs<T> a, int rh0, int
 // lanes as in the coupling (above 32 rows a lane takes every 32nd row)
 template <typename T, int NR>
 __global__ void __launch_bounds__(128) mv_backward_down(MvArgs<T> a, const int32_t* __restrict__ pairs, int np,
-                                                        int rh0, int nr, int nrhs) {
+                                                        int first, int count, int nrhs) {
+  const int rh0 = chunk_begin<NR>(first), nr = chunk_width<NR>(count);
   __shared__ C2<T> red[4][32 * NR];
   const int wl = threadIdx.x >> 5, w = blockIdx.x * 4 + wl, lane = threadIdx.x & 31;
   if (w >= np) return;
@@ -576,44 +592,54 @@ __device__ __forceinline__ void leaf_unit(const MvArgs<T>& a, const int32_t* __r
 }
 template <typename T, int NR>
 __global__ void __launch_bounds__(128) mv_backward_leaf(MvArgs<T> a, const int32_t* __restrict__ pairs,
-                                                        const NearUnit* __restrict__ units, int rh0, int nr, int nrhs,
-                                                        C2<T>* __restrict__ y, int64_t n) {
+                                                        const NearUnit* __restrict__ units, int first, int count,
+                                                        int nrhs, C2<T>* __restrict__ y, int64_t n) {
+  const int rh0 = chunk_begin<NR>(first), nr = chunk_width<NR>(count);
   __shared__ C2<T> red[128 * NR];
   leaf_unit<T, NR>(a, pairs, units[blockIdx.x], rh0, nr, nrhs, y, n, red);
 }
 
-// The right-hand sides in chunks of a compiled width: f(width constant, first,
-// count).  MOST: the widest kernel that keeps its sums in registers.  FP32
+// The right-hand sides in chunks of a compiled width, those of one width in one
+// launch: f(width constant, first, count), chunk blockIdx.y of the launch's
+// columns [first, first + count).  (One launch per chunk took n = 2000, sixteen
+// vectors, 146 us; every vector in one launch of the old kernels 126.)  MOST: the
+// widest kernel that keeps its sums in registers.  FP32
 // rounds 5 to 7 up to 8 (one read of the matrix; the extra multiply-adds cost
 // less than a second read); FP64 takes exact widths (they would cost the narrow
 // FP64 pipe).
+template <int NR>
+dim3 chunk_grid(int x, int count) { return dim3((unsigned)x, (unsigned)((count + NR - 1) / NR)); }
 template <int V>
 struct Int {
   static constexpr int value = V;
 };
+constexpr int kMaxChunks = 65535;  // a grid's y extent
 template <typename T, int MOST, typename F>
-void rhs_chunks(int nrhs, const F& f) {
+void rhs_chunks(int nrhs, const F& f, int most = MOST) {
+  constexpr int UP = sizeof(T) == 4 ? 3 : 0;  // columns a chunk of 8 may lack
   for (int rh = 0; rh < nrhs;) {
     const int left = nrhs - rh;
     int nr;
-    if (MOST >= 8 && left >= (sizeof(T) == 4 ? 5 : 8)) {
-      nr = left < 8 ? left : 8;
+    if (MOST >= 8 && most >= 8 && left >= 8 - UP) {
+      const int64_t full = (left + (int64_t)UP) / 8;
+      nr = (int)std::min<int64_t>(left, 8 * std::min<int64_t>(full, kMaxChunks));
       f(Int<(MOST >= 8 ? 8 : 1)>{}, rh, nr);
-    } else if (MOST >= 4 && left >= 3) {
-      nr = left < 4 ? left : 4;
-      if (nr == 4) f(Int<(MOST >= 4 ? 4 : 1)>{}, rh, nr);
-      else f(Int<(MOST >= 4 ? 3 : 1)>{}, rh, nr);
-    } else if (left >= 2) {
-      nr = 2;
+    } else if (MOST >= 4 && most >= 4 && left >= 4) {
+      nr = 4 * std::min(left / 4, kMaxChunks);
+      f(Int<(MOST >= 4 ? 4 : 1)>{}, rh, nr);
+    } else if (MOST >= 4 && most >= 4 && left == 3) {
+      nr = 3;
+      f(Int<(MOST >= 4 ? 3 : 1)>{}, rh, nr);
+    } else if (most >= 2 && left >= 2) {
+      nr = 2 * std::min(left / 2, kMaxChunks);
       f(Int<2>{}, rh, nr);
     } else {
-      nr = 1;
+      nr = std::min(left, kMaxChunks);
       f(Int<1>{}, rh, nr);
     }
     rh += nr;
   }
 }
-
 // ---------------------------------------------------------------- lists
 // items: one thread per inadmissible block, at the next free place of its
 // cluster (a cluster's blocks are summed, so their order is free)
@@ -670,7 +696,8 @@ void launch_mv_forward_leaf(const SideView<T>& W, const int32_t* pairs, int np, 
   if (np <= 0) return;
   rhs_chunks<T, sizeof(T) == 4 ? 4 : 2>(nrhs, [&](auto w, int rh, int nr) {
     mv_forward_leaf<T, decltype(w)::value>
-        <<<(np + 3) / 4, 128, 0, st>>>(W, pairs, np, rh, nr, x, nrhs, n, xh, hoff, rh == 0 ? y0 : nullptr, n * nrhs);
+        <<<chunk_grid<decltype(w)::value>((np + 3) / 4, nr), 128, 0, st>>>(W, pairs, np, rh, nr, x, nrhs, n, xh, hoff,
+                                                                          rh == 0 ? y0 : nullptr, n * nrhs);
   });
 }
 template <typename T>
@@ -678,28 +705,30 @@ void launch_mv_forward_up(const SideView<T>& W, const int32_t* pairs, int np, in
                           const int64_t* hoff, cudaStream_t st) {
   if (np <= 0) return;
   rhs_chunks<T, sizeof(T) == 4 ? 4 : 2>(nrhs, [&](auto w, int rh, int nr) {
-    mv_forward_up<T, decltype(w)::value><<<np, 128, 0, st>>>(W, pairs, rh, nr, nrhs, xh, hoff);
+    mv_forward_up<T, decltype(w)::value>
+        <<<chunk_grid<decltype(w)::value>(np, nr), 128, 0, st>>>(W, pairs, rh, nr, nrhs, xh, hoff);
   });
 }
 template <typename T>
 void launch_mv_coupling(const MvArgs<T>& a, int npairs_row, int nrhs, cudaStream_t st) {
   if (npairs_row <= 0) return;
   rhs_chunks<T, 8>(nrhs, [&](auto w, int rh, int nr) {
-    mv_coupling<T, decltype(w)::value><<<npairs_row, 128, 0, st>>>(a, rh, nr, nrhs);
+    mv_coupling<T, decltype(w)::value><<<chunk_grid<decltype(w)::value>(npairs_row, nr), 128, 0, st>>>(a, rh, nr, nrhs);
   });
 }
 template <typename T>
 void launch_mv_coupling_adj(const MvArgs<T>& a, int npairs_col, int nrhs, cudaStream_t st) {
   if (npairs_col <= 0) return;
   rhs_chunks<T, 8>(nrhs, [&](auto w, int rh, int nr) {
-    mv_coupling_adj<T, decltype(w)::value><<<npairs_col, 128, 0, st>>>(a, rh, nr, nrhs);
+    mv_coupling_adj<T, decltype(w)::value><<<chunk_grid<decltype(w)::value>(npairs_col, nr), 128, 0, st>>>(a, rh, nr, nrhs);
   });
 }
 template <typename T>
 void launch_mv_backward_down(const MvArgs<T>& a, const int32_t* pairs, int np, int nrhs, cudaStream_t st) {
   if (np <= 0) return;
   rhs_chunks<T, 8>(nrhs, [&](auto w, int rh, int nr) {
-    mv_backward_down<T, decltype(w)::value><<<(np + 3) / 4, 128, 0, st>>>(a, pairs, np, rh, nr, nrhs);
+    mv_backward_down<T, decltype(w)::value>
+        <<<chunk_grid<decltype(w)::value>((np + 3) / 4, nr), 128, 0, st>>>(a, pairs, np, rh, nr, nrhs);
   });
 }
 template <typename T>
@@ -707,7 +736,8 @@ void launch_mv_backward_leaf(const MvArgs<T>& a, const int32_t* pairs, const Nea
                              C2<T>* y, int64_t n, cudaStream_t st) {
   if (nunits <= 0) return;
   rhs_chunks<T, 8>(nrhs, [&](auto w, int rh, int nr) {
-    mv_backward_leaf<T, decltype(w)::value><<<nunits, 128, 0, st>>>(a, pairs, units, rh, nr, nrhs, y, n);
+    mv_backward_leaf<T, decltype(w)::value>
+        <<<chunk_grid<decltype(w)::value>(nunits, nr), 128, 0, st>>>(a, pairs, units, rh, nr, nrhs, y, n);
   });
 }
 template <typename T>
@@ -715,11 +745,17 @@ void launch_mv_near(const MvArgs<T>& a, bool adj, int nrhs, const C2<T>* x, C2<T
                     const int32_t* pairs, const NearUnit* leafs, int nleafs, cudaStream_t st) {
   const int grid = a.nunits + nleafs;
   if (grid <= 0) return;
+  // FP64, bound by its pipe: as narrow chunks as give every SM two CTAs (reading
+  // the matrix, then small, again from L2).  n = 400, seven vectors: 54 -> 25 us;
+  // two: 22 -> 18
+  int most = 8;
+  while (sizeof(T) == 8 && most > 1 && (int64_t)grid * ((nrhs + most - 1) / most) < 2 * 152) most /= 2;
+  if (most < 8 && nrhs % most != 0) most = 1;  // one launch instead of two, each of too few CTAs
   rhs_chunks<T, 8>(nrhs, [&](auto w, int rh, int nr) {
     constexpr int NR = decltype(w)::value;
-    if (adj) mv_near<T, NR, true><<<grid, 128, 0, st>>>(a, rh, nr, x, y, n, pairs, leafs, nrhs);
-    else mv_near<T, NR, false><<<grid, 128, 0, st>>>(a, rh, nr, x, y, n, pairs, leafs, nrhs);
-  });
+    if (adj) mv_near<T, NR, true><<<chunk_grid<NR>(grid, nr), 128, 0, st>>>(a, rh, nr, x, y, n, pairs, leafs, nrhs);
+    else mv_near<T, NR, false><<<chunk_grid<NR>(grid, nr), 128, 0, st>>>(a, rh, nr, x, y, n, pairs, leafs, nrhs);
+  }, most);
 }
 
 #define DH2_MV_INST(T)                                                                                      \
