@@ -1434,7 +1434,7 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
           ok_launch &= launch_gram(d_ga, codes, n, cls_maxm[c], st);  // row scales, then the Gram matrices
           counted(DH2_KC_GRAM_SCALES, true);
         } else {
-          ok_launch &= launch_gram_i64(d_pa, codes, nullptr, n, P, 0, st);
+          ok_launch &= launch_gram_i64(d_pa, codes, nullptr, n, P, 0, any_gen, st);
         }
         counted(DH2_KC_LEAF_GRAM + c, true);
         if (timed) cudaEventRecord(kev[4 * c + 1], st);
@@ -1644,7 +1644,7 @@ dh2_status run_compress(std::vector<dh2_matrix*>& Ms, const dh2_compress_params&
         int w = 0;
         for (const dh2_matrix* M : Ms)
           if (l <= M->tree->tr.depth) w = std::max(w, M->tree->tr.dev->gseg_cols_h[l]);
-        ok_launch &= launch_gram_i64(d_pa, nullptr, d_gseg[l], (int)n_gseg[l], P_level[l], w, st);
+        ok_launch &= launch_gram_i64(d_pa, nullptr, d_gseg[l], (int)n_gseg[l], P_level[l], w, false, st);
         counted(DH2_KC_LEVEL_GRAM, true);
         for (int c = merge ? 2 : 0; c < 3; ++c) {
           if (!merge && c > 0 && Pc[c - 1] >= P_level[l]) break;  // no pair of this level has more rows

@@ -287,7 +287,7 @@ bool launch_gram_jacobi(const PairArgs<float>* args_dev, const uint32_t* codes, 
 constexpr int kGramSegCols = 256, kGramSegMax = 4096;
 // seg_cols: of the segments, at most.
 bool launch_gram_i64(const PairArgs<float>* args_dev, const uint32_t* codes, const uint64_t* segs, int n, int P,
-                     int seg_cols, cudaStream_t st);
+                     int seg_cols, bool gen, cudaStream_t st);
 
 // R = Q^* A for the pairs of a pair-kernel launch, after it, by tiles of 32
 // columns, tiles[i] = launch code << 32 | first column (P as for the pair

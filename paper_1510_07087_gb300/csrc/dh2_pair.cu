@@ -1748,7 +1748,7 @@ constexpr int kGramI64Flush = 512;
 static_assert(kGramSegCols % kGramI64Chunk == 0 && kGramI64Flush % kGramI64Chunk == 0, "whole chunks");
 // WIDE: more than kGramI64Flush columns are possible (without the flush no
 // registers are spilled: plan of n = 8191, paper's parameters, 6.88 -> 6.56 ms)
-template <bool FROM_R, int NT, bool WIDE>
+template <bool FROM_R, int NT, bool WIDE, bool GEN>
 __global__ void __launch_bounds__(NT, NT <= 128 ? 4 : 3)
     gram_i64_kernel(const PairArgs<float>* __restrict__ args, const uint32_t* __restrict__ codes,
                     const uint64_t* __restrict__ segs, const int P) {
@@ -1796,7 +1796,7 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 4 : 3)
     src.G = a.G;
     src.ld = a.ld;
     src.entry = a.entry;
-    src.gen = a.gen;
+    src.gen = GEN;
   }
   if (p > P || p > kGramRows || p == 0 || N <= 0) return;  // p > kGramRows: an LQ launch's (FROM_R), or reported by the factor launch
   const int mp = (p + 7) & ~7;
@@ -1832,7 +1832,7 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 4 : 3)
   const int r = (warp % RG) * 32 + lane;   // the row this thread scans and converts
   const int c0 = warp / RG, cs = NW / RG;  // its columns c0, c0 + cs, ... (warps past cs * RG idle)
   const bool scan = r < p && c0 < cs;
-  const bool gen = !FROM_R && src.gen;
+  constexpr bool gen = GEN;
   const bool down = FROM_R || side == 0;  // consecutive threads on the contiguous direction
   // the column table of a chunk, and its entries: by cp.async, under the
   // products of the chunk before; generated ones are computed (with their weight)
@@ -1861,20 +1861,30 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 4 : 3)
   bool flushed = false;
   auto store = [&](bool last) {
     longlong2* red = reinterpret_cast<longlong2*>(smem);
-    for (int g = 0; g < G; ++g) {
+    // the last groups' onto those before them, as many at once as have room (small
+    // pairs have up to 128 groups: one by one took 250 barriers)
+    const int room = 4 * LD / ntile, t0 = tid % ntile;
+    auto put = [&](int slot) {
+#pragma unroll
+      for (int u = 0; u < 16; ++u)
+        red[(slot * 16 + u) * ntile + t0] = make_longlong2(ar[u >> 2][u & 3], ai[u >> 2][u & 3]);
+    };
+    __syncthreads();
+    for (int act = G; act > 1;) {
+      const int h = min(act >> 1, room);
+      if (grp >= act - h && grp < act) put(grp - (act - h));
       __syncthreads();
-      if (grp == g)
+      if (grp >= act - 2 * h && grp < act - h)
 #pragma unroll
         for (int u = 0; u < 16; ++u) {
-          longlong2 v = make_longlong2(ar[u >> 2][u & 3], ai[u >> 2][u & 3]);
-          if (g > 0) {
-            const longlong2 w = red[u * ntile + tid % ntile];
-            v.x += w.x;
-            v.y += w.y;
-          }
-          red[u * ntile + tid % ntile] = v;
+          const longlong2 v = red[((grp - (act - 2 * h)) * 16 + u) * ntile + t0];
+          ar[u >> 2][u & 3] += v.x;
+          ai[u >> 2][u & 3] += v.y;
         }
+      __syncthreads();
+      act -= h;
     }
+    if (grp == 0) put(0);
     __syncthreads();
     auto to_df = [](long long v, int ex) {
       const float hi = __ll2float_rn(v);
@@ -2546,20 +2556,21 @@ bool launch_pair_kernel(const PairArgs<T>* args, const uint32_t* codes, int nblo
   return launch_one<T, 128, true, 256>(args, codes, nblocks, P, st, count, segs);
 }
 
-template <bool FROM_R, int NT, bool WIDE>
+template <bool FROM_R, int NT, bool WIDE, bool GEN = false>
 bool launch_i64(const PairArgs<float>* args, const uint32_t* codes, const uint64_t* segs, int n, int P,
                 cudaStream_t st) {
-  auto kern = gram_i64_kernel<FROM_R, NT, WIDE>;
+  auto kern = gram_i64_kernel<FROM_R, NT, WIDE, GEN>;
   const size_t smem = 2 * (size_t)kGramI64Chunk * gram_i64_ld(P) * sizeof(int2);
   if (!set_smem(kern, smem)) return false;
   kern<<<n, NT, smem, st>>>(args, codes, segs, P);
   return true;
 }
 bool launch_gram_i64(const PairArgs<float>* args, const uint32_t* codes, const uint64_t* segs, int n, int P,
-                     int seg_cols, cudaStream_t st) {
+                     int seg_cols, bool gen, cudaStream_t st) {
   if (n <= 0) return true;
   P = std::min(P, kGramRows);
   // 55 tiles at 40 rows fill 110 of 128 threads; 78 at 48 rows 156 of 160, 136 at 64
+  if (!segs && gen) return P <= 40 ? launch_i64<false, 128, true, true>(args, codes, segs, n, P, st) : launch_i64<false, 160, true, true>(args, codes, segs, n, P, st);
   if (!segs) return P <= 40 ? launch_i64<false, 128, true>(args, codes, segs, n, P, st) : launch_i64<false, 160, true>(args, codes, segs, n, P, st);
   if (seg_cols > kGramI64Flush) return P <= 40 ? launch_i64<true, 128, true>(args, codes, segs, n, P, st) : launch_i64<true, 160, true>(args, codes, segs, n, P, st);
   return P <= 40 ? launch_i64<true, 128, false>(args, codes, segs, n, P, st) : launch_i64<true, 160, false>(args, codes, segs, n, P, st);
