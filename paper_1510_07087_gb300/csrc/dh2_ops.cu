@@ -646,10 +646,13 @@ __global__ void __launch_bounds__(256) norms_adm_kernel(const NormsArgs<T>* __re
 }
 
 // The admissible blocks' pass of the matrix-free mode, by the same pieces: the
-// entries are generated and their squares added in FP64 (two operations of the
-// narrow FP64 pipe per entry, under the ~120 instructions that generate it).
-// One warp per block had left the few coarse blocks of millions of entries to
-// one warp each.
+// entries are generated and their squares added in FP64: in FP32 or
+// double-float the squares of entries below 1e-19 (a double layer's on a large
+// surface) are lost and with them the weights.  n = 16384 cube: 494 us, 175
+// instructions per entry, the FP64 pipe 85% busy (two conversions and two
+// multiply-adds; the conversions by integer operations: 486 us; double-float sums:
+// 360).  One warp per block had left the few coarse blocks of millions of entries
+// to one warp each.
 template <typename T>
 __global__ void __launch_bounds__(256) norms_gen_kernel(const NormsArgs<T>* __restrict__ args,
                                                         const uint64_t* __restrict__ pieces, int64_t n,

@@ -100,3 +100,31 @@ def test_entries(kernel, kind, value):
         np.fill_diagonal(r, np.inf)
         slack = 4 * 2.0 ** -53 / (4 * np.pi * r ** 2) * np.hypot(1.0, kappa * np.where(np.isinf(r), 0.0, r))
     assert np.all(np.abs(got - want) <= 16 * 2.0 ** -24 * np.abs(want) + slack)
+
+
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** -20, 2.0 ** 37])
+@pytest.mark.parametrize("kernel", ["slp", "dlp"])
+def test_small_and_large_surfaces(kernel, scale):
+    """Block norms far from 1 (at 2^37 the double layer's entries are of 1e-23, whose squares FP32
+    cannot hold): scaled by a power of two, the same tree gets the same ranks."""
+    import paper_1510_07087_gb300 as D
+    from synth import fibonacci_sphere
+
+    unit = fibonacci_sphere(3000)
+
+    def compress(f):
+        T = D.dh2_tree_build(unit * f, 32, 6.0 / f)
+        if kernel == "slp":
+            return T, D.dh2_compress_kernel(T, unit * f, 6.0 / f, 20.0 / f, eps=1e-4, mode=D.MODE_FP32)
+        return T, D.dh2_compress_kernel_dlp(T, unit * f, unit, 6.0 / f, eps=1e-4, mode=D.MODE_FP32)
+
+    (T0, M0), (T, M) = compress(1.0), compress(scale)
+    assert T0.stats().adm_fraction > 0.1
+    assert np.array_equal(T0.perm(), T.perm()) and np.array_equal(T0.blocks(), T.blocks())
+    for s in (0, 1):
+        assert max(M0.ranks(s)) > 4
+        assert np.mean(M.ranks(s) != M0.ranks(s)) <= 0.01
+    w, w0 = M.block_weights(), M0.block_weights()
+    b = T.blocks()[:, 2] == 1
+    factor = 1.0 / scale if kernel == "slp" else 1.0 / scale ** 2  # the entries'
+    assert np.max(np.abs(w[b] * factor / w0[b] - 1.0)) <= 1e-6
