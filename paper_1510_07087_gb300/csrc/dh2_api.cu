@@ -933,7 +933,11 @@ struct PlanState {
 
 // Leaf pairs up to which one Jacobi launch takes all size classes (two waves of
 // the largest class's CTAs, 8 per SM), and non-leaf pairs of a level up to which
-// one Cholesky and one Jacobi launch take all row classes (4 per SM).
+// one Cholesky and one Jacobi launch take all row classes (4 per SM).  Leaf phase,
+// mixed, a launch per class / one launch: 64 pairs 0.45 / 0.30 ms, 1104 0.96 / 0.73,
+// 2598 0.92 / 0.77, 5527 2.20 / 2.12, 14628 3.99 / 3.96.  Level steps: levels of
+// 206 and 256 pairs 0.46 / 0.41 ms, of 16 to 388 (wide) 3.19 / 2.63, of 1080 and
+// 1868 1.52 / 1.60.
 constexpr int64_t kOneJacobi = 152 * 16;
 constexpr int kOneLevel = 152 * 4;
 // The class whose Jacobi launch takes the leaf pairs of every class up to it
@@ -2628,8 +2632,10 @@ class SideLease {
 };
 // nearfield entries from which the fork and join (about 6 us) pay: the product's
 // other kernels, ~20 us and more there, are bound by latency and leave HBM idle,
-// and the nearfield leaves them registers and threads.  n = 32768, one vector: 1224 -> 1158
-// us; n = 12289, adjoint, three vectors: 411 -> 367 us
+// and the nearfield leaves them registers and threads.  Without / with, one FP32
+// vector: 2^22.8 entries 62 / 63 us, 2^23.7 124 / 126 (eight vectors 249 / 246),
+// 2^24.4 159 / 150, 2^25 212 / 182, n = 32768 1224 / 1158.  (FP64 gains earlier:
+// 2^22.8 173 / 167, 2^23.7 272 / 247.)
 constexpr int64_t kOverlapElems = int64_t(1) << 23;
 
 // The launches of y = G~ x (adj = 0: forward transformation on W, coupling

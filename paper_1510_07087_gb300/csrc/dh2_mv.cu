@@ -106,7 +106,7 @@ __device__ __forceinline__ int chunk_width(int count) { return min(NR, count - (
 // entries.  Adjoint: a piece is a run of rows, its columns staged at an odd
 // distance so that threads on consecutive columns read without bank conflicts.
 // FP32 is bound by HBM: two stages ahead in 4 CTAs per SM keep ~100 KB per SM in
-// flight; n = 32768, one vector: 967 us, 6.4 TB/s (a row per thread with loads
+// flight; n = 32768, one vector: 975 us, 6.4 TB/s (a row per thread with loads
 // from global memory: 1808 us; eight loads in flight per thread: 2245 us, each
 // round of a 40-row block paid a DRAM and then an L2 latency).  FP64 is bound by
 // its pipe, 4 fused multiply-adds per entry and vector: n = 8192, eight

@@ -1736,10 +1736,11 @@ __global__ void __launch_bounds__(NT, MINB)
 // Threads: 4 x 4 tiles of the lower triangle, the columns of a chunk dealt to
 // G = NT / tiles threads per tile, summed at the end.
 // n = 8192, eps 1e-6, FP32 (leaf factors): streamed LQ with its Jacobi 2.32 ms;
-// this 0.58 ms, Cholesky 0.31, Jacobi 0.60 (with divisions in the staging and no
-// prefetch 1.12 ms).  Bound by issue: staging, scan and conversion, ~250 per 32
-// entries; the integer products are a fifth of it.  Singular values lie half as
-// far from FP64's as the LQ's (mean 2.3e-7 against 4.1e-7 of the largest).
+// this 0.60 ms, Cholesky 0.30, Jacobi 0.60 (with divisions in the staging and no
+// prefetch 1.12 ms).  387 million warp instructions, 340 per 32 entries, of which
+// the integer products are a sixth; half of the issue slots are used at a quarter
+// of the warps (ncu).  Singular values lie half as far from FP64's as the LQ's
+// (mean 2.3e-7 against 4.1e-7 of the largest).
 __host__ __device__ constexpr int gram_i64_ld(int p) {  // rows in fours, an odd number of them: staging by columns spreads over the banks
   return ((p + 3) / 4 | 1) * 4;
 }
