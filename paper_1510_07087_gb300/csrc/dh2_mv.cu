@@ -207,18 +207,27 @@ __global__ void __launch_bounds__(128) mv_near(MvArgs<T> a, int first, int count
   // pieces), and of those.  One chain over the unit's ~1600 columns had
   // 1.2 to 1.7 times the rounding error of block after block (n = 8192, leaf 64,
   // against FP64: 4.7e-7, by block 2.7e-7, now 1.5e-7), for 1% of the time in
-  // FP32 (n = 32768, one vector: 1162 -> 1171 us)
+  // FP32 (n = 32768, one vector: 1162 -> 1171 us) and 2% in FP64.  FP64, one and
+  // two vectors: four chains instead, which as well are a quarter as long (the
+  // second sums had cost 8%)
+  constexpr int U = sizeof(T) == 8 && NR <= 2 ? 4 : 1;
   constexpr int FOLD = sizeof(T) == 8 ? 8 : NR < 8 ? 1 : 4;
-  C2<T> acc[NR], sum[NR];
+  C2<T> acc[U][NR], sum[NR];
 #pragma unroll
-  for (int k = 0; k < NR; ++k) acc[k] = sum[k] = czero<T>();
+  for (int k = 0; k < NR; ++k) {
+    sum[k] = czero<T>();
+#pragma unroll
+    for (int u = 0; u < U; ++u) acc[u][k] = czero<T>();
+  }
   auto fold = [&]() {
 #pragma unroll
-    for (int k = 0; k < NR; ++k) {
-      sum[k].re += acc[k].re;
-      sum[k].im += acc[k].im;
-      acc[k] = czero<T>();
-    }
+    for (int k = 0; k < NR; ++k)
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        sum[k].re += acc[u][k].re;
+        sum[k].im += acc[u][k].im;
+        acc[u][k] = czero<T>();
+      }
   };
 #pragma unroll
   for (int s = 0; s < S - 1; ++s) {
@@ -235,15 +244,32 @@ __global__ void __launch_bounds__(128) mv_near(MvArgs<T> a, int first, int count
     const C2<T>* g = sm + (q % S) * (SG + SX) + (ADJ ? r * (w | 1) : r);
     const C2<T>* xs = sm + (q % S) * (SG + SX) + SG;
     if (c < cg) {
-#pragma unroll 4
-      for (int j = c; j < w; j += cg) {
+      auto add = [&](int j, int u) {
         const C2<T> v = ADJ ? g[j] : g[j * mr];
 #pragma unroll
         for (int k = 0; k < NR; ++k)
-          acc[k] = ADJ ? cfma_conj(acc[k], v, xs[j * NR + k]) : cfma(acc[k], v, xs[j * NR + k]);
+          acc[u][k] = ADJ ? cfma_conj(acc[u][k], v, xs[j * NR + k]) : cfma(acc[u][k], v, xs[j * NR + k]);
+      };
+      if constexpr (U == 1) {
+#pragma unroll 4
+        for (int j = c; j < w; j += cg) add(j, 0);
+      } else {
+        int j = c;
+        for (; j + (U - 1) * cg < w; j += U * cg)
+#pragma unroll
+          for (int u = 0; u < U; ++u) add(j + u * cg, u);
+        for (; j < w; j += cg) add(j, 0);
+        // the chain that took the rest goes to the back
+#pragma unroll
+        for (int k = 0; k < NR; ++k) {
+          const C2<T> t = acc[0][k];
+#pragma unroll
+          for (int u = 0; u + 1 < U; ++u) acc[u][k] = acc[u + 1][k];
+          acc[U - 1][k] = t;
+        }
       }
     }
-    if (q % FOLD == FOLD - 1) fold();
+    if (U == 1 && q % FOLD == FOLD - 1) fold();
   }
   fold();
   // (no copy is in flight: past the last piece nothing was issued)
