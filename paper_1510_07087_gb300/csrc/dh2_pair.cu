@@ -1727,7 +1727,7 @@ __global__ void __launch_bounds__(NT, MINB)
 // double-float and sixteen for the reflections of an LQ).  b: the sum of the
 // columns stays below 2^62: 27 bits up to 128 columns, 26 to 512.  Wider pairs
 // keep 26: where a diagonal sum (by Cauchy and Schwarz the largest are among
-// them) has passed 2^61 the sums go to H in double-float and start anew.  (In one
+// them) has passed 3 2^60 the sums go to H in double-float and start anew.  (In one
 // 64-bit sum a pair of 16k columns had 23 bits, and its noise, sqrt(N) 2^-(b+1) of
 // a row's largest entry, raised ranks beyond the compiled limits.)  The backward
 // error is 2^-(b+1) of each row's largest entry per entry.
@@ -1747,8 +1747,10 @@ __host__ __device__ constexpr int gram_i64_ld(int p) {  // rows in fours, an odd
 constexpr int kGramI64Chunk = 64;
 constexpr int kGramI64Flush = 512;
 static_assert(kGramSegCols % kGramI64Chunk == 0 && kGramI64Flush % kGramI64Chunk == 0, "whole chunks");
-// WIDE: more than kGramI64Flush columns are possible (without the flush no
-// registers are spilled: plan of n = 8191, paper's parameters, 6.88 -> 6.56 ms)
+// WIDE: more than kGramI64Flush columns are possible (without the flush fewer
+// registers are spilled: plan of n = 8191, paper's parameters, 6.88 -> 6.56 ms).
+// The flush and its looks: FP32 leaf factors at n = 32768, leaf 64, 16.0 -> 16.8 ms,
+// paper's parameters 48.6 -> 54.6 (streamed LQ: 26.3 and 77.9).
 template <bool FROM_R, int NT, bool WIDE, bool GEN>
 __global__ void __launch_bounds__(NT, NT <= 128 ? 4 : 3)
     gram_i64_kernel(const PairArgs<float>* __restrict__ args, const uint32_t* __restrict__ codes,
@@ -1824,10 +1826,10 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 4 : 3)
 #pragma unroll
     for (int j = 0; j < 4; ++j) ar[i][j] = ai[i][j] = 0;
   if (tid < kGramRows) rexp[tid] = -1000;
-  auto zero_pad = [&]() {  // the staging buffers' rows past p
-    for (int i = tid; i < 2 * CW * (LD - p); i += NT) buf[(i / (LD - p)) * LD + p + i % (LD - p)] = make_int2(0, 0);
+  auto zero_pad = [&](int col0, int n) {  // rows past p of n staged columns
+    for (int i = tid; i < n * (LD - p); i += NT) buf[(col0 + i / (LD - p)) * LD + p + i % (LD - p)] = make_int2(0, 0);
   };
-  zero_pad();
+  zero_pad(0, 2 * CW);
   bool bad = false;
   const int RG = (p + 31) >> 5;            // 32-row groups
   const int r = (warp % RG) * 32 + lane;   // the row this thread scans and converts
@@ -1856,15 +1858,16 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 4 : 3)
     }
     cp_async_commit();
   };
-  // the groups' sums (16 entries per tile) added up in the staging buffers, where
-  // no copy may be in flight, and from there into H, added to those of the
-  // columns before; last: both triangles
+  // the groups' sums (16 entries per tile) added up in staging buffer s, whose
+  // products are done (a buffer holds them for every p: 128 nt (nt + 1) <= 2048
+  // (nt | 1), nt = ceil(p / 4) <= 16), and from there into H, added to those of
+  // the columns before; last: both triangles
   bool flushed = false;
-  auto store = [&](bool last) {
-    longlong2* red = reinterpret_cast<longlong2*>(smem);
+  auto store = [&](int s, bool last) {
+    longlong2* red = reinterpret_cast<longlong2*>(buf + s * CW * LD);
     // the last groups' onto those before them, as many at once as have room (small
     // pairs have up to 128 groups: one by one took 250 barriers)
-    const int room = 4 * LD / ntile, t0 = tid % ntile;
+    const int room = 2 * LD / ntile, t0 = tid % ntile;
     auto put = [&](int slot) {
 #pragma unroll
       for (int u = 0; u < 16; ++u)
@@ -1895,22 +1898,36 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 4 : 3)
       const float s0 = __int_as_float((h + 127) << 23), s1 = __int_as_float((ex - h + 127) << 23);
       return Df{hi * s0 * s1, lo * s0 * s1};
     };
+    // four entries at a time, their old values in flight together
+    constexpr int EU = 4;
 #pragma unroll 1
-    for (int e = tid; e < 16 * ntile; e += NT) {
-      const int u = e / ntile, t = e - u * ntile;
-      const int rr = 4 * tile_i[t] + (u >> 2), cc = 4 * tile_j[t] + (u & 3);
-      if (rr >= p || cc > rr) continue;
-      const longlong2 v = red[e];
-      const int ex = rexp[rr] + rexp[cc] - 2 * b;
-      Df re = to_df(v.x, ex), im = to_df(v.y, ex);
-      float4* h = Hout + rr + (int64_t)cc * mp;
-      if (flushed) {
-        const float4 o = *h;
-        re = df_add(Df{o.x, o.y}, re);
-        im = df_add(Df{o.z, o.w}, im);
+    for (int e0 = tid; e0 < 16 * ntile; e0 += EU * NT) {
+      float4 o[EU];
+      int at[EU];  // -1: none, or outside the triangle
+#pragma unroll
+      for (int v = 0; v < EU; ++v) {
+        const int e = e0 + v * NT, u = e / ntile, t = e - u * ntile;
+        at[v] = -1;
+        o[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (e < 16 * ntile) {
+          const int rr = 4 * tile_i[t] + (u >> 2), cc = 4 * tile_j[t] + (u & 3);
+          if (rr < p && cc <= rr) at[v] = rr << 8 | cc;
+        }
+        if (at[v] >= 0 && flushed) o[v] = Hout[(at[v] >> 8) + (int64_t)(at[v] & 255) * mp];
       }
-      *h = make_float4(re.hi, re.lo, im.hi, im.lo);
-      if (last && cc != rr) Hout[cc + (int64_t)rr * mp] = make_float4(re.hi, re.lo, -im.hi, -im.lo);
+#pragma unroll
+      for (int v = 0; v < EU; ++v) {
+        if (at[v] < 0) continue;
+        const int rr = at[v] >> 8, cc = at[v] & 255, ex = rexp[rr] + rexp[cc] - 2 * b;
+        const longlong2 w = red[e0 + v * NT];
+        Df re = to_df(w.x, ex), im = to_df(w.y, ex);
+        if (flushed) {
+          re = df_add(Df{o[v].x, o[v].y}, re);
+          im = df_add(Df{o[v].z, o[v].w}, im);
+        }
+        Hout[rr + (int64_t)cc * mp] = make_float4(re.hi, re.lo, im.hi, im.lo);
+        if (last && cc != rr) Hout[cc + (int64_t)rr * mp] = make_float4(re.hi, re.lo, -im.hi, -im.lo);
+      }
     }
   };
   table(0, 0);
@@ -1924,16 +1941,20 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 4 : 3)
     if (more) table(j0 + CW, s ^ 1);
     cp_async_wait_all();
     // flush after this chunk?  Looked at every kGramI64Flush columns, which add at
-    // most 2^62 to a sum: those of 2^61 at one look stay below 2^63 beyond the next
-    bool big = false;
-    if (WIDE && more && (j0 + CW) % kGramI64Flush == 0 && grp < G && ti == tj)
-#pragma unroll
-      for (int i = 0; i < 4; ++i) big = big || ar[i][i] > (1ll << 61) / G;
-    // this chunk has landed; the other buffer's products are done
+    // most 2^62 to a sum: those of 3 2^60 at one look stay below 2^63 until after the
+    // chunk of the next (3 2^60 + 2^62 + 2^59)
     bool full = false;
-    if constexpr (WIDE) full = __syncthreads_or(big);
-    else __syncthreads();
-    if (more && !gen && !full) entries(j0 + CW, s ^ 1);
+    if (WIDE && more && (j0 + CW) % kGramI64Flush == 0) {
+      bool big = false;
+      if (grp < G && ti == tj)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) big = big || ar[i][i] > (3ll << 60) / G;
+      full = __syncthreads_or(big);
+    } else {
+      __syncthreads();
+    }
+    // (this chunk has landed; the other buffer's products are done)
+    if (more && !gen) entries(j0 + CW, s ^ 1);
     if (scan) {
       int m = 0;  // largest |re|, |im| as bits (NaN and infinity above every finite value)
       for (int j = c0; j < cw; j += cs) {
@@ -1997,17 +2018,17 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 4 : 3)
         }
       }
     if (full || !more) {
-      store(!more);
+      store(s, !more);
       if (!more) break;
       flushed = true;
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) ar[i][j] = ai[i][j] = 0;
-      __syncthreads();  // the staging buffers are free again
-      zero_pad();
+      __syncthreads();  // the buffer is free again
+      zero_pad(s * CW, CW);
     }
-    if (gen || full) entries(j0 + CW, s ^ 1);
+    if (gen) entries(j0 + CW, s ^ 1);
   }
   if (__syncthreads_or(bad)) {  // non-finite entries: reported, H zero
     if (tid == 0) atomicOr(a.status, kStatusNaN);
