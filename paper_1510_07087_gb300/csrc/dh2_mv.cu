@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(128) mv_near(MvArgs<T> a, int first, int count
     }
   };
   // sums in two steps: of a piece (where the additions cost pipe time, of several:
-  // 5 to 8 vectors in FP32 four, 12% slower by single ones; FP64 eight half
+  // 5 to 8 vectors in FP32 two, forward 5% slower by single ones; FP64 eight half
   // pieces), and of those.  One chain over the unit's ~1600 columns had
   // 1.2 to 1.7 times the rounding error of block after block (n = 8192, leaf 64,
   // against FP64: 4.7e-7, by block 2.7e-7, now 1.5e-7), for 1% of the time in
@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(128) mv_near(MvArgs<T> a, int first, int count
   // two vectors: four chains instead, which as well are a quarter as long (the
   // second sums had cost 8%)
   constexpr int U = sizeof(T) == 8 && NR <= 2 ? 4 : 1;
-  constexpr int FOLD = sizeof(T) == 8 ? 8 : NR < 8 ? 1 : 4;
+  constexpr int FOLD = sizeof(T) == 8 ? 8 : NR < 8 || ADJ ? 1 : 2;
   C2<T> acc[U][NR], sum[NR];
 #pragma unroll
   for (int k = 0; k < NR; ++k) {
